@@ -1,20 +1,29 @@
 // pf_batch.cu -- batched 1D pulled fronts in one persistent launch.
 //
-// Each CTA owns one 1D directional-solidification instance (frozen
-// temperature of Eq. ds1, moving window of Sec. "Numerical technique",
-// no-flux cold end, fixed hot end) and keeps its whole state in shared memory
-// for `nsteps` steps: phi, c = p c_s + (1-p) c_l, d = c_s - c_l, the diffusion
-// potentials and the phase-field rate.  Global memory is touched only at the
-// start and the end of a launch.  The discrete step is the one of the other
-// kernels (Eq. phasefield_nonvar with the re-derived driving force at cells;
-// the brackets of Eqs. cs_nonvar / cl_nonvar at faces; forward Euler on phi, c,
-// d).  Every `check_every` steps the CTA evaluates k_v = c_inf / c_max (Sec.
-// "Effect of parameter A on velocity-dependent partition coefficient") and
-// marks the instance converged once |dk_v/dt| stays below a tolerance over a
-// window of at least `window` time units; converged instances return at once in
-// later launches.  Instances are grouped by the block size an autotuner picks
-// for their length; the groups run concurrently on forked streams and the whole
-// chunk of launches is captured in a CUDA graph and replayed.
+// Each 1D directional-solidification instance (frozen temperature of Eq. ds1,
+// moving window of Sec. "Numerical technique", no-flux cold end, fixed hot end)
+// belongs to one CTA, or to a cluster of CTAs where there are fewer instances
+// than SMs, which keeps its state phi, c = p c_s + (1-p) c_l, d = c_s - c_l in
+// shared memory for `nsteps` steps; global memory is touched only at the start
+// and the end of a launch.  Warps step strips of the line in registers
+// (pf_line.cuh): the discrete step is the one of the other kernels (Eq.
+// phasefield_nonvar with the re-derived driving force at cells; the brackets of
+// Eqs. cs_nonvar / cl_nonvar at faces; forward Euler on phi, c, d).  Every
+// `check_every` steps the instance's k_v = c_inf / c_max (Sec. "Effect of
+// parameter A on velocity-dependent partition coefficient") is evaluated and the
+// instance marked converged once |dk_v/dt| stays below a tolerance over a window
+// of at least `window` time units; converged instances return at once in later
+// launches.  Instances are grouped by block size; the groups run concurrently
+// on forked streams and the whole chunk of launches is captured in a CUDA graph
+// and replayed.
+//
+// Bound (256 fronts of 512..8192 cells, FP32): the FP32 pipe, on which a packed
+// instruction takes two cycles, at 60 % of its cycles; the rest is warps waiting
+// at the block barrier for uneven numbers of strips.  500 steps: 17 ms with one
+// cell per thread through shared memory, every face evaluated twice with IEEE
+// divisions (634 instructions per cell and step), 4.5 ms with strips (115).  16
+// fronts of 2048 cells (a few SMs' work, bound by a step's latency): 8.9 us per
+// step, now 1.5 us on clusters of 8.  Their tangents: 32 us, now 3.9 us.
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -22,15 +31,18 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 #include "pf.h"
 #include "pf_dual.cuh"
 #include "pf_internal.cuh"
 #include "pf_kernels.h"
+#include "pf_line.cuh"
+#include <cooperative_groups.h>
 
 namespace pf {
 
-constexpr int BATCH_J = 8;   // cells per thread at most
+namespace cg = cooperative_groups;
 
 // per-instance persistent state (device)
 struct BatchState {
@@ -53,12 +65,12 @@ struct BatchArgs {
     int count;
     int nsteps;
     int check_every;
+    int cluster;        // CTAs per instance
+    int room;           // cells of one buffer of a CTA
     double tol, window, min_travel;
-    Consts<T> C;        // shared model parameters (dt unused; per instance)
+    LineConsts<T> K;    // shared model parameters
+    Consts<double> C;   // the same in FP64, rounded to T (energy records, clock)
     double theta_ref, G_theta, x0, c_inf;
-    T gphi, gcs, gcl, gmus, gmul;   // Dirichlet (hot end) ghost
-    T fc, fd;                       // fresh-layer state of the moving window
-    int hot_noflux;                 // 1: mirror ghost and zero flux at the hot end too
     long long energy_every;         // record F_h every this many steps (0: never)
     int energy_slots;               // records per instance in `energy`
     double* energy;                 // [instance][slot] F_h records (device)
@@ -66,262 +78,343 @@ struct BatchArgs {
     T* rec;                         // if set: every step's state and intermediates,
                                     // [instance block of 6 rec_steps n][step][phi|c|d|mu_s|mu_l|phidot][n]
     long long rec_steps;
+    double inv_dx2;
 };
 
+constexpr int BATCH_TAB = 32;       // steps whose clock is tabulated at once
+// cells per lane at most.  FP32: four (8192-cell fronts 4.6 ms per 512 steps;
+// with eight, whose 168 registers leave 12 warps per CTA, 4.9 ms).  FP64, bound
+// by the FP64 pipe, and runs with derivatives: two (with four, 12 FP64 fronts
+// took 5.4 ms instead of 2.9, and the tangents of 16 fronts spilled).
 template <typename T>
-__device__ __forceinline__ T frcp_b(T x) { return T(1) / x; }
+constexpr int batch_jmax() {
+    return sizeof(T) == 4 ? 4 : 2;
+}
+// warps per CTA at most: FP32 fits 128 registers a thread, the others 168
+template <typename T>
+constexpr int batch_warps() {
+    return sizeof(T) == 4 ? 16 : 12;
+}
+constexpr int BATCH_WARPS = 16;     // the largest of them
+constexpr int BATCH_CLUSTER = 8;    // CTAs per instance at most
 
-// 1D face (L, R): normal differences only
-template <typename T>
-__device__ __forceinline__ void face1(const Consts<T>& C, T fL, T fR, T csL, T csR, T clL, T clR,
-                                      T pdL, T pdR, T nphi, T nY, T nS, T nL, T& Fc, T& Fd) {
-    const T f = T(0.5) * (fL + fR);
-    const T cs = T(0.5) * (csL + csR), cl = T(0.5) * (clL + clR);
-    const T d = cs - cl;
-    const T pdot = T(0.5) * (pdL + pdR);
-    const T p = p_of(C, f);
-    const T omp = T(1) - p;
-    const T Ms = Ms_of(C, cs), Ml = Ml_of(C, cl);
-    const T bMl = C.b * Ml;
-    const T iMbar = frcp_b(Ms * omp + bMl * p);
-    const T gt2d = C.delta2;
-    const T r = frcp_b(nphi * nphi + gt2d);
-    const T Ts = Ms * nS * gt2d;
-    const T Tl = Ml * nL * gt2d;
-    const T at = C.one_m_A * d * pdot * nphi;
-    const T q = Ms * Ml * (C.b * p + omp) * iMbar;
-    const T afn = (Ms - bMl) * p * omp * iMbar;
-    Fc = r * (q * nphi * nphi * nY + p * Ts + omp * Tl + at * afn);
-    Fd = r * (Ts - Tl + at);
+// a pair's state before the step and its potentials and rate, into the record
+// of the step (cells i of the line go to i - m)
+template <typename T, int J>
+struct LineRecord {
+    using X = typename LineNum<T>::X;
+    T* base;          // nullptr: nothing is recorded
+    int n, i0, m;
+    double inv_dx2;
+    static constexpr bool on = true;
+    __device__ __forceinline__ void one(int i, T f, T c, T d, T s, T l, T r) const {
+        if (i < 0 || i >= n) return;
+        base[i] = f;
+        base[n + i] = c;
+        base[2 * n + i] = d;
+        base[3 * n + i] = s;
+        base[4 * n + i] = l;
+        base[5 * n + i] = r * T(inv_dx2);
+    }
+    __device__ __forceinline__ void operator()(int q, const X& f, const X& c, const X& d, const X& s, const X& l,
+                                               const X& r) const {
+        if (base == nullptr) return;
+        const int i = i0 - m + q;
+        one(i, x_lo(f), x_lo(c), x_lo(d), x_lo(s), x_lo(l), x_lo(r));
+        one(i + J / 2, x_hi(f), x_hi(c), x_hi(d), x_hi(s), x_hi(l), x_hi(r));
+    }
+};
+
+// J consecutive elements between shared memory and registers, in the widest
+// accesses their alignment (J elements, at most 16 bytes) allows
+template <typename T, int J>
+struct CellBlock {
+    using W = typename std::conditional<(J * sizeof(T)) % 16 == 0, uint4, uint2>::type;
+    static constexpr int N = (int)(J * sizeof(T) / sizeof(W));
+};
+template <int J, typename T>
+__device__ __forceinline__ void load_cells(const T* p, T (&w)[J]) {
+    using B = CellBlock<T, J>;
+    typename B::W u[B::N];
+#pragma unroll
+    for (int k = 0; k < B::N; ++k) u[k] = reinterpret_cast<const typename B::W*>(p)[k];
+    memcpy(w, u, sizeof(u));
+}
+template <int J, typename T>
+__device__ __forceinline__ void store_cells(T* p, const T (&w)[J]) {
+    using B = CellBlock<T, J>;
+    typename B::W u[B::N];
+    memcpy(u, w, sizeof(u));
+#pragma unroll
+    for (int k = 0; k < B::N; ++k) reinterpret_cast<typename B::W*>(p)[k] = u[k];
 }
 
-template <typename T, int NT>
-__global__ void __launch_bounds__(NT)
-batch_kernel(BatchArgs<T> a) {
-    const int inst = a.ids[blockIdx.x];
-    BatchState& S = a.st[inst];
-    if (S.converged) return;
-    const int n = S.n;
-    const Consts<T>& C = a.C;
+// One instance per cluster of a.cluster CTAs (one CTA: no cluster launch).  Each
+// CTA keeps a segment of the line's (phi, c, d) in shared memory, twice; in a
+// block of up to J/2 steps every warp takes strips of the line from one copy
+// through registers (pf_line.cuh) into the other, so that there is one barrier
+// per block and none inside it.  Cells at a segment's ends are also written to
+// the neighbouring CTA's copy of them (distributed shared memory).
+template <typename T, int J, bool STD, bool REC>
+__global__ void __launch_bounds__(32 * batch_warps<T>())
+batch_kernel(const __grid_constant__ BatchArgs<T> a) {
+    using X = typename LineNum<T>::X;
+    using V = typename LineNum<T>::V;
+    using S = typename LineNum<T>::S;
+    constexpr int H = J / 2;
+    constexpr int USE = 30 * J;      // cells of a strip that hold results
+    const int csize = a.cluster;
+    const int inst = a.ids[blockIdx.x / csize];
+    BatchState& St = a.st[inst];
+    if (St.converged) return;        // the same for every CTA of the cluster
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = csize > 1 ? (int)cluster.block_rank() : 0;
+    const int n = St.n;
+    // The line is stored up to a whole number of strips, its cells from n on
+    // holding the Dirichlet state (J of them at least: a block of J/2 steps moves
+    // the window by fewer).  Each CTA keeps `mine` cells from lo on, with J copies
+    // of its neighbours' cells on either side.
+    const int strips = (n + J + USE - 1) / USE;
+    const int seg = (strips + csize - 1) / csize * USE;
+    const int lo = rank * seg;
+    const int mine = max(0, min(seg, strips * USE - lo));
+    const LineConsts<T>& K = a.K;
     extern __shared__ __align__(16) unsigned char smem[];
-    T* sPhi = reinterpret_cast<T*>(smem);          // n
-    T* sC = sPhi + n;                               // n
-    T* sD = sC + n;                                 // n
-    T* sMs = sD + n;                                // n: mu_s
-    T* sMl = sMs + n;                               // n: mu_l
-    T* sPd = sMl + n;                               // n: phase-field rate
-    __shared__ double red[NT / 32];
+    __shared__ double red[BATCH_WARPS], cred[BATCH_CLUSTER];
+    __shared__ double th0[BATCH_TAB];           // (1 - k_e) theta0 of the tabulated steps
+    __shared__ int sh[BATCH_TAB + 1];           // window shifts before each of them since the first, and after the last
     __shared__ int s_done;
 
-    const int tid = threadIdx.x;
-    const long long off = S.off;
-    for (int i = tid; i < n; i += NT) {
-        sPhi[i] = a.phi[off + i];
-        sC[i] = a.c[off + i];
-        sD[i] = a.d[off + i];
+    const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, warps = NT >> 5;
+    const long long off = St.off;
+    const int room = a.room;                    // cells of one field: J + segment + J
+    T* const sm = reinterpret_cast<T*>(smem) + J;   // own cell 0 of the first field
+    for (int i = tid - J; i < room - J; i += NT) {
+        const int g = lo + i;
+        const bool in = g >= 0 && g < n;
+        const T f = in ? a.phi[off + g] : T(K.gphi), c = in ? a.c[off + g] : T(K.fc), d = in ? a.d[off + g] : T(K.fd);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            sm[3 * b * room + i] = f;
+            sm[(3 * b + 1) * room + i] = c;
+            sm[(3 * b + 2) * room + i] = d;
+        }
     }
-    long long step = S.step, shifts = S.shifts;
-    double k_prev = S.k_prev, t_prev = S.t_prev, k_last = S.k_last, dkdt_last = S.dkdt_last;
+    long long step = St.step, shifts = St.shifts;
+    double k_prev = St.k_prev, t_prev = St.t_prev, k_last = St.k_last, dkdt_last = St.dkdt_last;
     int converged = 0;
-    const double v = a.v[inst];
-    const T dt = T(a.dt[inst]);
-    const T dtdx = dt * C.inv_dx;
+    const double v = a.v[inst], dtd = a.dt[inst], dxd = a.C.dx;
+    const S dtq1 = S(dtd * a.inv_dx2);
+    V dtq;
+    dtq.x = dtq1;
+    dtq.y = dtq1;
     if (tid == 0) s_done = 0;
-    __syncthreads();
-
-    auto cs_cl = [&](int i, T& p, T& cs, T& cl) {
-        p = p_of(C, sPhi[i]);
-        cs = sC[i] + (T(1) - p) * sD[i];
-        cl = sC[i] - p * sD[i];
+    auto sync = [&]() {
+        if (csize > 1) cluster.sync();
+        else __syncthreads();
     };
+    // steps to the next look at the state
+    int to_check = a.check_every > 0 ? a.check_every - (int)(step % a.check_every) : 0x7fffffff;
+    long long to_energy = a.energy_every > 0 ? a.energy_every - step % a.energy_every : 0x7fffffffffffffffll;
+    sync();
 
-    for (int it = 0; it < a.nsteps; ++it) {
-        const double t = (double)step * a.dt[inst];
-        const T theta0 = T(a.theta_ref + a.G_theta * (a.x0 + v * t - (double)shifts * (double)C.dx));
-        // for a reverse sweep: the pre-step state, then mu_s, mu_l, phidot below
-        T* const rec = a.rec != nullptr ? a.rec + 6 * a.rec_steps * off + (long long)it * 6 * n : nullptr;
-        if (rec != nullptr) {
-            for (int i = tid; i < n; i += NT) {
-                rec[i] = sPhi[i];
-                rec[n + i] = sC[i];
-                rec[2 * n + i] = sD[i];
-            }
-        }
-        // P1: diffusion potentials
-        for (int i = tid; i < n; i += NT) {
-            T p, cs, cl;
-            cs_cl(i, p, cs, cl);
-            sMs[i] = flog(cs) - C.log_ke;
-            sMl[i] = flog(cl);
-            if (rec != nullptr) {
-                rec[3 * n + i] = sMs[i];
-                rec[4 * n + i] = sMl[i];
-            }
-        }
-        __syncthreads();
-        // P2: phase-field rate (cold end: mirror ghost; hot end: Dirichlet or
-        // mirror ghost)
-        for (int i = tid; i < n; i += NT) {
-            const int im = (i == 0) ? 0 : i - 1;
-            const bool last = i == n - 1, mirror_hot = last && a.hot_noflux;
-            const int ip = last ? i : i + 1;
-            const T fc = sPhi[i];
-            const T fW = sPhi[im];
-            const T fE = (last && !mirror_hot) ? a.gphi : sPhi[ip];
-            const T mW_s = sMs[im], mW_l = sMl[im];
-            const T mE_s = (last && !mirror_hot) ? a.gmus : sMs[ip];
-            const T mE_l = (last && !mirror_hot) ? a.gmul : sMl[ip];
-            T p, cs, cl;
-            cs_cl(i, p, cs, cl);
-            const T mus = sMs[i], mul = sMl[i];
-            const T dp = dp_of(C, fc);
-            const T lap = (fW - T(2) * fc + fE) * C.inv_dx2;
-            const T gp = (fE - fW) * C.inv_2dx;
-            const T gs = (mE_s - mW_s) * C.inv_2dx;
-            const T gl = (mE_l - mW_l) * C.inv_2dx;
-            const T Ms = Ms_of(C, cs), Ml = Ml_of(C, cl);
-            const T bMl = C.b * Ml;
-            const T Msq = Ms * (T(1) - p);
-            const T iMbar = frcp_b(Msq + bMl * p);
-            const T d = cs - cl;
-            const T rr = frcp_b(gp * gp + C.delta2);
-            const T pq = p * (T(1) - p);
-            const T Kc = C.inv_Mphi + C.one_m_A * C.one_m_A * d * d * C.b * pq * rr * iMbar /
-                                          (C.b * p + T(1) - p);
-            const T theta = theta0 - C.G_theta * ((T(i) + T(0.5)) * C.dx);
-            const T dmu = mus - mul;
-            const T Dd = (Msq * (T(1) - C.A * (T(1) - p)) + C.A * bMl * p * p) * iMbar;
-            const T dG = cs * dmu - d - C.one_m_ke * theta - Dd * d * dmu;
-            const T dfdw = T(2) * fc * (T(1) - fc) * (T(1) - T(2) * fc);
-            const T R = C.sigma * lap - C.H * dfdw - dG * dp +
-                        C.one_m_A * d * pq * iMbar * (Ms * gs - bMl * gl) * gp * rr;
-            sPd[i] = R / Kc;
-            if (rec != nullptr) rec[5 * n + i] = sPd[i];
-        }
-        __syncthreads();
-        // P3: faces of each owned cell and the new state (kept in registers)
-        T nphi[BATCH_J], nc[BATCH_J], nd[BATCH_J];
-#pragma unroll
-        for (int j = 0; j < BATCH_J; ++j) {
-            const int i = tid + j * NT;
-            if (i >= n) break;
-            T pL, csL, clL, pR, csR, clR, p0, cs0, cl0;
-            cs_cl(i, p0, cs0, cl0);
-            const T f0 = sPhi[i], ms0 = sMs[i], ml0 = sMl[i], pd0 = sPd[i];
-            const T Y0 = ml0 + p0 * (ms0 - ml0);
-            T FcL = T(0), FdL = T(0), FcR, FdR;
-            if (i > 0) {   // face (i-1, i); the face at the cold end is no-flux
-                cs_cl(i - 1, pL, csL, clL);
-                const T fL = sPhi[i - 1], msL = sMs[i - 1], mlL = sMl[i - 1];
-                const T YL = mlL + pL * (msL - mlL);
-                face1(C, fL, f0, csL, cs0, clL, cl0, sPd[i - 1], pd0, (f0 - fL) * C.inv_dx,
-                      (Y0 - YL) * C.inv_dx, (ms0 - msL) * C.inv_dx, (ml0 - mlL) * C.inv_dx, FcL, FdL);
-            }
-            if (i < n - 1) {
-                cs_cl(i + 1, pR, csR, clR);
-                const T fR = sPhi[i + 1], msR = sMs[i + 1], mlR = sMl[i + 1];
-                const T YR = mlR + pR * (msR - mlR);
-                face1(C, f0, fR, cs0, csR, cl0, clR, pd0, sPd[i + 1], (fR - f0) * C.inv_dx,
-                      (YR - Y0) * C.inv_dx, (msR - ms0) * C.inv_dx, (mlR - ml0) * C.inv_dx, FcR, FdR);
-            } else if (a.hot_noflux) {   // closed hot end: no flux through the last face
-                FcR = T(0);
-                FdR = T(0);
-            } else {       // face to the fixed hot-end ghost (phase-field rate 0)
-                const T gp = p_of(C, a.gphi);
-                const T YR = a.gmul + gp * (a.gmus - a.gmul);
-                face1(C, f0, a.gphi, cs0, a.gcs, cl0, a.gcl, pd0, T(0), (a.gphi - f0) * C.inv_dx,
-                      (YR - Y0) * C.inv_dx, (a.gmus - ms0) * C.inv_dx, (a.gmul - ml0) * C.inv_dx, FcR, FdR);
-            }
-            nphi[j] = f0 + dt * pd0;
-            nc[j] = sC[i] + dtdx * (FcR - FcL);
-            nd[j] = sD[i] + dtdx * (FdR - FdL);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int j = 0; j < BATCH_J; ++j) {
-            const int i = tid + j * NT;
-            if (i >= n) break;
-            sPhi[i] = nphi[j];
-            sC[i] = nc[j];
-            sD[i] = nd[j];
-        }
-        step += 1;
-        // moving window: drop the cold-end cell, append the fresh hot-end state
-        const double tn = (double)step * a.dt[inst];
-        while (v * tn >= (double)(shifts + 1) * (double)C.dx) {
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < BATCH_J; ++j) {
-                const int i = tid + j * NT;
-                if (i >= n) break;
-                if (i < n - 1) {
-                    nphi[j] = sPhi[i + 1]; nc[j] = sC[i + 1]; nd[j] = sD[i + 1];
-                } else {
-                    nphi[j] = a.gphi; nc[j] = a.fc; nd[j] = a.fd;
+    int cur = 0;                       // offset of the current copy
+    int tab = BATCH_TAB;               // next entry of the clock table (full: refill)
+    long long tab_shifts = shifts;     // shifts at the table's first step
+    for (int it = 0; it < a.nsteps;) {
+        if (tab == BATCH_TAB) {
+            // the clock of the next steps: shifts after step j is the smallest
+            // count whose successor's distance the window has not yet covered
+            if (warp == 0) {
+                const double t = (double)(step + lane) * dtd;
+                long long k = shifts;
+                if (lane > 0)
+                    while (v * t >= (double)(k + 1) * dxd) k += 1;
+                sh[lane] = (int)(k - shifts);
+                th0[lane] = K.one_m_ke * (a.theta_ref + a.G_theta * (a.x0 + v * t - (double)k * dxd));
+                if (lane == 31) {
+                    const double t2 = (double)(step + BATCH_TAB) * dtd;
+                    while (v * t2 >= (double)(k + 1) * dxd) k += 1;
+                    sh[BATCH_TAB] = (int)(k - shifts);
                 }
             }
+            tab = 0;
+            tab_shifts = shifts;
             __syncthreads();
-#pragma unroll
-            for (int j = 0; j < BATCH_J; ++j) {
-                const int i = tid + j * NT;
-                if (i >= n) break;
-                sPhi[i] = nphi[j]; sC[i] = nc[j]; sD[i] = nd[j];
-            }
-            shifts += 1;
         }
-        __syncthreads();
+        // a block: up to J/2 steps, ending where the state is looked at
+        int kb = min(min(H, a.nsteps - it), min(BATCH_TAB - tab, to_check));
+        if (to_energy < kb) kb = (int)to_energy;
+        const int s0 = sh[tab];
+        const int mt = sh[tab + kb] - s0;                 // shifts in the block
+        const int nxt = 3 * room - cur;
+        for (int u = warp * USE; u < mine; u += warps * USE) {
+            const int w0 = u + (lane - 1) * J;            // own index; lane 0 and lane 31: the strip's stale ends
+            const int i0 = lo + w0;
+            Strip<T, J, false> s;
+            {
+                const T* p = sm + cur + w0;
+                T w[J];
+                auto get = [&](const T* q, X (&x)[H]) {
+                    load_cells<J>(q, w);
+#pragma unroll
+                    for (int k = 0; k < H; ++k) x[k] = x_pair(w[k], w[k + H]);
+                };
+                get(p, s.phi);
+                get(p + room, s.c);
+                get(p + 2 * room, s.d);
+            }
+            // an end of the line in the strip
+            const bool edge = lo + u < mt + J + 1 || lo + u + USE + J >= n;
+            auto steps = [&](auto e) {
+                constexpr bool EDGE = decltype(e)::value;
+                for (int k = 0; k < kb; ++k) {
+                    const int m = sh[tab + k] - s0;
+                    if constexpr (REC) {
+                        LineRecord<T, J> rec;
+                        rec.base = (lane == 0 || lane == 31)
+                                       ? nullptr
+                                       : a.rec + 6 * a.rec_steps * off + (long long)(it + k) * 6 * n;
+                        rec.n = n;
+                        rec.i0 = i0;
+                        rec.m = m;
+                        rec.inv_dx2 = a.inv_dx2;
+                        line_step<STD, EDGE, T, J, false>(K, s, i0, n, m, dtq, th0[tab + k], rec);
+                    } else {
+                        line_step<STD, EDGE, T, J, false>(K, s, i0, n, m, dtq, th0[tab + k], NoRecord());
+                    }
+                }
+            };
+            if (edge) steps(std::true_type());
+            else steps(std::false_type());
+            if (lane != 0 && lane != 31) {
+                if (mt == 0) {
+                    auto put = [&](T* q, const X (&x)[H]) {
+                        T w[J];
+#pragma unroll
+                        for (int k = 0; k < H; ++k) {
+                            w[k] = x_lo(x[k]);
+                            w[k + H] = x_hi(x[k]);
+                        }
+                        store_cells<J>(q, w);
+                    };
+                    auto put3 = [&](T* p) {
+                        put(p, s.phi);
+                        put(p + room, s.c);
+                        put(p + 2 * room, s.d);
+                    };
+                    T* const p = sm + nxt + w0;
+                    put3(p);
+                    // the neighbours' copies of this CTA's first and last cells
+                    if (csize > 1) {
+                        if (w0 == 0 && rank > 0) put3(cluster.map_shared_rank(p + seg, rank - 1));
+                        if (w0 + J == seg && rank < csize - 1) put3(cluster.map_shared_rank(p - seg, rank + 1));
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < J; ++k) {
+                        const int i = i0 + k - mt;      // the window has dropped mt cells
+                        if (i < 0) continue;
+                        auto put1 = [&](T* q) {
+                            q[0] = k < H ? x_lo(s.phi[k % H]) : x_hi(s.phi[k % H]);
+                            q[room] = k < H ? x_lo(s.c[k % H]) : x_hi(s.c[k % H]);
+                            q[2 * room] = k < H ? x_lo(s.d[k % H]) : x_hi(s.d[k % H]);
+                        };
+                        const int r = i >= lo ? rank : rank - 1;     // mt < seg
+                        const int l = i - r * seg;
+                        T* const q = sm + nxt + l;
+                        put1(r == rank ? q : cluster.map_shared_rank(q, r));
+                        if (csize > 1) {
+                            if (l < J && r > 0) put1(cluster.map_shared_rank(q + seg, r - 1));
+                            if (l >= seg - J && r < csize - 1)
+                                put1(r + 1 == rank ? q - seg : cluster.map_shared_rank(q - seg, r + 1));
+                        }
+                    }
+                }
+            }
+        }
+        it += kb;
+        step += kb;
+        tab += kb;
+        to_check -= kb;
+        to_energy -= kb;
+        shifts = tab_shifts + sh[tab];
+        cur = nxt;
+        sync();
+        const int own = min(mine, n - lo);     // own cells of the line (may be negative)
+        T* const sPhi = sm + cur;
+        T* const sC = sPhi + room;
+        T* const sD = sC + room;
         // F_h of the new state (the discrete free energy of pf_energy), FP64
-        if (a.energy_every > 0 && (step % a.energy_every) == 0) {
-            const double t = (double)step * a.dt[inst];
-            const double th0 = a.theta_ref + a.G_theta * (a.x0 + v * t - (double)shifts * (double)C.dx);
-            const double dxd = (double)C.dx, ke = (double)C.one_m_ke;
+        if (to_energy == 0) {
+            to_energy = a.energy_every;
+            const double tn = (double)step * dtd;
+            const Consts<double>& C = a.C;
+            const double th = a.theta_ref + a.G_theta * (a.x0 + v * tn - (double)shifts * dxd);
             double e = 0.0;
-            for (int i = tid; i < n; i += NT) {
-                const double f = (double)sPhi[i], cc = (double)sC[i], dd = (double)sD[i];
+            for (int i = tid; i < own; i += NT) {
+                const double f = (double)value_of(sPhi[i]), cc = (double)value_of(sC[i]), dd = (double)value_of(sD[i]);
                 const double g = f * (1.0 - f);
-                const double h = f * f * ((double)C.h2 + f * ((double)C.h3 + f * ((double)C.h4 + f * (double)C.h5)));
-                const double p = h + (double)C.a * (f - 0.5) * g * g;
+                const double p = p_of(C, f);
                 const double cs = cc + (1.0 - p) * dd, cl = cc - p * dd;
-                const double th = th0 - (double)C.G_theta * (((double)i + 0.5) * dxd);
-                const double fs = -ke * th + cs * (log(cs) - (double)C.log_ke - 1.0);
+                const double tx = th - C.G_theta * (((double)(lo + i) + 0.5) * dxd);
+                const double fs = -C.one_m_ke * tx + cs * (log(cs) - C.log_ke - 1.0);
                 const double fl = cl * (log(cl) - 1.0);
                 // gradient energy: each pair of cells once, from its left cell;
                 // mirror ghosts add nothing and the pair with a Dirichlet ghost
                 // counts half, as in pf_energy
                 double gs = 0.0;
-                if (i < n - 1) {
-                    const double dphi = (double)sPhi[i + 1] - f;
+                if (lo + i < n - 1) {
+                    const double dphi = (double)value_of(sPhi[i + 1]) - f;
                     gs = dphi * dphi;
-                } else if (!a.hot_noflux) {
+                } else if (!K.hot_noflux) {
                     const double dphi = a.dir_phi - f;
                     gs = 0.5 * dphi * dphi;
                 }
-                e += (double)C.H * g * g + p * fs + (1.0 - p) * fl + 0.5 * (double)C.sigma * gs / (dxd * dxd);
+                e += C.H * g * g + p * fs + (1.0 - p) * fl + 0.5 * C.sigma * gs / (dxd * dxd);
             }
             for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-            if ((tid & 31) == 0) red[tid >> 5] = e;
+            if (lane == 0) red[warp] = e;
             __syncthreads();
             if (tid == 0) {
                 double tot = 0.0;
-                for (int w = 0; w < NT / 32; ++w) tot += red[w];
+                for (int w = 0; w < warps; ++w) tot += red[w];
+                if (csize > 1) *cluster.map_shared_rank(&cred[rank], 0) = tot;
+                else cred[0] = tot;
+            }
+            sync();
+            if (tid == 0 && rank == 0) {
+                double tot = 0.0;
+                for (int r = 0; r < csize; ++r) tot += cred[r];
                 const long long slot = step / a.energy_every - 1;
                 if (slot < a.energy_slots) a.energy[(long long)inst * a.energy_slots + slot] = tot * dxd;
             }
-            __syncthreads();
+            sync();
         }
         // steady-state check on k_v = c_inf / c_max
-        if (a.check_every > 0 && (step % a.check_every) == 0) {
+        if (to_check == 0) {
+            to_check = a.check_every;
+            const double tn = (double)step * dtd;
             // a maximum that keeps a NaN (fmax would drop it): a state that has
             // stopped being finite must not look steady
             auto nanmax = [](double x, double y) { return (y > x || y != y) ? y : x; };
             double cm = -1e300;
-            for (int i = tid; i < n; i += NT) cm = nanmax(cm, (double)sC[i]);
+            for (int i = tid; i < own; i += NT) cm = nanmax(cm, (double)value_of(sC[i]));
             for (int o = 16; o > 0; o >>= 1) cm = nanmax(cm, __shfl_xor_sync(0xffffffffu, cm, o));
-            if ((tid & 31) == 0) red[tid >> 5] = cm;
+            if (lane == 0) red[warp] = cm;
             __syncthreads();
             if (tid == 0) {
                 double m = red[0];
-                for (int w = 1; w < NT / 32; ++w) m = nanmax(m, red[w]);
+                for (int w = 1; w < warps; ++w) m = nanmax(m, red[w]);
+                for (int r = 0; r < csize; ++r) {      // every CTA keeps its own copy of the maxima
+                    if (csize > 1) *cluster.map_shared_rank(&cred[rank], r) = m;
+                    else cred[0] = m;
+                }
+            }
+            sync();
+            if (tid == 0) {
+                double m = cred[0];
+                for (int r = 1; r < csize; ++r) m = nanmax(m, cred[r]);
                 const double k = a.c_inf / m;
                 k_last = k;
                 if (!isfinite(m)) {
@@ -333,26 +426,26 @@ batch_kernel(BatchArgs<T> a) {
                     t_prev = tn;
                 }
             }
-            __syncthreads();
+            sync();
             if (s_done) {
                 converged = s_done;
                 break;
             }
         }
     }
-    for (int i = tid; i < n; i += NT) {
-        a.phi[off + i] = sPhi[i];
-        a.c[off + i] = sC[i];
-        a.d[off + i] = sD[i];
+    for (int i = tid; i < min(mine, n - lo); i += NT) {
+        a.phi[off + lo + i] = sm[cur + i];
+        a.c[off + lo + i] = sm[cur + room + i];
+        a.d[off + lo + i] = sm[cur + 2 * room + i];
     }
-    if (tid == 0) {
-        S.step = step;
-        S.shifts = shifts;
-        S.k_prev = k_prev;
-        S.t_prev = t_prev;
-        S.k_last = k_last;
-        S.dkdt_last = dkdt_last;
-        S.converged = converged;
+    if (tid == 0 && rank == 0) {
+        St.step = step;
+        St.shifts = shifts;
+        St.k_prev = k_prev;
+        St.t_prev = t_prev;
+        St.k_last = k_last;
+        St.dkdt_last = dkdt_last;
+        St.converged = converged;
     }
 }
 
@@ -388,27 +481,52 @@ __global__ void batch_from_state(const T* __restrict__ phi, const T* __restrict_
 
 namespace {
 
-double p_of_host(const pf_params& P, double f) {
-    const double g = f * (1.0 - f);
-    const double h = (P.interp == 1) ? f * f * (3.0 - 2.0 * f) : f * f * f * (6.0 * f * f - 15.0 * f + 10.0);
-    return h + P.a * (f - 0.5) * g * g;
+// cells per lane: the request rounded to what the type's kernels have (two at
+// least, as cells are computed in pairs)
+template <typename T>
+int cells_per_lane(int cpt) {
+    return std::max(2, std::min(cpt, batch_jmax<T>()));
 }
 
-int threads_for(int64_t n, int cpt) {
-    int nt = 128;
-    while (nt < 1024 && (int64_t)nt * cpt < n) nt *= 2;
-    return nt;
+// warps of a CTA that has `strips` strips to take: as few as finish them in the
+// smallest number of rounds
+int warps_for(int64_t strips, int most) {
+    const int64_t rounds = (strips + most - 1) / most;
+    return (int)((strips + rounds - 1) / rounds);
 }
 
 template <typename T>
-cudaError_t launch_group(int nt, const BatchArgs<T>& a, size_t smem, cudaStream_t s) {
-    switch (nt) {
-        case 128: batch_kernel<T, 128><<<a.count, 128, smem, s>>>(a); break;
-        case 256: batch_kernel<T, 256><<<a.count, 256, smem, s>>>(a); break;
-        case 512: batch_kernel<T, 512><<<a.count, 512, smem, s>>>(a); break;
-        default: batch_kernel<T, 1024><<<a.count, 1024, smem, s>>>(a); break;
-    }
-    return cudaGetLastError();
+using BatchFn = void (*)(const BatchArgs<T>);
+template <typename T, bool STD, bool REC>
+BatchFn<T> batch_fn_J(int J) {
+    if constexpr (batch_jmax<T>() >= 4)
+        if (J == 4) return batch_kernel<T, 4, STD, REC>;
+    return batch_kernel<T, 2, STD, REC>;
+}
+// the instance for J cells per lane, the default physics or not, recording every
+// step or not (a run with derivatives never does)
+template <typename T>
+BatchFn<T> batch_fn(int J, bool std_phys, bool rec) {
+    if constexpr (!IsDual<T>::value)
+        if (rec) return std_phys ? batch_fn_J<T, true, true>(J) : batch_fn_J<T, false, true>(J);
+    return std_phys ? batch_fn_J<T, true, false>(J) : batch_fn_J<T, false, false>(J);
+}
+
+template <typename T>
+cudaError_t launch_group(int warps, int J, bool std_phys, const BatchArgs<T>& a, size_t smem, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(a.count * a.cluster);
+    cfg.blockDim = dim3(32 * warps);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = a.cluster;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = a.cluster > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, batch_fn<T>(J, std_phys, a.rec != nullptr), a);
 }
 
 // raise each instantiation's dynamic shared-memory limit to what the device
@@ -423,7 +541,7 @@ cudaError_t raise_smem(K kern, int optin) {
 }
 
 template <typename T>
-cudaError_t set_smem_limits(size_t* max_dynamic) {
+cudaError_t set_smem_limits(size_t* max_dynamic, int* sms) {
     static DeviceSetup setup;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -433,22 +551,25 @@ cudaError_t set_smem_limits(size_t* max_dynamic) {
     if (!setup.done[dev]) {
         int optin = 0;
         e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (e == cudaSuccess) e = raise_smem(batch_kernel<T, 128>, optin);
-        if (e == cudaSuccess) e = raise_smem(batch_kernel<T, 256>, optin);
-        if (e == cudaSuccess) e = raise_smem(batch_kernel<T, 512>, optin);
-        if (e == cudaSuccess) e = raise_smem(batch_kernel<T, 1024>, optin);
-        setup.value[dev] = (size_t)optin - 1024;   // static part: reduction scratch and flag
+        for (int J = 2; J <= batch_jmax<T>(); J *= 2) {
+            for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = raise_smem(batch_fn<T>(J, i & 1, i & 2), optin);
+        }
+        int n = 1;
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        setup.sms[dev] = n;
+        setup.value[dev] = (size_t)optin - 1024;   // static part: clock table, reduction scratch, flag
         setup.err[dev] = e;
         setup.done[dev] = true;
     }
     *max_dynamic = setup.value[dev];
+    *sms = setup.sms[dev];
     return setup.err[dev];
 }
 
 struct Group {
-    int nt;
+    int warps;         // of a CTA
     int dir = -1;      // seeded parameter of a tangent run (0 M_phi, 1 A, 2 b), -1 none
-    int nmax;
+    int room = 0;      // cells of one shared-memory copy
     std::vector<int> ids;
     int* d_ids = nullptr;
     cudaStream_t stream = nullptr;
@@ -467,6 +588,9 @@ struct BatchRun {
     BatchState* st = nullptr;
     double *dv = nullptr, *ddt = nullptr;
     std::vector<Group> groups;
+    int J = 2, cluster = 1;     // cells per lane and CTAs per instance of the groups
+    bool std_phys = false;
+    int sms = 1;
     std::vector<int> rep_dir;   // tangent runs: seeded parameter of each instance
     double* energy = nullptr;   // F_h records [instance][slot] (device), or null
     int energy_slots = 0;
@@ -490,6 +614,14 @@ struct BatchRun {
         if (t1) cudaEventDestroy(t1);
     }
 
+    // the line of the batch as a problem description (lengths and clocks are the instances')
+    HostProblem problem() const {
+        pf_grid g1{1, {8, 1, 1}, D.dx};
+        HostProblem P;
+        fill_problem(P, &g1, &D.bc, &D.params);
+        return P;
+    }
+
     BatchArgs<T> args(const Group& g, int nsteps) const {
         BatchArgs<T> a;
         a.phi = phi; a.c = c; a.d = d; a.st = st; a.ids = g.d_ids; a.v = dv; a.dt = ddt;
@@ -499,50 +631,41 @@ struct BatchRun {
         a.tol = D.tol;
         a.window = D.window;
         a.min_travel = D.min_travel;
-        const pf_params& P = D.params;
-        Consts<T>& C = a.C;
-        C = Consts<T>{};   // every member zero (Dual members by their constructor)
-        C.dim = 1; C.interp = P.interp; C.lap = 3; C.mobility = P.mobility_mode;
-        C.dx = T(D.dx); C.inv_dx = T(1.0 / D.dx); C.inv_2dx = T(0.5 / D.dx); C.inv_dx2 = T(1.0 / (D.dx * D.dx));
-        C.H = T(P.H); C.sigma = T(P.sigma); C.inv_Mphi = T(1.0 / P.M_phi); C.D_s = T(P.D_s); C.D_l = T(P.D_l);
-        C.log_ke = T(std::log(P.k_e)); C.one_m_ke = T(1.0 - P.k_e); C.A = T(P.A); C.one_m_A = T(1.0 - P.A);
-        C.b = T(P.b); C.a = T(P.a); C.delta2 = T(P.delta * P.delta); C.G_theta = T(P.G_theta);
+        a.cluster = cluster;
+        a.room = g.room;
+        const HostProblem P = problem();
+        a.K = make_line_consts<T>(P, g.dir);
+        using S = typename LineNum<T>::S;
+        auto r = [](double x) { return (double)S(x); };
+        Consts<double>& C = a.C;
+        C = Consts<double>{};
+        C.interp = P.interp; C.mobility = P.mobility;
+        C.dx = r(P.dx); C.H = r(P.H); C.sigma = r(P.sigma); C.D_s = r(P.D_s); C.D_l = r(P.D_l);
+        C.log_ke = r(std::log(P.k_e)); C.one_m_ke = r(1.0 - P.k_e); C.a = r(P.a); C.G_theta = r(P.G_theta);
         set_coefficients(C);
+        a.inv_dx2 = 1.0 / (P.dx * P.dx);
         a.theta_ref = P.theta_ref; a.G_theta = P.G_theta; a.x0 = P.x0; a.c_inf = P.c_inf;
-        a.gphi = T(D.bc.dir_phi); a.gcs = T(D.bc.dir_cs); a.gcl = T(D.bc.dir_cl);
-        a.gmus = T(std::log(D.bc.dir_cs) - std::log(P.k_e));
-        a.gmul = T(std::log(D.bc.dir_cl));
-        const double pg = p_of_host(P, D.bc.dir_phi);
-        a.fc = T(pg * D.bc.dir_cs + (1.0 - pg) * D.bc.dir_cl);
-        a.fd = T(D.bc.dir_cs - D.bc.dir_cl);
-        a.hot_noflux = D.bc.hi[0] == PF_BC_NOFLUX;
         a.energy_every = D.energy_every;
         a.energy_slots = energy_slots;
         a.energy = energy;
         a.dir_phi = D.bc.dir_phi;
         a.rec = rec;
         a.rec_steps = rec_steps;
-        if constexpr (IsDual<T>::value) {
-            // seed d/dtheta = 1 on the parameter of this group
-            using VT = decltype(C.A.v);
-            if (g.dir == 0) C.inv_Mphi = make_dual<VT>(VT(1.0 / P.M_phi), VT(-1.0 / (P.M_phi * P.M_phi)));
-            if (g.dir == 1) {
-                C.A = make_dual<VT>(VT(P.A), VT(1));
-                C.one_m_A = make_dual<VT>(VT(1.0 - P.A), VT(-1));
-            }
-            if (g.dir == 2) C.b = make_dual<VT>(VT(P.b), VT(1));
-        }
         return a;
     }
 
-    cudaError_t issue(int nsteps) {
+    // `count` launches of nsteps steps each, every group's on its own stream: a
+    // group does not wait for the others' launches until the last is done
+    cudaError_t issue(int nsteps, int count = 1) {
         cudaError_t e = cudaEventRecord(fork, main);
         for (Group& g : groups) {
             if (e == cudaSuccess) e = cudaStreamWaitEvent(g.stream, fork, 0);
-            if (e == cudaSuccess) e = launch_group<T>(g.nt, args(g, nsteps), (size_t)6 * g.nmax * sizeof(T), g.stream);
+            const BatchArgs<T> a = args(g, nsteps);
+            for (int l = 0; l < count && e == cudaSuccess; ++l)
+                e = launch_group<T>(g.warps, J, std_phys, a, (size_t)6 * g.room * sizeof(T), g.stream);
             if (e == cudaSuccess) e = cudaEventRecord(g.done, g.stream);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(main, g.done, 0);
-            launches += 1;
+            launches += count;
         }
         return e;
     }
@@ -554,14 +677,32 @@ struct BatchRun {
             if (g.done) cudaEventDestroy(g.done);
         }
         groups.clear();
+        J = cells_per_lane<T>(cpt);
+        std_phys = line_std(problem());
+        // an instance is spread over a cluster where that fills SMs that would
+        // otherwise have no instance
+        const int64_t use = 30 * J;
+        int64_t most = 0;
+        for (int i = 0; i < D.n_instances; ++i) most = std::max(most, (D.n[i] + J + use - 1) / use);
+        cluster = 1;
+        while (2 * cluster <= BATCH_CLUSTER && 2 * cluster <= most && (int64_t)2 * cluster * D.n_instances <= sms)
+            cluster *= 2;
         std::map<std::pair<int, int>, Group> by;
         for (int i = 0; i < D.n_instances; ++i) {
-            const int nt = threads_for(D.n[i], cpt);
+            const int64_t strips = ((D.n[i] + J + use - 1) / use + cluster - 1) / cluster;
+            // few block sizes, so that few launches make up a chunk
+            const int top = batch_warps<T>();
+            int w = warps_for(strips, top);
+            for (int step : {1, 2, 4, 6, 9, 12, 16})
+                if (w <= step) {
+                    w = std::min(step, top);
+                    break;
+                }
             const int dir = rep_dir.empty() ? -1 : rep_dir[i];
-            Group& g = by[{nt, dir}];
-            g.nt = nt;
+            Group& g = by[{w, dir}];
+            g.warps = w;
             g.dir = dir;
-            g.nmax = std::max(g.nmax, (int)D.n[i]);
+            g.room = std::max(g.room, (int)(strips * use + 2 * J));
             g.ids.push_back(i);
         }
         // largest instances first inside a group: the long CTAs start early
@@ -657,11 +798,11 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
     cudaFree(scs);
     cudaFree(scl);
     size_t max_dyn = 0;
-    if (e == cudaSuccess) e = set_smem_limits<T>(&max_dyn);
+    if (e == cudaSuccess) e = set_smem_limits<T>(&max_dyn, &B.sms);
     if (e == cudaSuccess) {
         int64_t nbig = 0;
         for (int i = 0; i < N; ++i) nbig = std::max(nbig, (int64_t)D.n[i]);
-        if ((size_t)6 * nbig * sizeof(T) > max_dyn) {
+        if ((size_t)6 * (nbig + 34 * batch_jmax<T>()) * sizeof(T) > max_dyn) {   // a copy's padding included
             err = "longest instance does not fit in shared memory";
             return PF_EINVAL;
         }
@@ -674,9 +815,14 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         return PF_ECUDA;
     }
 
-    // autotune the cells per thread: time a short probe of every candidate on a
-    // scratch copy of the initial state
+    // The cells per lane: the one kernel there is (FP64); for a short run two
+    // where the instances leave SMs over for clusters (the run is then bound by
+    // the latency of a step) and four otherwise; for a run of at least 1024 steps,
+    // in which it is 6 % at most, a timed probe of both on a scratch copy of the
+    // initial state.
     int cpt = D.cells_per_thread;
+    if (cpt == 0 && batch_jmax<T>() == 2) cpt = 2;
+    if (cpt == 0 && D.max_steps < 1024) cpt = 2 * N <= B.sms ? 2 : 4;
     if (cpt == 0) {
         T *bp = nullptr, *bc = nullptr, *bd = nullptr;
         e = cudaMalloc(&bp, fb);
@@ -687,12 +833,8 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         if (e == cudaSuccess) e = cudaMemcpyAsync(bd, B.d, fb, cudaMemcpyDeviceToDevice, main);
         float best = 1e30f;
         const int probe = 32;
-        for (int cand : {1, 2, 4, 8}) {
+        for (int cand : {2, 4}) {
             if (e != cudaSuccess) break;
-            bool ok = true;
-            for (int i = 0; i < N; ++i)
-                if (D.n[i] > (int64_t)1024 * cand) ok = false;
-            if (!ok) continue;
             e = B.make_groups(cand);
             if (e == cudaSuccess) e = cudaEventRecord(B.t0, main);
             if (e == cudaSuccess) e = B.issue(probe);
@@ -730,7 +872,7 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     e = cudaStreamBeginCapture(main, cudaStreamCaptureModeThreadLocal);
-    for (int l = 0; l < D.launches_per_graph && e == cudaSuccess; ++l) e = B.issue((int)D.steps_per_launch);
+    if (e == cudaSuccess) e = B.issue((int)D.steps_per_launch, D.launches_per_graph);
     cudaError_t e2 = cudaStreamEndCapture(main, &graph);
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
@@ -1029,11 +1171,11 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
         e = cudaGetLastError();
     }
     size_t max_dyn = 0;
-    if (e == cudaSuccess) e = set_smem_limits<T>(&max_dyn);
+    if (e == cudaSuccess) e = set_smem_limits<T>(&max_dyn, &B.sms);
     if (e == cudaSuccess) {
         int64_t nbig = 0;
         for (int i = 0; i < N; ++i) nbig = std::max(nbig, (int64_t)D.n[i]);
-        if ((size_t)6 * nbig * sizeof(T) > max_dyn) {
+        if ((size_t)6 * (nbig + 34 * batch_jmax<T>()) * sizeof(T) > max_dyn) {   // a copy's padding included
             free_tmp();
             err = "longest instance does not fit in shared memory";
             return PF_EINVAL;
@@ -1579,6 +1721,20 @@ static RevFn<V> reverse_for(int64_t nmax) {
     return reverse_kernel<V, 512, 8>;
 }
 
+// the step's parameters in the arithmetic type, as the reverse sweep uses them
+template <typename V>
+static Consts<V> value_consts_T(const pf_batch_desc& D) {
+    const pf_params& P = D.params;
+    Consts<V> C = {};
+    C.dim = 1; C.interp = P.interp; C.lap = 3; C.mobility = P.mobility_mode;
+    C.dx = V(D.dx); C.inv_dx = V(1.0 / D.dx); C.inv_2dx = V(0.5 / D.dx); C.inv_dx2 = V(1.0 / (D.dx * D.dx));
+    C.H = V(P.H); C.sigma = V(P.sigma); C.inv_Mphi = V(1.0 / P.M_phi); C.D_s = V(P.D_s); C.D_l = V(P.D_l);
+    C.log_ke = V(std::log(P.k_e)); C.one_m_ke = V(1.0 - P.k_e); C.A = V(P.A); C.one_m_A = V(1.0 - P.A);
+    C.b = V(P.b); C.a = V(P.a); C.delta2 = V(P.delta * P.delta); C.G_theta = V(P.G_theta);
+    set_coefficients(C);
+    return C;
+}
+
 template <typename V>
 static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStream_t main, std::string& err) {
     constexpr int NT = 512;
@@ -1653,7 +1809,7 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
         e = cudaGetLastError();
     }
     size_t max_dyn = 0;
-    if (e == cudaSuccess) e = set_smem_limits<V>(&max_dyn);
+    if (e == cudaSuccess) e = set_smem_limits<V>(&max_dyn, &B.sms);
     const size_t rsmem = (size_t)13 * nmax * sizeof(V);
     if (e == cudaSuccess) {
         static DeviceSetup setup;
@@ -1680,7 +1836,7 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
             }
         }
     }
-    if (e == cudaSuccess && (size_t)6 * nmax * sizeof(V) > max_dyn) {
+    if (e == cudaSuccess && (size_t)6 * (nmax + 34 * batch_jmax<V>()) * sizeof(V) > max_dyn) {
         free_tmp();
         err = "longest instance does not fit in shared memory";
         return PF_EINVAL;
@@ -1752,15 +1908,15 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
             ra.v = B.dv;
             ra.dt = B.ddt;
             ra.nsteps = (int)len;
-            ra.C = ba.C;
+            ra.C = value_consts_T<V>(D);
             ra.theta_ref = ba.theta_ref;
             ra.G_theta = ba.G_theta;
             ra.x0 = ba.x0;
-            ra.gphi = ba.gphi;
-            ra.gcs = ba.gcs;
-            ra.gcl = ba.gcl;
-            ra.gmus = ba.gmus;
-            ra.gmul = ba.gmul;
+            ra.gphi = V(D.bc.dir_phi);
+            ra.gcs = V(D.bc.dir_cs);
+            ra.gcl = V(D.bc.dir_cl);
+            ra.gmus = V(std::log(D.bc.dir_cs) - std::log(D.params.k_e));
+            ra.gmul = V(std::log(D.bc.dir_cl));
             reverse_for<V>(nmax)<<<N, NT, rsmem, rs>>>(ra);
             e = cudaGetLastError();
         }
