@@ -55,10 +55,18 @@ struct BatchState {
 
 template <typename T>
 struct BatchArgs {
-    T* phi;             // packed fields
-    T* c;
-    T* d;
-    BatchState* st;
+    const T* phi;       // packed fields before the launch
+    const T* c;
+    const T* d;
+    const BatchState* st;
+    T* phi_out;         // and after it (the same arrays, or others)
+    T* c_out;
+    T* d_out;
+    // COMP: the low words of the values of phi, c, d, one array after the other
+    const typename LineNum<T>::S* low;
+    typename LineNum<T>::S* low_out;
+    long long low_stride;
+    BatchState* st_out;
     const int* ids;     // instances of this launch group
     const double* v;    // per-instance pulling velocity
     const double* dt;   // per-instance time step
@@ -76,7 +84,7 @@ struct BatchArgs {
     double* energy;                 // [instance][slot] F_h records (device)
     double dir_phi;                 // hot-end ghost phi, for the gradient energy
     T* rec;                         // if set: every step's state and intermediates,
-                                    // [instance block of 6 rec_steps n][step][phi|c|d|mu_s|mu_l|phidot][n]
+                                    // [instance block of 6 rec_steps n][step][phi|c_s|c_l|mu_s|mu_l|dx^2 phidot][n]
     long long rec_steps;
     double inv_dx2;
 };
@@ -98,14 +106,13 @@ constexpr int batch_warps() {
 constexpr int BATCH_WARPS = 16;     // the largest of them
 constexpr int BATCH_CLUSTER = 8;    // CTAs per instance at most
 
-// a pair's state before the step and its potentials and rate, into the record
+// a pair's phi, c_s and c_l before the step and its potentials and rate, into the record
 // of the step (cells i of the line go to i - m)
 template <typename T, int J>
 struct LineRecord {
     using X = typename LineNum<T>::X;
     T* base;          // nullptr: nothing is recorded
     int n, i0, m;
-    double inv_dx2;
     static constexpr bool on = true;
     __device__ __forceinline__ void one(int i, T f, T c, T d, T s, T l, T r) const {
         if (i < 0 || i >= n) return;
@@ -114,7 +121,7 @@ struct LineRecord {
         base[2 * n + i] = d;
         base[3 * n + i] = s;
         base[4 * n + i] = l;
-        base[5 * n + i] = r * T(inv_dx2);
+        base[5 * n + i] = r;
     }
     __device__ __forceinline__ void operator()(int q, const X& f, const X& c, const X& d, const X& s, const X& l,
                                                const X& r) const {
@@ -155,7 +162,12 @@ __device__ __forceinline__ void store_cells(T* p, const T (&w)[J]) {
 // through registers (pf_line.cuh) into the other, so that there is one barrier
 // per block and none inside it.  Cells at a segment's ends are also written to
 // the neighbouring CTA's copy of them (distributed shared memory).
-template <typename T, int J, bool STD, bool REC>
+//
+// MODE: a plain run, or one for derivatives without and with records.  COMP: the
+// values of phi, c and d are kept as unevaluated FP32 pairs in the runs for
+// derivatives, whose error is mostly that of the values' accumulated rounding.
+enum { BATCH_PLAIN = 0, BATCH_DERIV = 1, BATCH_RECORD = 2 };
+template <typename T, int J, bool STD, int MODE>
 __global__ void __launch_bounds__(32 * batch_warps<T>())
 batch_kernel(const __grid_constant__ BatchArgs<T> a) {
     using X = typename LineNum<T>::X;
@@ -163,9 +175,11 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
     using S = typename LineNum<T>::S;
     constexpr int H = J / 2;
     constexpr int USE = 30 * J;      // cells of a strip that hold results
+    constexpr bool REC = MODE == BATCH_RECORD;
+    constexpr bool COMP = MODE != BATCH_PLAIN && sizeof(S) == 4;
     const int csize = a.cluster;
     const int inst = a.ids[blockIdx.x / csize];
-    BatchState& St = a.st[inst];
+    const BatchState St = a.st[inst];
     if (St.converged) return;        // the same for every CTA of the cluster
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = csize > 1 ? (int)cluster.block_rank() : 0;
@@ -189,6 +203,7 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
     const long long off = St.off;
     const int room = a.room;                    // cells of one field: J + segment + J
     T* const sm = reinterpret_cast<T*>(smem) + J;   // own cell 0 of the first field
+    S* const sl = reinterpret_cast<S*>(reinterpret_cast<T*>(smem) + 6 * room) + J;   // and of its low word
     for (int i = tid - J; i < room - J; i += NT) {
         const int g = lo + i;
         const bool in = g >= 0 && g < n;
@@ -198,6 +213,14 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
             sm[3 * b * room + i] = f;
             sm[(3 * b + 1) * room + i] = c;
             sm[(3 * b + 2) * room + i] = d;
+        }
+        if constexpr (COMP) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const S l = in ? a.low[k * a.low_stride + off + g] : k == 0 ? K.gphi_lo : k == 1 ? K.fc_lo : K.fd_lo;
+                sl[k * room + i] = l;
+                sl[(3 + k) * room + i] = l;
+            }
         }
     }
     long long step = St.step, shifts = St.shifts;
@@ -251,7 +274,7 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
         for (int u = warp * USE; u < mine; u += warps * USE) {
             const int w0 = u + (lane - 1) * J;            // own index; lane 0 and lane 31: the strip's stale ends
             const int i0 = lo + w0;
-            Strip<T, J, false> s;
+            Strip<T, J, COMP> s;
             {
                 const T* p = sm + cur + w0;
                 T w[J];
@@ -263,6 +286,18 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
                 get(p, s.phi);
                 get(p + room, s.c);
                 get(p + 2 * room, s.d);
+                if constexpr (COMP) {
+                    const S* l = sl + cur + w0;
+                    S z[J];
+                    auto getl = [&](const S* q, V (&x)[H]) {
+                        load_cells<J>(q, z);
+#pragma unroll
+                        for (int k = 0; k < H; ++k) x[k] = x_pair(z[k], z[k + H]);
+                    };
+                    getl(l, s.plo);
+                    getl(l + room, s.clo);
+                    getl(l + 2 * room, s.dlo);
+                }
             }
             // an end of the line in the strip
             const bool edge = lo + u < mt + J + 1 || lo + u + USE + J >= n;
@@ -278,10 +313,9 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
                         rec.n = n;
                         rec.i0 = i0;
                         rec.m = m;
-                        rec.inv_dx2 = a.inv_dx2;
-                        line_step<STD, EDGE, T, J, false>(K, s, i0, n, m, dtq, th0[tab + k], rec);
+                        line_step<STD, EDGE, T, J, COMP>(K, s, i0, n, m, dtq, th0[tab + k], rec);
                     } else {
-                        line_step<STD, EDGE, T, J, false>(K, s, i0, n, m, dtq, th0[tab + k], NoRecord());
+                        line_step<STD, EDGE, T, J, COMP>(K, s, i0, n, m, dtq, th0[tab + k], NoRecord());
                     }
                 }
             };
@@ -298,36 +332,64 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
                         }
                         store_cells<J>(q, w);
                     };
-                    auto put3 = [&](T* p) {
+                    auto putl = [&](S* q, const V (&x)[H]) {
+                        S w[J];
+#pragma unroll
+                        for (int k = 0; k < H; ++k) {
+                            w[k] = x[k].x;
+                            w[k + H] = x[k].y;
+                        }
+                        store_cells<J>(q, w);
+                    };
+                    auto put3 = [&](T* p, S* l) {
                         put(p, s.phi);
                         put(p + room, s.c);
                         put(p + 2 * room, s.d);
+                        if constexpr (COMP) {
+                            putl(l, s.plo);
+                            putl(l + room, s.clo);
+                            putl(l + 2 * room, s.dlo);
+                        }
                     };
                     T* const p = sm + nxt + w0;
-                    put3(p);
+                    S* const l = sl + nxt + w0;
+                    put3(p, l);
                     // the neighbours' copies of this CTA's first and last cells
                     if (csize > 1) {
-                        if (w0 == 0 && rank > 0) put3(cluster.map_shared_rank(p + seg, rank - 1));
-                        if (w0 + J == seg && rank < csize - 1) put3(cluster.map_shared_rank(p - seg, rank + 1));
+                        auto put_at = [&](int by, int r) {
+                            put3(cluster.map_shared_rank(p + by, r), cluster.map_shared_rank(l + by, r));
+                        };
+                        if (w0 == 0 && rank > 0) put_at(seg, rank - 1);
+                        if (w0 + J == seg && rank < csize - 1) put_at(-seg, rank + 1);
                     }
                 } else {
 #pragma unroll
                     for (int k = 0; k < J; ++k) {
                         const int i = i0 + k - mt;      // the window has dropped mt cells
                         if (i < 0) continue;
-                        auto put1 = [&](T* q) {
+                        // cell l of CTA r
+                        auto put1 = [&](int l, int r) {
+                            T* q = sm + nxt + l;
+                            S* z = sl + nxt + l;
+                            if (r != rank) {
+                                q = cluster.map_shared_rank(q, r);
+                                z = cluster.map_shared_rank(z, r);
+                            }
                             q[0] = k < H ? x_lo(s.phi[k % H]) : x_hi(s.phi[k % H]);
                             q[room] = k < H ? x_lo(s.c[k % H]) : x_hi(s.c[k % H]);
                             q[2 * room] = k < H ? x_lo(s.d[k % H]) : x_hi(s.d[k % H]);
+                            if constexpr (COMP) {
+                                z[0] = k < H ? s.plo[k % H].x : s.plo[k % H].y;
+                                z[room] = k < H ? s.clo[k % H].x : s.clo[k % H].y;
+                                z[2 * room] = k < H ? s.dlo[k % H].x : s.dlo[k % H].y;
+                            }
                         };
                         const int r = i >= lo ? rank : rank - 1;     // mt < seg
                         const int l = i - r * seg;
-                        T* const q = sm + nxt + l;
-                        put1(r == rank ? q : cluster.map_shared_rank(q, r));
+                        put1(l, r);
                         if (csize > 1) {
-                            if (l < J && r > 0) put1(cluster.map_shared_rank(q + seg, r - 1));
-                            if (l >= seg - J && r < csize - 1)
-                                put1(r + 1 == rank ? q - seg : cluster.map_shared_rank(q - seg, r + 1));
+                            if (l < J && r > 0) put1(l + seg, r - 1);
+                            if (l >= seg - J && r < csize - 1) put1(l - seg, r + 1);
                         }
                     }
                 }
@@ -434,34 +496,37 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
         }
     }
     for (int i = tid; i < min(mine, n - lo); i += NT) {
-        a.phi[off + lo + i] = sm[cur + i];
-        a.c[off + lo + i] = sm[cur + room + i];
-        a.d[off + lo + i] = sm[cur + 2 * room + i];
+        a.phi_out[off + lo + i] = sm[cur + i];
+        a.c_out[off + lo + i] = sm[cur + room + i];
+        a.d_out[off + lo + i] = sm[cur + 2 * room + i];
+        if constexpr (COMP)
+            for (int k = 0; k < 3; ++k) a.low_out[k * a.low_stride + off + lo + i] = sl[cur + k * room + i];
     }
-    if (tid == 0 && rank == 0) {
-        St.step = step;
-        St.shifts = shifts;
-        St.k_prev = k_prev;
-        St.t_prev = t_prev;
-        St.k_last = k_last;
-        St.dkdt_last = dkdt_last;
-        St.converged = converged;
-    }
+    if (tid == 0 && rank == 0)
+        a.st_out[inst] = BatchState{off, n, converged, step, shifts, k_prev, t_prev, k_last, dkdt_last};
 }
 
 
-// (phi, c_s, c_l) -> (phi, c, d) for packed instances
+// (phi, c_s, c_l) -> (phi, c, d) for packed instances, with their low words
+// [phi, c, d][n] if low is set
 template <typename T>
 __global__ void batch_to_state(const T* __restrict__ cs, const T* __restrict__ cl, T* __restrict__ phi,
-                               T* __restrict__ c, T* __restrict__ d, long long n, int interp, double a) {
+                               T* __restrict__ c, T* __restrict__ d, long long n, int interp, double a,
+                               T* __restrict__ low = nullptr) {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         const double f = (double)phi[i], s = (double)cs[i], l = (double)cl[i];
         const double g = f * (1.0 - f);
         const double h = (interp == 1) ? f * f * (3.0 - 2.0 * f) : f * f * f * (6.0 * f * f - 15.0 * f + 10.0);
         const double p = h + a * (f - 0.5) * g * g;
-        c[i] = (T)(p * s + (1.0 - p) * l);
-        d[i] = (T)(s - l);
+        const double cc = p * s + (1.0 - p) * l, dd = s - l;
+        c[i] = (T)cc;
+        d[i] = (T)dd;
+        if (low != nullptr) {
+            low[i] = T(0);
+            low[n + i] = (T)(cc - (double)(T)cc);
+            low[2 * n + i] = (T)(dd - (double)(T)dd);
+        }
     }
 }
 
@@ -497,36 +562,62 @@ int warps_for(int64_t strips, int most) {
 
 template <typename T>
 using BatchFn = void (*)(const BatchArgs<T>);
-template <typename T, bool STD, bool REC>
+template <typename T, bool STD, int MODE>
 BatchFn<T> batch_fn_J(int J) {
-    if constexpr (batch_jmax<T>() >= 4)
-        if (J == 4) return batch_kernel<T, 4, STD, REC>;
-    return batch_kernel<T, 2, STD, REC>;
+    if constexpr (batch_jmax<T>() >= 4 && MODE == BATCH_PLAIN)
+        if (J == 4) return batch_kernel<T, 4, STD, MODE>;
+    return batch_kernel<T, 2, STD, MODE>;
 }
-// the instance for J cells per lane, the default physics or not, recording every
-// step or not (a run with derivatives never does)
+// the instance for J cells per lane, the default physics or not, and a mode (in
+// FP64, which has no low words, BATCH_DERIV is the plain run of the values; dual
+// numbers are only run for derivatives and never recorded)
 template <typename T>
-BatchFn<T> batch_fn(int J, bool std_phys, bool rec) {
-    if constexpr (!IsDual<T>::value)
-        if (rec) return std_phys ? batch_fn_J<T, true, true>(J) : batch_fn_J<T, false, true>(J);
-    return std_phys ? batch_fn_J<T, true, false>(J) : batch_fn_J<T, false, false>(J);
+BatchFn<T> batch_fn(int J, bool std_phys, int mode) {
+    if constexpr (IsDual<T>::value) {
+        return std_phys ? batch_fn_J<T, true, BATCH_DERIV>(J) : batch_fn_J<T, false, BATCH_DERIV>(J);
+    } else {
+        if (mode == BATCH_RECORD)
+            return std_phys ? batch_fn_J<T, true, BATCH_RECORD>(J) : batch_fn_J<T, false, BATCH_RECORD>(J);
+        if constexpr (sizeof(T) == 4)
+            if (mode == BATCH_DERIV)
+                return std_phys ? batch_fn_J<T, true, BATCH_DERIV>(J) : batch_fn_J<T, false, BATCH_DERIV>(J);
+        return std_phys ? batch_fn_J<T, true, BATCH_PLAIN>(J) : batch_fn_J<T, false, BATCH_PLAIN>(J);
+    }
+}
+// bytes of shared memory per cell of a CTA: two copies of the state
+template <typename T>
+size_t batch_cell_bytes(int mode) {
+    using S = typename LineNum<T>::S;
+    return 2 * 3 * (sizeof(T) + (mode != BATCH_PLAIN && sizeof(S) == 4 ? sizeof(S) : 0));
 }
 
-template <typename T>
-cudaError_t launch_group(int warps, int J, bool std_phys, const BatchArgs<T>& a, size_t smem, cudaStream_t s) {
+// `count` clusters of `cluster` CTAs (1: a plain launch)
+template <typename Args>
+cudaError_t launch_clusters(void (*kern)(const Args), int count, int cluster, int warps, size_t smem, cudaStream_t s,
+                            const Args& a) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.count * a.cluster);
+    cfg.gridDim = dim3(count * cluster);
     cfg.blockDim = dim3(32 * warps);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = a.cluster;
+    at.val.clusterDim.x = cluster;
     at.val.clusterDim.y = 1;
     at.val.clusterDim.z = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = a.cluster > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, batch_fn<T>(J, std_phys, a.rec != nullptr), a);
+    cfg.numAttrs = cluster > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+// CTAs per instance: an instance is spread over a cluster where that fills SMs
+// that would otherwise have no instance (16 fronts of 2048 cells, FP32: 2.9 us
+// per step on one CTA each, 1.5 us on clusters of 8; sizes in between that are
+// no power of two were no faster)
+int cluster_for(int64_t strips, int instances, int sms) {
+    int c = 1;
+    while (2 * c <= BATCH_CLUSTER && 2 * c <= strips && (int64_t)2 * c * instances <= sms) c *= 2;
+    return c;
 }
 
 // raise each instantiation's dynamic shared-memory limit to what the device
@@ -552,7 +643,7 @@ cudaError_t set_smem_limits(size_t* max_dynamic, int* sms) {
         int optin = 0;
         e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         for (int J = 2; J <= batch_jmax<T>(); J *= 2) {
-            for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = raise_smem(batch_fn<T>(J, i & 1, i & 2), optin);
+            for (int i = 0; i < 6 && e == cudaSuccess; ++i) e = raise_smem(batch_fn<T>(J, i & 1, i / 2), optin);
         }
         int n = 1;
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
@@ -586,11 +677,15 @@ struct BatchRun {
     std::vector<double> dt;
     T *phi = nullptr, *c = nullptr, *d = nullptr;
     BatchState* st = nullptr;
+    typename LineNum<T>::S* low = nullptr;   // runs for derivatives, FP32: [copy][phi, c, d][total] low words
+    bool deriv = false;                      // a run for derivatives
+    int64_t slot_in = 0, slot_out = 0;   // the copies of the state a launch reads and writes
     double *dv = nullptr, *ddt = nullptr;
     std::vector<Group> groups;
     int J = 2, cluster = 1;     // cells per lane and CTAs per instance of the groups
     bool std_phys = false;
     int sms = 1;
+    size_t max_dyn = 0;         // dynamic shared memory of a CTA
     std::vector<int> rep_dir;   // tangent runs: seeded parameter of each instance
     double* energy = nullptr;   // F_h records [instance][slot] (device), or null
     int energy_slots = 0;
@@ -606,13 +701,15 @@ struct BatchRun {
             if (g.stream) cudaStreamDestroy(g.stream);
             if (g.done) cudaEventDestroy(g.done);
         }
-        void* ptrs[] = {phi, c, d, st, dv, ddt, energy};
+        void* ptrs[] = {phi, c, d, st, dv, ddt, energy, low};
         for (void* p : ptrs)
             if (p) cudaFree(p);
         if (fork) cudaEventDestroy(fork);
         if (t0) cudaEventDestroy(t0);
         if (t1) cudaEventDestroy(t1);
     }
+
+    int mode() const { return rec ? BATCH_RECORD : low ? BATCH_DERIV : BATCH_PLAIN; }
 
     // the line of the batch as a problem description (lengths and clocks are the instances')
     HostProblem problem() const {
@@ -624,7 +721,13 @@ struct BatchRun {
 
     BatchArgs<T> args(const Group& g, int nsteps) const {
         BatchArgs<T> a;
-        a.phi = phi; a.c = c; a.d = d; a.st = st; a.ids = g.d_ids; a.v = dv; a.dt = ddt;
+        const int64_t i = slot_in * total, o = slot_out * total;
+        a.phi = phi + i; a.c = c + i; a.d = d + i; a.st = st + slot_in * D.n_instances;
+        a.phi_out = phi + o; a.c_out = c + o; a.d_out = d + o; a.st_out = st + slot_out * D.n_instances;
+        a.low = low + (low ? 3 * i : 0);
+        a.low_out = low + (low ? 3 * o : 0);
+        a.low_stride = total;
+        a.ids = g.d_ids; a.v = dv; a.dt = ddt;
         a.count = (int)g.ids.size();
         a.nsteps = nsteps;
         a.check_every = (int)D.check_every;
@@ -662,7 +765,8 @@ struct BatchRun {
             if (e == cudaSuccess) e = cudaStreamWaitEvent(g.stream, fork, 0);
             const BatchArgs<T> a = args(g, nsteps);
             for (int l = 0; l < count && e == cudaSuccess; ++l)
-                e = launch_group<T>(g.warps, J, std_phys, a, (size_t)6 * g.room * sizeof(T), g.stream);
+                e = launch_clusters(batch_fn<T>(J, std_phys, mode()), a.count, cluster, g.warps,
+                                    g.room * batch_cell_bytes<T>(mode()), g.stream, a);
             if (e == cudaSuccess) e = cudaEventRecord(g.done, g.stream);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(main, g.done, 0);
             launches += count;
@@ -677,15 +781,15 @@ struct BatchRun {
             if (g.done) cudaEventDestroy(g.done);
         }
         groups.clear();
-        J = cells_per_lane<T>(cpt);
+        J = deriv ? 2 : cells_per_lane<T>(cpt);
         std_phys = line_std(problem());
-        // an instance is spread over a cluster where that fills SMs that would
-        // otherwise have no instance
         const int64_t use = 30 * J;
         int64_t most = 0;
         for (int i = 0; i < D.n_instances; ++i) most = std::max(most, (D.n[i] + J + use - 1) / use);
-        cluster = 1;
-        while (2 * cluster <= BATCH_CLUSTER && 2 * cluster <= most && (int64_t)2 * cluster * D.n_instances <= sms)
+        cluster = cluster_for(most, D.n_instances, sms);
+        // a segment has to fit a CTA's shared memory
+        const size_t cell = batch_cell_bytes<T>(deriv ? BATCH_DERIV : BATCH_PLAIN);
+        while (2 * cluster <= BATCH_CLUSTER && ((most + cluster - 1) / cluster * use + 2 * J) * cell > max_dyn)
             cluster *= 2;
         std::map<std::pair<int, int>, Group> by;
         for (int i = 0; i < D.n_instances; ++i) {
@@ -797,12 +901,11 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
     if (e == cudaSuccess) e = cudaStreamSynchronize(main);
     cudaFree(scs);
     cudaFree(scl);
-    size_t max_dyn = 0;
-    if (e == cudaSuccess) e = set_smem_limits<T>(&max_dyn, &B.sms);
+    if (e == cudaSuccess) e = set_smem_limits<T>(&B.max_dyn, &B.sms);
     if (e == cudaSuccess) {
         int64_t nbig = 0;
         for (int i = 0; i < N; ++i) nbig = std::max(nbig, (int64_t)D.n[i]);
-        if ((size_t)6 * (nbig + 34 * batch_jmax<T>()) * sizeof(T) > max_dyn) {   // a copy's padding included
+        if ((size_t)6 * (nbig + 34 * batch_jmax<T>()) * sizeof(T) > B.max_dyn) {   // a copy's padding included
             err = "longest instance does not fit in shared memory";
             return PF_EINVAL;
         }
@@ -1039,7 +1142,8 @@ int run_batch(const pf_batch_desc* D, pf_batch_result* R, void* stream, std::str
 // depend on the parameters)
 template <typename V>
 __global__ void adjoint_replicate(const V* __restrict__ phi, const V* __restrict__ c, const V* __restrict__ d,
-                                  long long total, int reps, Dual<V>* P, Dual<V>* Cc, Dual<V>* Dd) {
+                                  const V* __restrict__ low, long long total, int reps, Dual<V>* P, Dual<V>* Cc,
+                                  Dual<V>* Dd, V* __restrict__ L) {
     const long long n = total * reps;
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (long long)gridDim.x * blockDim.x) {
@@ -1047,20 +1151,22 @@ __global__ void adjoint_replicate(const V* __restrict__ phi, const V* __restrict
         P[k] = make_dual<V>(phi[s], V(0));
         Cc[k] = make_dual<V>(c[s], V(0));
         Dd[k] = make_dual<V>(d[s], V(0));
+        if (low != nullptr)
+            for (int q = 0; q < 3; ++q) L[q * n + k] = low[q * total + s];
     }
 }
 
 // per replica: max_x c and the derivative of c at the maximising cell (lowest
 // index among ties)
 template <typename V>
-__global__ void __launch_bounds__(256) adjoint_cmax(const Dual<V>* __restrict__ c, const BatchState* __restrict__ st,
-                                                    double* __restrict__ out) {
+__global__ void __launch_bounds__(256) adjoint_cmax(const Dual<V>* __restrict__ c, const V* __restrict__ clo,
+                                                    const BatchState* __restrict__ st, double* __restrict__ out) {
     const BatchState S = st[blockIdx.x];
     double best = -INFINITY, tan = 0.0;
     int bi = 0x7fffffff;
     for (int i = threadIdx.x; i < S.n; i += blockDim.x) {
         const Dual<V> x = c[S.off + i];
-        const double v = (double)x.v;
+        const double v = (double)x.v + (clo != nullptr ? (double)clo[S.off + i] : 0.0);
         if (v > best || (v == best && i < bi)) {
             best = v;
             tan = (double)x.t;
@@ -1132,7 +1238,8 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
         B.total += rn[r];
     }
     const size_t fb = (size_t)B.total * sizeof(T), vb = (size_t)total1 * sizeof(V);
-    V *vphi = nullptr, *vcs = nullptr, *vcl = nullptr, *vc = nullptr, *vd = nullptr;
+    B.deriv = true;
+    V *vphi = nullptr, *vcs = nullptr, *vcl = nullptr, *vc = nullptr, *vd = nullptr, *vlow = nullptr;
     double* dout = nullptr;
     cudaError_t e = cudaMalloc(&B.phi, fb);
     if (e == cudaSuccess) e = cudaMalloc(&B.c, fb);
@@ -1145,9 +1252,11 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
     if (e == cudaSuccess) e = cudaMalloc(&vcl, vb);
     if (e == cudaSuccess) e = cudaMalloc(&vc, vb);
     if (e == cudaSuccess) e = cudaMalloc(&vd, vb);
+    if (e == cudaSuccess && sizeof(V) == 4) e = cudaMalloc(&vlow, 3 * vb);
+    if (e == cudaSuccess && sizeof(V) == 4) e = cudaMalloc(&B.low, 3 * (size_t)B.total * sizeof(V));
     if (e == cudaSuccess) e = cudaMalloc(&dout, 2 * M * sizeof(double));
     auto free_tmp = [&] {
-        void* ptrs[] = {vphi, vcs, vcl, vc, vd, dout};
+        void* ptrs[] = {vphi, vcs, vcl, vc, vd, vlow, dout};
         for (void* p : ptrs)
             if (p) cudaFree(p);
     };
@@ -1166,16 +1275,15 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
     if (e == cudaSuccess) e = cudaMemcpyAsync(B.dv, rv.data(), M * sizeof(double), cudaMemcpyHostToDevice, main);
     if (e == cudaSuccess) e = cudaMemcpyAsync(B.ddt, rdt.data(), M * sizeof(double), cudaMemcpyHostToDevice, main);
     if (e == cudaSuccess) {
-        batch_to_state<V><<<1216, 256, 0, main>>>(vcs, vcl, vphi, vc, vd, total1, D.params.interp, D.params.a);
-        adjoint_replicate<V><<<1216, 256, 0, main>>>(vphi, vc, vd, total1, ND, B.phi, B.c, B.d);
+        batch_to_state<V><<<1216, 256, 0, main>>>(vcs, vcl, vphi, vc, vd, total1, D.params.interp, D.params.a, vlow);
+        adjoint_replicate<V><<<1216, 256, 0, main>>>(vphi, vc, vd, vlow, total1, ND, B.phi, B.c, B.d, B.low);
         e = cudaGetLastError();
     }
-    size_t max_dyn = 0;
-    if (e == cudaSuccess) e = set_smem_limits<T>(&max_dyn, &B.sms);
+    if (e == cudaSuccess) e = set_smem_limits<T>(&B.max_dyn, &B.sms);
     if (e == cudaSuccess) {
         int64_t nbig = 0;
         for (int i = 0; i < N; ++i) nbig = std::max(nbig, (int64_t)D.n[i]);
-        if ((size_t)6 * (nbig + 34 * batch_jmax<T>()) * sizeof(T) > max_dyn) {   // a copy's padding included
+        if ((size_t)6 * (nbig + 34 * batch_jmax<T>()) * sizeof(T) > B.max_dyn) {   // a copy's padding included
             free_tmp();
             err = "longest instance does not fit in shared memory";
             return PF_EINVAL;
@@ -1192,7 +1300,7 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
         e = B.issue((int)std::min(chunk, A.nsteps - done));
     if (e == cudaSuccess) e = cudaEventRecord(B.t1, main);
     if (e == cudaSuccess) {
-        adjoint_cmax<V><<<M, 256, 0, main>>>(B.c, B.st, dout);
+        adjoint_cmax<V><<<M, 256, 0, main>>>(B.c, B.low ? B.low + B.total : nullptr, B.st, dout);
         e = cudaGetLastError();
     }
     std::vector<double> hout(2 * M);
@@ -1228,102 +1336,226 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
 }
 
 // ---------------------------------------------------------------------------
-// Reverse sweep (pf_adjoint, PF_ADJ_REVERSE): the adjoint of one fused 1D step
-// of batch_kernel, applied backwards over recorded states.  lambda = dk/du for
+// Reverse sweep (pf_adjoint, PF_ADJ_REVERSE): the adjoint of one step of
+// batch_kernel, applied backwards over recorded states.  lambda = dk/du for
 // the state u = (phi, c, d) of one instance; the parameter derivatives collect
 // dk/d(1/M_phi), dk/dA, dk/db from every use inside the step.
 
-// p''(phi) (d/dphi of dp_of)
+// constants of the reverse sweep beside the step's
 template <typename T>
-__device__ __forceinline__ T d2p_of(const Consts<T>& C, T f) {
-    const T g = f * (T(1) - f);
-    const T d2h = C.dh1 + f * (T(2) * C.dh2 + f * (T(3) * C.dh3 + f * (T(4) * C.dh4)));
-    const T s = T(1) - T(2) * f;
-    const T dw = T(2) * g * s;
-    return d2h + C.a * (T(2) * dw + (f - T(0.5)) * T(2) * (s * s - T(2) * g));
-}
-
-// adjoints of the inputs of face1 (and of A, b) from those of its outputs (gc, gd)
-template <typename T>
-struct FaceAdj {
-    T f, cs, cl, pd;          // of each of the two cells' phi, c_s, c_l, phidot (half the face's)
-    T nphi, nY, nS, nL;       // of the normal differences
-    T A, b;                   // of the parameters
+struct RevConsts {
+    using V = typename LineNum<T>::V;
+    V A, oA, b, bm1, c4, dx2, H, inv_Mphi;   // oA = 1 - A, bm1 = b - 1, c4 = 4 dx^2
+    T gphi, gcs, gcl, gmus, gmul;            // Dirichlet (hot end) ghost
 };
 
-template <typename T>
-__device__ void face1_rev(const Consts<T>& C, T fL, T fR, T csL, T csR, T clL, T clR, T pdL, T pdR,
-                          T nphi, T nY, T nS, T nL, T gc, T gd, FaceAdj<T>& o) {
-    // forward values (as face1)
-    const T f = T(0.5) * (fL + fR);
-    const T cs = T(0.5) * (csL + csR), cl = T(0.5) * (clL + clR);
-    const T d = cs - cl;
-    const T pdot = T(0.5) * (pdL + pdR);
-    const T p = p_of(C, f);
-    const T omp = T(1) - p;
-    const T Ms = Ms_of(C, cs), Ml = Ml_of(C, cl);
-    const T bMl = C.b * Ml;
-    const T iM = T(1) / (Ms * omp + bMl * p);
-    const T g2 = C.delta2;
-    const T r = T(1) / (nphi * nphi + g2);
-    const T Ts = Ms * nS * g2;
-    const T Tl = Ml * nL * g2;
-    const T at = C.one_m_A * d * pdot * nphi;
-    const T u = C.b * p + omp;
-    const T q = Ms * Ml * u * iM;
-    const T ppo = p * omp;
-    const T afn = (Ms - bMl) * ppo * iM;
-    const T Ssum = q * nphi * nphi * nY + p * Ts + omp * Tl + at * afn;
+// adjoints of a face's inputs (and of A, b) from those of its fluxes (gc, gd)
+template <typename V>
+struct FaceAdj {
+    V f, cs, cl, pd;          // of each of the two cells' phi, c_s, c_l, rate (half the face's)
+    V nphi, nY, nS, nL;       // of the normal differences
+    V A, b;                   // of the parameters
+};
+
+template <bool STD, typename T, typename V>
+__device__ __forceinline__ void line_face_rev(const LineConsts<T>& K, const RevConsts<T>& R, V fL, V fR, V csL, V csR,
+                                              V clL, V clR, V pdL, V pdR, V n1, V n2, V n3, V gc, V gd,
+                                              FaceAdj<V>& o) {
+    const V half = vlit<V>(0.5), two = vlit<V>(2.0), zero = vlit<V>(0.0);
+    // forward values (line_face)
+    const V f = vmul(vadd(fL, fR), half), cs = vmul(vadd(csL, csR), half), cl = vmul(vadd(clL, clR), half);
+    const V d = vsub(cs, cl), P = vmul(vadd(pdL, pdR), half);
+    const V p = line_p<STD>(K, f);
+    const V omp = vsub(vlit<V>(1.0), p);
+    const V Ms = line_M<STD>(K.Ms_c, K.Ms_0, cs), Ml = line_M<STD>(K.Ml_c, K.Ml_0, cl);
+    const V bMl = vmul(R.b, Ml);
+    const V n0 = vsub(fR, fL), nn = vmul(n0, n0);
+    const V M = vfma(bMl, p, vmul(Ms, omp)), G = vadd(nn, K.delta2_dx2);
+    V iM, r;
+    if constexpr (STD) {
+        const V t = vrcp_n(vmul(M, G));
+        iM = vmul(t, G);
+        r = vmul(t, M);
+    } else {
+        iM = vrcp_n(M);
+        r = vrcp_n(G);
+    }
+    // F_c = q n_Y w + rd Z + a e afn, F_d = rd (T_s - T_l) + a e (as line_face with
+    // a derivative, whose comment gives the reason)
+    const V rd = vmul(K.delta2_dx2, r), w = vmul(nn, r), e = vmul(n0, r);
+    const V Ts = vmul(Ms, n2), Tl = vmul(Ml, n3), TD = vsub(Ts, Tl);
+    const V oAd = vmul(R.oA, d), av = vmul(oAd, P);
+    const V u = vfma(R.b, p, omp), ui = vmul(u, iM), MsMl = vmul(Ms, Ml), q = vmul(MsMl, ui);
+    const V ppo = vmul(p, omp), D = vsub(Ms, bMl), pi = vmul(ppo, iM);
+    const V afn = vmul(D, pi);
     // reverse
-    const T lr = gc * Ssum + gd * (Ts - Tl + at);
-    const T lS = gc * r;
-    const T lTs = lS * p + gd * r;
-    const T lTl = lS * omp - gd * r;
-    const T lat = lS * afn + gd * r;
-    const T lq = lS * nphi * nphi * nY;
-    T lnphi = lS * q * T(2) * nphi * nY;
-    const T lnY = lS * q * nphi * nphi;
-    T lp = lS * (Ts - Tl);
-    const T lafn = lS * at;
-    T lMs = lafn * ppo * iM;
-    T lbMl = -lafn * ppo * iM;
-    lp += lafn * (Ms - bMl) * (omp - p) * iM;
-    T liM = lafn * (Ms - bMl) * ppo;
-    lMs += lq * Ml * u * iM;
-    T lMl = lq * Ms * u * iM;
-    const T lu = lq * Ms * Ml * iM;
-    liM += lq * Ms * Ml * u;
-    lp += lu * (C.b - T(1));
-    T lb = lu * p;
-    const T ld = lat * C.one_m_A * pdot * nphi;
-    const T lpdot = lat * C.one_m_A * d * nphi;
-    lnphi += lat * C.one_m_A * d * pdot;
-    const T lA = -lat * d * pdot * nphi;
-    lMs += lTs * nS * g2;
-    const T lnS = lTs * Ms * g2;
-    lMl += lTl * nL * g2;
-    const T lnL = lTl * Ml * g2;
-    lnphi += lr * (-r * r) * (T(2) * nphi);
-    const T lMb = -liM * iM * iM;
-    lMs += lMb * omp;
-    lp += lMb * (bMl - Ms);
-    lbMl += lMb * p;
-    lMl += lbMl * C.b;
-    lb += lbMl * Ml;
-    T lcs = lMs * C.Ms_c + ld;
-    T lcl = lMl * C.Ml_c - ld;
-    const T lf = lp * dp_of(C, f);
-    o.f = T(0.5) * lf;
-    o.cs = T(0.5) * lcs;
-    o.cl = T(0.5) * lcl;
-    o.pd = T(0.5) * lpdot;
+    const V gcq = vmul(gc, q), gcn = vmul(gc, n1);
+    o.nY = vmul(gcq, w);
+    const V lrd = vfma(gc, vfma(p, TD, Tl), vmul(gd, TD));
+    const V gae = vfma(gc, afn, gd);                      // adjoint of a e
+    const V lnphi = vfma(vmul(vmul(e, rd), two), vsub(vmul(gcq, n1), lrd),
+                         vmul(vmul(av, gae), vmul(r, vsub(rd, w))));
+    const V gr = vmul(gc, rd), gdr = vmul(gd, rd);
+    const V lTs = vfma(gr, p, gdr), lTl = vsub(vmul(gr, omp), gdr);
+    V lp = vmul(gr, TD);
+    const V lafn = vmul(gc, vmul(av, e)), lD = vmul(lafn, D);
+    const V lq = vmul(gcn, w);
+    const V w1 = vmul(lafn, pi);
+    V lMs = vfma(lq, vmul(Ml, ui), w1), lbMl = vsub(zero, w1), lMl = vmul(vmul(lq, Ms), ui);
+    lp = vfma(lD, vmul(iM, vsub(omp, p)), lp);
+    const V lqM = vmul(lq, MsMl), lu = vmul(lqM, iM);
+    const V liM = vfma(lD, ppo, vmul(lqM, u));
+    lp = vfma(lu, R.bm1, lp);
+    V lb = vmul(lu, p);
+    const V la = vmul(e, gae);
+    const V loAd = vmul(la, P);                           // adjoint of (1 - A) d
+    const V ld = vmul(loAd, R.oA);
+    o.A = vsub(zero, vmul(loAd, d));
+    o.pd = vmul(vmul(la, oAd), half);
+    lMs = vfma(lTs, n2, lMs);
+    o.nS = vmul(lTs, Ms);
+    lMl = vfma(lTl, n3, lMl);
+    o.nL = vmul(lTl, Ml);
+    const V lMb = vsub(zero, vmul(liM, vmul(iM, iM)));
+    lMs = vfma(lMb, omp, lMs);
+    lp = vsub(lp, vmul(lMb, D));
+    lbMl = vfma(lMb, p, lbMl);
+    lMl = vfma(lbMl, R.b, lMl);
+    o.b = vfma(lbMl, Ml, lb);
     o.nphi = lnphi;
-    o.nY = lnY;
-    o.nS = lnS;
-    o.nL = lnL;
-    o.A = lA;
-    o.b = lb;
+    o.cs = vmul(vfma(lMs, K.Ms_c, ld), half);
+    o.cl = vmul(vsub(vmul(lMl, K.Ml_c), ld), half);
+    o.f = vmul(vmul(lp, line_dp<STD>(K, f)), half);
 }
+
+// adjoints of a rate's inputs from that of the rate, lpd
+template <typename V>
+struct RateAdj {
+    V f, cs, cl, mus, mul, p;   // of the cell's own values (phi without the stencil terms)
+    V lap, gp, gs, gl;          // of the stencil sums f_W - 2 f + f_E, f_E - f_W, mu_E - mu_W
+    V iMphi, A, b;              // of the parameters
+};
+
+template <bool STD, typename T, typename V>
+__device__ __forceinline__ void line_rate_rev(const LineConsts<T>& K, const RevConsts<T>& R, V f, V fL, V fR, V sL,
+                                              V sR, V lL, V lR, V cs, V cl, V mus, V mul, V p, V pd, V ke_theta, V lpd,
+                                              RateAdj<V>& o) {
+    const V zero = vlit<V>(0.0), one = vlit<V>(1.0), two = vlit<V>(2.0);
+    // forward values (line_rate)
+    const V gp = vsub(fR, fL), gs = vsub(sR, sL), gl = vsub(lR, lL);
+    const V dp = line_dp<STD>(K, f);
+    const V omp = vsub(one, p);
+    const V Ms = line_M<STD>(K.Ms_c, K.Ms_0, cs), Ml = line_M<STD>(K.Ml_c, K.Ml_0, cl);
+    const V bMl = vmul(R.b, Ml), Msq = vmul(Ms, omp);
+    const V M = vfma(bMl, p, Msq), G = vfma(gp, gp, K.delta2_4dx2);
+    const V u = vfma(R.b, p, omp);
+    V iM, rr, iu;
+    if constexpr (STD) {
+        const V t = vrcp_n(vmul(M, G));
+        iM = vmul(t, G);
+        rr = vmul(t, M);
+    } else {
+        iM = vrcp_n(M);
+        rr = vrcp_n(G);
+    }
+    iu = vrcp_n(u);
+    const V d = vsub(cs, cl), pq = vmul(p, omp);
+    const V oAb = vmul(R.oA, R.b), dd = vmul(d, d);
+    const V com = vmul(vmul(R.c4, vmul(rr, iM)), iu);              // 4 dx^2 rr / (Mbar u)
+    const V K2 = vmul(vmul(R.oA, oAb), vmul(com, vmul(dd, pq)));
+    const V iKc = vrcp_n(vadd(R.inv_Mphi, K2));
+    const V dmu = vsub(mus, mul);
+    const V AbMl = vmul(R.A, bMl), pp = vmul(p, p), oAo = vsub(one, vmul(R.A, omp));
+    const V Nv = vfma(Msq, oAo, vmul(AbMl, pp));
+    const V Dd = vmul(Nv, iM);
+    const V Ddd = vmul(Dd, d);
+    const V dG = vsub(vsub(vmul(vsub(cs, Ddd), dmu), d), ke_theta);
+    const V W = vsub(vmul(Ms, gs), vmul(bMl, gl));
+    const V X = vmul(vmul(W, gp), rr);
+    // reverse: rate = R / Kc
+    const V lRt = vmul(lpd, iKc);
+    const V lKc = vsub(zero, vmul(lRt, pd));
+    o.iMphi = lKc;
+    o.lap = vmul(lRt, K.sigma);
+    const V lZ = vmul(lRt, R.dx2);
+    const V ldG = vsub(zero, vmul(lZ, dp));
+    const V ldp = vsub(zero, vmul(lZ, dG));
+    // Z = (1-A) d pq iM X
+    const V zi = vmul(lZ, iM), zX = vmul(lZ, X), dpq = vmul(d, pq), oAzX = vmul(R.oA, zX);
+    V loA = vmul(vmul(zX, iM), dpq);
+    const V e1 = vmul(oAzX, iM);
+    V ld = vmul(e1, pq), lpq = vmul(e1, d), liM = vmul(oAzX, dpq);
+    const V lX = vmul(vmul(R.oA, zi), dpq);
+    const V lW = vmul(lX, vmul(gp, rr));
+    // d(gp rr)/dgp = rr (1 - 2 gp^2 rr), without the terms that cancel
+    const V lgp0 = vmul(vmul(vmul(lX, W), rr), vfma(vmul(vmul(gp, gp), rr), vlit<V>(-2.0), one));
+    V lMs = vmul(lW, gs), lbMl = vsub(zero, vmul(lW, gl));
+    o.gs = vmul(lW, Ms);
+    o.gl = vsub(zero, vmul(lW, bMl));
+    // Kc = 1/M_phi + (1-A)^2 b c4 d^2 pq rr iM / u
+    const V ko = vmul(lKc, R.oA), kob = vmul(lKc, oAb);
+    const V kd = vmul(dd, pq);
+    loA = vfma(vmul(two, kob), vmul(com, kd), loA);
+    const V kk = vmul(ko, oAb);                                    // lKc (1-A)^2 b
+    ld = vfma(vmul(two, kk), vmul(com, dpq), ld);
+    V lb = vmul(vmul(ko, R.oA), vmul(com, kd));
+    lpq = vfma(kk, vmul(com, dd), lpq);
+    const V kcd = vmul(vmul(kk, vmul(R.c4, iu)), kd);
+    const V lrr = vmul(kcd, iM);                                   // of Kc's rr alone
+    liM = vfma(kcd, rr, liM);
+    const V lu = vsub(zero, vmul(lKc, vmul(K2, iu)));
+    V lp = vmul(lu, R.bm1);
+    lb = vfma(lu, p, lb);
+    // dG = cs dmu - d - (1-k_e) theta - Dd d dmu
+    V lcs = vmul(ldG, dmu);
+    const V ldmu = vmul(ldG, vsub(cs, Ddd));
+    ld = vsub(ld, vmul(ldG, vfma(Dd, dmu, one)));
+    const V lDd = vsub(zero, vmul(ldG, vmul(d, dmu)));
+    // Dd = Nv iM
+    const V lN = vmul(lDd, iM);
+    liM = vfma(lDd, Nv, liM);
+    V lMsq = vmul(lN, oAo);
+    o.A = vsub(vmul(lN, vsub(vmul(bMl, pp), vmul(Msq, omp))), loA);   // (1-A) = 1 - A
+    lp = vfma(lN, vmul(R.A, vfma(vmul(two, bMl), p, Msq)), lp);
+    lbMl = vfma(lN, vmul(R.A, pp), lbMl);
+    // pq, rr, iM, Msq, bMl, Ms, Ml, d
+    lp = vfma(lpq, vsub(omp, p), lp);
+    o.gp = vsub(lgp0, vmul(vmul(two, lrr), vmul(vmul(rr, rr), gp)));
+    const V lden = vsub(zero, vmul(liM, vmul(iM, iM)));
+    lMsq = vadd(lMsq, lden);
+    lbMl = vfma(lden, p, lbMl);
+    lp = vfma(lden, bMl, lp);
+    lMs = vfma(lMsq, omp, lMs);
+    lp = vsub(lp, vmul(lMsq, Ms));
+    const V lMl = vmul(lbMl, R.b);
+    o.b = vfma(lbMl, Ml, lb);
+    o.cs = vadd(lcs, vfma(lMs, K.Ms_c, ld));
+    o.cl = vsub(vmul(lMl, K.Ml_c), ld);
+    o.mus = ldmu;
+    o.mul = vsub(zero, ldmu);
+    o.p = lp;
+    // phi of the cell itself: f_dw' and p' (f_dw'' = 2 (1 - 6 phi + 6 phi^2))
+    const V ddw = vmul(vfma(f, vfma(f, vlit<V>(6.0), vlit<V>(-6.0)), one), two);
+    o.f = vsub(vmul(ldp, line_d2p<STD>(K, f)), vmul(vmul(lZ, R.H), ddw));
+}
+
+// a running sum kept as an unevaluated pair in FP32 (TwoSum)
+template <typename V>
+struct RunningSum {
+    V hi, lo;
+    __device__ __forceinline__ void add(V x) {
+        if constexpr (sizeof(V) == sizeof(float2)) {
+            const V s = vadd(hi, x), bb = vsub(s, hi);
+            lo = vadd(lo, vadd(vsub(hi, vsub(s, bb)), vsub(x, bb)));
+            hi = s;
+        } else {
+            hi = vadd(hi, x);
+        }
+    }
+    __device__ __forceinline__ double total() const {
+        return ((double)hi.x + (double)hi.y) + ((double)lo.x + (double)lo.y);
+    }
+};
 
 template <typename T>
 struct RevArgs {
@@ -1337,343 +1569,255 @@ struct RevArgs {
     const double* v;
     const double* dt;
     int nsteps;              // steps of this segment (<= RMAX_SEG)
-    Consts<T> C;
-    double theta_ref, G_theta, x0;
-    T gphi, gcs, gcl, gmus, gmul;   // Dirichlet (hot end) ghost
+    int cluster, room;       // as BatchArgs
+    LineConsts<T> K;
+    RevConsts<T> R;
+    double theta_ref, G_theta, x0, dx, inv_dx2;
 };
 
 constexpr int RMAX_SEG = 1024;
+template <typename T>
+constexpr int rev_warps() {
+    return sizeof(T) == 4 ? 12 : 8;   // 168 or 255 registers a thread
+}
 
-template <typename T, int NT, int RJ>
-__global__ void __launch_bounds__(NT, 1) reverse_kernel(RevArgs<T> a) {
-    const int inst = blockIdx.x;
+// Bound by the latency of a step's chain of dependent operations and by the
+// shuffles.  It replaces one CTA of 512 threads per instance with 13 arrays of the
+// line in shared memory and FP64 sums in every thread: 16 fronts of 2048 cells
+// take 4 us per step instead of 21.
+//
+// One instance per cluster, as batch_kernel, with two cells per lane: one step
+// backwards moves information by two cells, so the first and the last lane of a
+// strip are stale after it, and a block is one step.  lambda is kept in the
+// frame of the state before the step that is swept next.
+template <typename T, bool STD>
+__global__ void __launch_bounds__(32 * rev_warps<T>()) reverse_kernel(const __grid_constant__ RevArgs<T> a) {
+    using V = typename LineNum<T>::V;
+    constexpr int J = 2, USE = 30 * J;
+    const int csize = a.cluster;
+    const int inst = blockIdx.x / csize;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = csize > 1 ? (int)cluster.block_rank() : 0;
     const BatchState S0 = a.st0[inst];
     const int n = S0.n;
     const long long off = S0.off;
-    const Consts<T>& C = a.C;
+    const int strips = (n + J + USE - 1) / USE;
+    const int seg = (strips + csize - 1) / csize * USE;
+    const int lo = rank * seg;
+    const int mine = max(0, min(seg, strips * USE - lo));
+    const LineConsts<T>& K = a.K;
+    const RevConsts<T>& R = a.R;
     extern __shared__ __align__(16) unsigned char smem[];
-    T* sF = reinterpret_cast<T*>(smem);   // phi
-    T* sCs = sF + n;                      // c_s
-    T* sCl = sCs + n;                     // c_l
-    T* sMs = sCl + n;                     // mu_s
-    T* sMl = sMs + n;                     // mu_l
-    T* sPd = sMl + n;                     // phidot
-    T* sLf = sPd + n;                     // adjoints of phi, c, d
-    T* sLc = sLf + n;
-    T* sLd = sLc + n;
-    T* sXl = sLd + n;                     // per cell: adjoints of its rate's lap, d_x phi, d_x mu_s, d_x mu_l
-    T* sXg = sXl + n;
-    T* sXs = sXg + n;
-    T* sXm = sXs + n;
     __shared__ int nsh[RMAX_SEG];         // window shifts that followed each step
-    __shared__ double th0[RMAX_SEG];      // theta0 of each step
-    __shared__ double red[NT / 32];
-    const int tid = threadIdx.x;
-    const double v = a.v[inst];
-    const double dtd = a.dt[inst];
-    const T dt = T(dtd);
-    const T dtdx = dt * C.inv_dx;
-    if (tid == 0) {   // replay the clock of batch_kernel over the segment
-        long long step = S0.step, shifts = S0.shifts;
-        for (int it = 0; it < a.nsteps; ++it) {
-            th0[it] = a.theta_ref + a.G_theta * (a.x0 + v * ((double)step * dtd) - (double)shifts * (double)C.dx);
-            step += 1;
-            const double tn = (double)step * dtd;
-            int k = 0;
-            while (v * tn >= (double)(shifts + 1) * (double)C.dx) {
-                shifts += 1;
-                k += 1;
-            }
-            nsh[it] = k;
-        }
-    }
-    for (int i = tid; i < n; i += NT) {
-        sLf[i] = a.lphi[off + i];
-        sLc[i] = a.lc[off + i];
-        sLd[i] = a.ld[off + i];
+    __shared__ double th0[RMAX_SEG];      // (1 - k_e) theta0 of each step
+    __shared__ double red[rev_warps<T>()][3], cred[BATCH_CLUSTER][3];
+    const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, warps = NT >> 5;
+    const int room = a.room;
+    T* const sm = reinterpret_cast<T*>(smem) + J;
+    const double v = a.v[inst], dtd = a.dt[inst];
+    V dtq;
+    dtq.x = dtq.y = T(dtd * a.inv_dx2);
+    // batch_kernel's clock over the segment: the shifts after j steps are the
+    // smallest count, from the segment's start on, that the distance covers
+    auto shifts_at = [&](int j) {
+        if (j == 0) return S0.shifts;
+        const double t = (double)(S0.step + j) * dtd;
+        long long k = max(S0.shifts, (long long)floor(v * t / a.dx) - 1);
+        while (v * t >= (double)(k + 1) * a.dx) k += 1;
+        return k;
+    };
+    for (int j = tid; j < a.nsteps; j += NT) {
+        const long long k0 = shifts_at(j);
+        nsh[j] = (int)(shifts_at(j + 1) - k0);
+        th0[j] = K.one_m_ke *
+                 (a.theta_ref + a.G_theta * (a.x0 + v * ((double)(S0.step + j) * dtd) - (double)k0 * a.dx));
     }
     __syncthreads();
-    double gM = 0.0, gA = 0.0, gB = 0.0;
-    const T pg = p_of(C, a.gphi);
-    const T Yg = a.gmul + pg * (a.gmus - a.gmul);
-
-    for (int it = a.nsteps - 1; it >= 0; --it) {
-        // the window shifts after this step, undone: lambda moves one cell back
-        for (int k = 0; k < nsh[it]; ++k) {
-            T tf[RJ], tc[RJ], td[RJ];
-#pragma unroll
-            for (int j = 0; j < RJ; ++j) {
-                const int i = tid + j * NT;
-                if (i >= n) break;
-                tf[j] = i > 0 ? sLf[i - 1] : T(0);
-                tc[j] = i > 0 ? sLc[i - 1] : T(0);
-                td[j] = i > 0 ? sLd[i - 1] : T(0);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < RJ; ++j) {
-                const int i = tid + j * NT;
-                if (i >= n) break;
-                sLf[i] = tf[j];
-                sLc[i] = tc[j];
-                sLd[i] = td[j];
-            }
-            __syncthreads();
+    {
+        // lambda after the last step, moved back by the shifts that followed it
+        const int s = nsh[a.nsteps - 1];
+        for (int i = tid - J; i < room - J; i += NT) {
+            const int g = lo + i, j = g - s;
+            const bool in = j >= 0 && g < n;
+            const T f = in ? a.lphi[off + j] : T(0), c = in ? a.lc[off + j] : T(0), d = in ? a.ld[off + j] : T(0);
+            sm[i] = f;
+            sm[room + i] = c;
+            sm[2 * room + i] = d;
+            sm[3 * room + i] = sm[4 * room + i] = sm[5 * room + i] = T(0);
         }
-        // the step's state and intermediates, as the forward run recorded them
+    }
+    auto sync = [&]() {
+        if (csize > 1) cluster.sync();
+        else __syncthreads();
+    };
+    sync();
+    RunningSum<V> gM, gA, gB;
+    gM.hi = gM.lo = gA.hi = gA.lo = gB.hi = gB.lo = vlit<V>(0.0);
+    // the recorded values of a lane's two cells: phi, c_s, c_l, mu_s, mu_l, rate
+    struct Cells {
+        T a[12];
+    };
+    auto fetch = [&](int it, int u) {
+        Cells w;
+        const int i0 = lo + u + (lane - 1) * J;
         const T* r = a.rec + 6 * a.rec_steps * off + (long long)it * 6 * n;
-        T dval[RJ], pval[RJ];
 #pragma unroll
-        for (int j = 0; j < RJ; ++j) {
-            const int i = tid + j * NT;
-            if (i >= n) break;
-            const T f = r[i], c = r[n + i], d = r[2 * n + i];
-            const T p = p_of(C, f);
-            sF[i] = f;
-            sCs[i] = c + (T(1) - p) * d;
-            sCl[i] = c - p * d;
-            sMs[i] = r[3 * n + i];
-            sMl[i] = r[4 * n + i];
-            sPd[i] = r[5 * n + i];
-            dval[j] = d;
-            pval[j] = p;
+        for (int k = 0; k < 2; ++k) {
+            const int i = i0 + k;
+            const bool in = i >= 0 && i < n;
+            w.a[k] = in ? r[i] : R.gphi;
+            w.a[2 + k] = in ? r[n + i] : R.gcs;
+            w.a[4 + k] = in ? r[2 * n + i] : R.gcl;
+            w.a[6 + k] = in ? r[3 * n + i] : R.gmus;
+            w.a[8 + k] = in ? r[4 * n + i] : R.gmul;
+            w.a[10 + k] = in ? r[5 * n + i] : T(0);
         }
-        __syncthreads();
-        const T theta0 = T(th0[it]);
-        // R1: the two faces of each cell, their parts that act on the cell
-        T aF[RJ], aCs[RJ], aCl[RJ], aMs[RJ], aMl[RJ], aP[RJ], aPd[RJ];
-#pragma unroll
-        for (int j = 0; j < RJ; ++j) {
-            const int i = tid + j * NT;
-            if (i >= n) break;
-            const T f0 = sF[i], cs0 = sCs[i], cl0 = sCl[i], ms0 = sMs[i], ml0 = sMl[i], pd0 = sPd[i];
-            const T p0 = pval[j];
-            const T Y0 = ml0 + p0 * (ms0 - ml0);
-            T lf = T(0), lcs = T(0), lcl = T(0), lms = T(0), lml = T(0), lY = T(0);
-            T lpd = dt * sLf[i];
-            FaceAdj<T> o;
-            if (i > 0) {   // face (i-1, i): this cell is its right side
-                const T fL = sF[i - 1], csL = sCs[i - 1], clL = sCl[i - 1], msL = sMs[i - 1], mlL = sMl[i - 1];
-                const T pL = p_of(C, fL);
-                const T YL = mlL + pL * (msL - mlL);
-                const T gc = dtdx * (sLc[i - 1] - sLc[i]), gd = dtdx * (sLd[i - 1] - sLd[i]);
-                face1_rev(C, fL, f0, csL, cs0, clL, cl0, sPd[i - 1], pd0, (f0 - fL) * C.inv_dx,
-                          (Y0 - YL) * C.inv_dx, (ms0 - msL) * C.inv_dx, (ml0 - mlL) * C.inv_dx, gc, gd, o);
-                lf += o.f + o.nphi * C.inv_dx;
-                lcs += o.cs;
-                lcl += o.cl;
-                lpd += o.pd;
-                lY += o.nY * C.inv_dx;
-                lms += o.nS * C.inv_dx;
-                lml += o.nL * C.inv_dx;
-            }
-            {              // face (i, i+1), or (n-1, ghost): this cell is its left side
-                const bool last = i == n - 1;
-                const T fR = last ? a.gphi : sF[i + 1];
-                const T csR = last ? a.gcs : sCs[i + 1], clR = last ? a.gcl : sCl[i + 1];
-                const T msR = last ? a.gmus : sMs[i + 1], mlR = last ? a.gmul : sMl[i + 1];
-                const T YR = last ? Yg : mlR + p_of(C, fR) * (msR - mlR);
-                const T pdR = last ? T(0) : sPd[i + 1];
-                const T gc = dtdx * (sLc[i] - (last ? T(0) : sLc[i + 1]));
-                const T gd = dtdx * (sLd[i] - (last ? T(0) : sLd[i + 1]));
-                face1_rev(C, f0, fR, cs0, csR, cl0, clR, pd0, pdR, (fR - f0) * C.inv_dx,
-                          (YR - Y0) * C.inv_dx, (msR - ms0) * C.inv_dx, (mlR - ml0) * C.inv_dx, gc, gd, o);
-                lf += o.f - o.nphi * C.inv_dx;
-                lcs += o.cs;
-                lcl += o.cl;
-                lpd += o.pd;
-                lY -= o.nY * C.inv_dx;
-                lms -= o.nS * C.inv_dx;
-                lml -= o.nL * C.inv_dx;
-                gA += (double)o.A;   // each face's parameter terms counted once, by its left cell
-                gB += (double)o.b;
-            }
+        return w;
+    };
+    Cells next = {};
+    if (warp * USE < mine) next = fetch(a.nsteps - 1, warp * USE);
+    int cur = 0;
+    for (int it = a.nsteps - 1; it >= 0; --it) {
+        const int nxt = 3 * room - cur;
+        const int s = it > 0 ? nsh[it - 1] : 0;     // shifts before this step: into the earlier frame
+        for (int u = warp * USE; u < mine; u += warps * USE) {
+            const int w0 = u + (lane - 1) * J, i0 = lo + w0;
+            const Cells w = u == warp * USE ? next : fetch(it, u);
+            auto pair = [](T x, T y) { return x_pair(x, y); };
+            const V f = pair(w.a[0], w.a[1]), cs = pair(w.a[2], w.a[3]), cl = pair(w.a[4], w.a[5]);
+            const V mus = pair(w.a[6], w.a[7]), mul = pair(w.a[8], w.a[9]), pd = pair(w.a[10], w.a[11]);
+            const T* q = sm + cur + w0;
+            const V lf = pair(q[0], q[1]), lc = pair(q[room], q[room + 1]), ld = pair(q[2 * room], q[2 * room + 1]);
+            if (u == warp * USE && it > 0) next = fetch(it - 1, u);
+            auto left_of = [&](V x) { return x_pair(from_below(x.y), x.x); };
+            auto right_of = [&](V x) { return x_pair(x.y, from_above(x.x)); };
+            const V p = line_p<STD>(K, f), omp = vsub(vlit<V>(1.0), p);
+            const V dmu = vsub(mus, mul), Y = vfma(p, dmu, mul);
+            const V fR = right_of(f), sR = right_of(mus), lR = right_of(mul);
+            // R1: the face to the right, by its left cell
+            const bool real0 = i0 >= 0 && i0 < n, real1 = i0 + 1 >= 0 && i0 + 1 < n;
+            FaceAdj<V> o;
+            line_face_rev<STD>(K, R, f, fR, cs, right_of(cs), cl, right_of(cl), pd, right_of(pd),
+                               vsub(right_of(Y), Y), vsub(sR, mus), vsub(lR, mul), vmul(dtq, vsub(lc, right_of(lc))),
+                               vmul(dtq, vsub(ld, right_of(ld))), o);
+            auto keep = [&](V x) { return vmask(x, !real0, !real1); };   // no face left of the line or beyond its ghost
+            o.f = keep(o.f); o.cs = keep(o.cs); o.cl = keep(o.cl); o.pd = keep(o.pd);
+            o.nphi = keep(o.nphi); o.nY = keep(o.nY); o.nS = keep(o.nS); o.nL = keep(o.nL);
+            const bool useful = lane != 0 && lane != 31;
+            // this cell as the face's left side, and as the right side of its left face
+            V af = vadd(vsub(o.f, o.nphi), left_of(vadd(o.f, o.nphi)));
+            V acs = vadd(o.cs, left_of(o.cs)), acl = vadd(o.cl, left_of(o.cl));
+            const V lpd = vfma(dtq, lf, vadd(o.pd, left_of(o.pd)));
+            const V lY = vsub(left_of(o.nY), o.nY);
             // Y = mu_l + p (mu_s - mu_l)
-            lms += lY * p0;
-            lml += lY * (T(1) - p0);
-            aP[j] = lY * (ms0 - ml0);
-            aF[j] = lf;
-            aCs[j] = lcs;
-            aCl[j] = lcl;
-            aMs[j] = lms;
-            aMl[j] = lml;
-            aPd[j] = lpd;
-        }
-        // R2: the phase-field rate of each cell, backwards
+            V ams = vfma(lY, p, vsub(left_of(o.nS), o.nS)), aml = vfma(lY, omp, vsub(left_of(o.nL), o.nL));
+            V ap = vmul(lY, dmu);
+            // R2: the rate, backwards (cold end: mirror ghost; hot end: Dirichlet)
+            V fL = left_of(f), sL = left_of(mus), lL = left_of(mul);
+            if (i0 == 0) { fL.x = f.x; sL.x = mus.x; lL.x = mul.x; }
+            if (i0 == -1) { fL.y = f.y; sL.y = mus.y; lL.y = mul.y; }
+            V xc;
+            xc.x = T(i0) + T(0.5);
+            xc.y = T(i0 + 1) + T(0.5);
+            V th;
+            th.x = th.y = T(th0[it]);
+            RateAdj<V> z;
+            line_rate_rev<STD>(K, R, f, fL, fR, sL, sR, lL, lR, cs, cl, mus, mul, p, pd, vfma(K.ke_G, xc, th), lpd, z);
+            auto only = [&](V x) { return vmask(x, !real0, !real1); };
+            z.lap = only(z.lap); z.gp = only(z.gp); z.gs = only(z.gs); z.gl = only(z.gl);
+            if (useful) {
+                gM.add(only(z.iMphi));
+                gA.add(vadd(only(z.A), keep(o.A)));
+                gB.add(vadd(only(z.b), keep(o.b)));
+            }
+            // R3: the own rate's stencil centre and its neighbours' stencils
+            af = vadd(af, vfma(z.lap, vlit<V>(-2.0), z.f));
+            ams = vadd(ams, z.mus);
+            aml = vadd(aml, z.mul);
+            ap = vadd(ap, z.p);
+            acs = vadd(acs, z.cs);
+            acl = vadd(acl, z.cl);
+            const V up = vadd(z.lap, z.gp), dn = vsub(z.lap, z.gp);   // to the east and to the west neighbour
+            V fromL = left_of(up), sfromL = left_of(z.gs), lfromL = left_of(z.gl);
+            V fromR = right_of(dn), sfromR = right_of(z.gs), lfromR = right_of(z.gl);
+            // the mirrored cold end: the first cell is its own west neighbour
+            if (i0 == 0) { fromL.x = dn.x; sfromL.x = -z.gs.x; lfromL.x = -z.gl.x; }
+            if (i0 == -1) { fromL.y = dn.y; sfromL.y = -z.gs.y; lfromL.y = -z.gl.y; }
+            af = vadd(af, vadd(fromL, fromR));
+            ams = vadd(ams, vsub(sfromL, sfromR));
+            aml = vadd(aml, vsub(lfromL, lfromR));
+            // the pointwise values
+            acs = vfma(ams, vrcp_n(cs), acs);
+            acl = vfma(aml, vrcp_n(cl), acl);
+            const V asum = vadd(acs, acl);
+            ap = vsub(ap, vmul(vsub(cs, cl), asum));
+            const V nf = only(vadd(lf, vfma(ap, line_dp<STD>(K, f), af)));
+            const V nc = only(vadd(lc, asum));
+            const V nd = only(vadd(ld, vsub(vmul(acs, omp), vmul(acl, p))));
+            const T out[6] = {nf.x, nf.y, nc.x, nc.y, nd.x, nd.y};
+            auto put = [&](T* t, int k) {
+                t[0] = out[k];
+                t[room] = out[2 + k];
+                t[2 * room] = out[4 + k];
+            };
+            if (useful || (s > 0 && i0 < 0)) {
 #pragma unroll
-        for (int j = 0; j < RJ; ++j) {
-            const int i = tid + j * NT;
-            if (i >= n) break;
-            const int im = (i == 0) ? 0 : i - 1;
-            const bool last = i == n - 1;
-            const T fc = sF[i], fW = sF[im], fE = last ? a.gphi : sF[i + 1];
-            const T mWs = sMs[im], mWl = sMl[im];
-            const T mEs = last ? a.gmus : sMs[i + 1], mEl = last ? a.gmul : sMl[i + 1];
-            const T p = pval[j], cs = sCs[i], cl = sCl[i], mus = sMs[i], mul = sMl[i];
-            const T dp = dp_of(C, fc);
-            const T lap = (fW - T(2) * fc + fE) * C.inv_dx2;
-            const T gp = (fE - fW) * C.inv_2dx;
-            const T gs = (mEs - mWs) * C.inv_2dx;
-            const T gl = (mEl - mWl) * C.inv_2dx;
-            const T Ms = Ms_of(C, cs), Ml = Ml_of(C, cl);
-            const T bMl = C.b * Ml;
-            const T omp = T(1) - p;
-            const T Msq = Ms * omp;
-            const T iM = T(1) / (Msq + bMl * p);
-            const T d = cs - cl;
-            const T rr = T(1) / (gp * gp + C.delta2);
-            const T pq = p * omp;
-            const T u = C.b * p + omp;
-            const T oA = C.one_m_A;
-            const T K2 = oA * oA * d * d * C.b * pq * rr * iM / u;
-            const T Kc = C.inv_Mphi + K2;
-            const T theta = theta0 - C.G_theta * ((T(i) + T(0.5)) * C.dx);
-            const T dmu = mus - mul;
-            const T Nv = Msq * (T(1) - C.A * omp) + C.A * bMl * p * p;
-            const T Dd = Nv * iM;
-            const T dG = cs * dmu - d - C.one_m_ke * theta - Dd * d * dmu;
-            const T W = Ms * gs - bMl * gl;
-            const T Xv = W * gp * rr;
-            const T pd = sPd[i];
-            const T lpd = aPd[j];
-            const T lR = lpd / Kc;
-            const T lKc = -lpd * pd / Kc;
-            const T llap = lR * C.sigma;
-            const T ldfdw = -lR * C.H;
-            const T ldG = -lR * dp;
-            const T ldp = -lR * dG;
-            // Z = (1-A) d pq iM X
-            T loA = lR * d * pq * iM * Xv;
-            T ld = lR * oA * pq * iM * Xv;
-            T lpq = lR * oA * d * iM * Xv;
-            T liM = lR * oA * d * pq * Xv;
-            const T lX = lR * oA * d * pq * iM;
-            const T lW = lX * gp * rr;
-            T lgp = lX * W * rr;
-            T lrr = lX * W * gp;
-            T lMs = lW * gs;
-            const T lgs = lW * Ms;
-            T lbMl = -lW * gl;
-            const T lgl = -lW * bMl;
-            // Kc = 1/M_phi + (1-A)^2 d^2 b pq rr iM / u
-            gM += (double)lKc;
-            loA += lKc * T(2) * oA * d * d * C.b * pq * rr * iM / u;
-            ld += lKc * oA * oA * T(2) * d * C.b * pq * rr * iM / u;
-            T lb = lKc * oA * oA * d * d * pq * rr * iM / u;
-            lpq += lKc * oA * oA * d * d * C.b * rr * iM / u;
-            lrr += lKc * oA * oA * d * d * C.b * pq * iM / u;
-            liM += lKc * oA * oA * d * d * C.b * pq * rr / u;
-            const T lu = -lKc * K2 / u;
-            T lp = lu * (C.b - T(1));
-            lb += lu * p;
-            // dG = cs dmu - d - (1-k_e) theta - Dd d dmu
-            T lcs = ldG * dmu;
-            const T ldmu = ldG * (cs - Dd * d);
-            ld += -ldG * (T(1) + Dd * dmu);
-            const T lDd = -ldG * d * dmu;
-            // Dd = Nv iM
-            const T lN = lDd * iM;
-            liM += lDd * Nv;
-            T lMsq = lN * (T(1) - C.A * omp);
-            gA += (double)(lN * (-Msq * omp + bMl * p * p));
-            lp += lN * (Msq * C.A + T(2) * C.A * bMl * p);
-            lbMl += lN * C.A * p * p;
-            // dmu, pq, rr, iM, Msq, bMl, Ms, Ml, d
-            const T lmus = ldmu, lmul = -ldmu;
-            lp += lpq * (T(1) - T(2) * p);
-            lgp += lrr * (-rr * rr) * (T(2) * gp);
-            const T lden = -liM * iM * iM;
-            lMsq += lden;
-            lbMl += lden * p;
-            lp += lden * bMl;
-            lMs += lMsq * omp;
-            lp -= lMsq * Ms;
-            T lMl = lbMl * C.b;
-            lb += lbMl * Ml;
-            lcs += lMs * C.Ms_c + ld;
-            T lcl = lMl * C.Ml_c - ld;
-            gA -= (double)loA;   // one_m_A = 1 - A
-            gB += (double)lb;
-            // phi of the cell itself: f_dw', p', the Laplacian's centre (and its own
-            // west neighbour at the mirrored cold end)
-            T lf = ldfdw * T(2) * (T(1) - T(6) * fc + T(6) * fc * fc) + ldp * d2p_of(C, fc)
-                   - T(2) * llap * C.inv_dx2;
-            T lms_self = lmus, lml_self = lmul;
-            if (i == 0) {
-                lf += llap * C.inv_dx2 - lgp * C.inv_2dx;
-                lms_self -= lgs * C.inv_2dx;
-                lml_self -= lgl * C.inv_2dx;
+                for (int k = 0; k < 2; ++k) {
+                    const int i = i0 + k + s;       // its place in the earlier frame
+                    if (i < 0 || i >= n) continue;
+                    const int r = i < lo + seg ? rank : rank + 1;
+                    const int l = i - r * seg;
+                    T* const t = sm + nxt + l;
+                    put(r == rank ? t : cluster.map_shared_rank(t, r), k);
+                    if (csize > 1) {
+                        if (l < J && r > 0)
+                            put(r - 1 == rank ? t + seg : cluster.map_shared_rank(t + seg, r - 1), k);
+                        if (l >= seg - J && r < csize - 1)
+                            put(r + 1 == rank ? t - seg : cluster.map_shared_rank(t - seg, r + 1), k);
+                    }
+                }
             }
-            aF[j] += lf;
-            aCs[j] += lcs;
-            aCl[j] += lcl;
-            aMs[j] += lms_self;
-            aMl[j] += lml_self;
-            aP[j] += lp;
-            sXl[i] = llap;
-            sXg[i] = lgp;
-            sXs[i] = lgs;
-            sXm[i] = lgl;
         }
-        __syncthreads();
-        // R3: the neighbours' rates, then the pointwise values, into the adjoint
-        // of the pre-step state (in place: R3 reads only its own cells' lambda)
+        cur = nxt;
+        sync();
+    }
+    for (int i = tid; i < min(mine, n - lo); i += NT) {
+        a.lphi[off + lo + i] = sm[cur + i];
+        a.lc[off + lo + i] = sm[cur + room + i];
+        a.ld[off + lo + i] = sm[cur + 2 * room + i];
+    }
+    // parameter derivatives: sums over the lanes, the warps and the CTAs in fixed order
+    double vals[3] = {gM.total(), gA.total(), gB.total()};
 #pragma unroll
-        for (int j = 0; j < RJ; ++j) {
-            const int i = tid + j * NT;
-            if (i >= n) break;
-            T lf = aF[j], lms = aMs[j], lml = aMl[j];
-            if (i > 0) {        // this cell is the east neighbour of cell i-1
-                lf += sXl[i - 1] * C.inv_dx2 + sXg[i - 1] * C.inv_2dx;
-                lms += sXs[i - 1] * C.inv_2dx;
-                lml += sXm[i - 1] * C.inv_2dx;
-            }
-            if (i < n - 1) {    // and the west neighbour of cell i+1
-                lf += sXl[i + 1] * C.inv_dx2 - sXg[i + 1] * C.inv_2dx;
-                lms -= sXs[i + 1] * C.inv_2dx;
-                lml -= sXm[i + 1] * C.inv_2dx;
-            }
-            const T cs = sCs[i], cl = sCl[i];
-            const T lcs = aCs[j] + lms / cs;
-            const T lcl = aCl[j] + lml / cl;
-            const T p = pval[j];
-            const T lp = aP[j] - dval[j] * (lcs + lcl);
-            sLf[i] = sLf[i] + lf + lp * dp_of(C, sF[i]);
-            sLc[i] = sLc[i] + lcs + lcl;
-            sLd[i] = sLd[i] + lcs * (T(1) - p) - lcl * p;
-        }
-        __syncthreads();
-    }
-    for (int i = tid; i < n; i += NT) {
-        a.lphi[off + i] = sLf[i];
-        a.lc[off + i] = sLc[i];
-        a.ld[off + i] = sLd[i];
-    }
-    // parameter derivatives: block sums, one writer per instance
-    double vals[3] = {gM, gA, gB};
     for (int q = 0; q < 3; ++q) {
-        double x = vals[q];
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if ((tid & 31) == 0) red[tid >> 5] = x;
-        __syncthreads();
-        if (tid == 0) {
-            double tot = 0.0;
-            for (int w = 0; w < NT / 32; ++w) tot += red[w];
-            a.grad[3 * inst + q] += tot;
-        }
-        __syncthreads();
+        for (int o = 16; o > 0; o >>= 1) vals[q] += __shfl_xor_sync(0xffffffffu, vals[q], o);
+        if (lane == 0) red[warp][q] = vals[q];
+    }
+    __syncthreads();
+    if (tid < 3) {
+        double tot = 0.0;
+        for (int w = 0; w < warps; ++w) tot += red[w][tid];
+        if (csize > 1) *cluster.map_shared_rank(&cred[rank][tid], 0) = tot;
+        else cred[0][tid] = tot;
+    }
+    sync();
+    if (rank == 0 && tid < 3) {
+        double tot = 0.0;
+        for (int r = 0; r < csize; ++r) tot += cred[r][tid];
+        a.grad[3 * inst + tid] += tot;
     }
 }
 
 // per instance: max_x c and the lowest maximising index
 template <typename V>
-__global__ void __launch_bounds__(256) value_cmax(const V* __restrict__ c, const BatchState* __restrict__ st,
-                                                  double* __restrict__ cmax, int* __restrict__ imax) {
+__global__ void __launch_bounds__(256) value_cmax(const V* __restrict__ c, const V* __restrict__ clo,
+                                                  const BatchState* __restrict__ st, double* __restrict__ cmax,
+                                                  int* __restrict__ imax) {
     const BatchState S = st[blockIdx.x];
     double best = -INFINITY;
     int bi = 0x7fffffff;
     for (int i = threadIdx.x; i < S.n; i += blockDim.x) {
-        const double x = (double)c[S.off + i];
+        const double x = (double)c[S.off + i] + (clo != nullptr ? (double)clo[S.off + i] : 0.0);
         if (x > best || (x == best && i < bi)) {
             best = x;
             bi = i;
@@ -1710,34 +1854,32 @@ __global__ void seed_lambda(V* __restrict__ lc, const BatchState* __restrict__ s
     if (i < N && imax[i] >= 0 && imax[i] < st[i].n) lc[st[i].off + imax[i]] = V(-cinf / (cmax[i] * cmax[i]));
 }
 
-// 512 threads per instance, RJ cells each: the smallest RJ that covers the
-// longest instance (registers hold RJ cells' partial adjoints)
+// the reverse sweep's kernel limits, per device
 template <typename V>
-using RevFn = void (*)(RevArgs<V>);
-template <typename V>
-static RevFn<V> reverse_for(int64_t nmax) {
-    if (nmax <= 1024) return reverse_kernel<V, 512, 2>;
-    if (nmax <= 2048) return reverse_kernel<V, 512, 4>;
-    return reverse_kernel<V, 512, 8>;
-}
-
-// the step's parameters in the arithmetic type, as the reverse sweep uses them
-template <typename V>
-static Consts<V> value_consts_T(const pf_batch_desc& D) {
-    const pf_params& P = D.params;
-    Consts<V> C = {};
-    C.dim = 1; C.interp = P.interp; C.lap = 3; C.mobility = P.mobility_mode;
-    C.dx = V(D.dx); C.inv_dx = V(1.0 / D.dx); C.inv_2dx = V(0.5 / D.dx); C.inv_dx2 = V(1.0 / (D.dx * D.dx));
-    C.H = V(P.H); C.sigma = V(P.sigma); C.inv_Mphi = V(1.0 / P.M_phi); C.D_s = V(P.D_s); C.D_l = V(P.D_l);
-    C.log_ke = V(std::log(P.k_e)); C.one_m_ke = V(1.0 - P.k_e); C.A = V(P.A); C.one_m_A = V(1.0 - P.A);
-    C.b = V(P.b); C.a = V(P.a); C.delta2 = V(P.delta * P.delta); C.G_theta = V(P.G_theta);
-    set_coefficients(C);
-    return C;
+static cudaError_t reverse_setup(size_t* max_dynamic) {
+    static DeviceSetup setup;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= DeviceSetup::MAX_DEVICES) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lock(setup.mu);
+    if (!setup.done[dev]) {
+        int optin = 0;
+        cudaFuncAttributes fa = {};
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess) e = raise_smem(reverse_kernel<V, true>, optin);
+        if (e == cudaSuccess) e = raise_smem(reverse_kernel<V, false>, optin);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, reverse_kernel<V, true>);
+        setup.err[dev] = e;
+        setup.value[dev] = (size_t)optin - fa.sharedSizeBytes;
+        setup.done[dev] = true;
+    }
+    *max_dynamic = setup.value[dev];
+    return setup.err[dev];
 }
 
 template <typename V>
 static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStream_t main, std::string& err) {
-    constexpr int NT = 512;
     pf_batch_desc D = A.batch;
     D.check_every = 0;   // a fixed number of steps
     D.energy_every = 0;
@@ -1757,28 +1899,28 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
          (int64_t)RMAX_SEG, A.nsteps});
     const int64_t nseg = (A.nsteps + seg - 1) / seg;
     const size_t fb = (size_t)B.total * sizeof(V);
-    V *scs = nullptr, *scl = nullptr, *ckp = nullptr, *ckc = nullptr, *ckd = nullptr, *rec = nullptr;
-    V *lphi = nullptr, *lc = nullptr, *ld = nullptr;
-    BatchState* ckst = nullptr;
+    // States before every segment (each segment's run reads its own and writes the
+    // next), the final state, and one for the re-runs' results, which nothing
+    // reads: slots 0 .. nseg + 1 of every array.
+    const size_t slots = (size_t)nseg + 2;
+    B.deriv = true;
+    V *scs = nullptr, *scl = nullptr, *rec = nullptr, *lphi = nullptr, *lc = nullptr, *ld = nullptr;
     double *grad = nullptr, *cmax = nullptr;
     int* imax = nullptr;
     auto free_tmp = [&] {
-        void* ptrs[] = {scs, scl, ckp, ckc, ckd, rec, lphi, lc, ld, ckst, grad, cmax, imax};
+        void* ptrs[] = {scs, scl, rec, lphi, lc, ld, grad, cmax, imax};
         for (void* p : ptrs)
             if (p) cudaFree(p);
     };
-    cudaError_t e = cudaMalloc(&B.phi, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.c, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.d, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.st, N * sizeof(BatchState));
+    cudaError_t e = cudaMalloc(&B.phi, fb * slots);
+    if (e == cudaSuccess) e = cudaMalloc(&B.c, fb * slots);
+    if (e == cudaSuccess) e = cudaMalloc(&B.d, fb * slots);
+    if (e == cudaSuccess && sizeof(V) == 4) e = cudaMalloc(&B.low, 3 * fb * slots);
+    if (e == cudaSuccess) e = cudaMalloc(&B.st, N * slots * sizeof(BatchState));
     if (e == cudaSuccess) e = cudaMalloc(&B.dv, N * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&B.ddt, N * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&scs, fb);
     if (e == cudaSuccess) e = cudaMalloc(&scl, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&ckp, fb * nseg);
-    if (e == cudaSuccess) e = cudaMalloc(&ckc, fb * nseg);
-    if (e == cudaSuccess) e = cudaMalloc(&ckd, fb * nseg);
-    if (e == cudaSuccess) e = cudaMalloc(&ckst, (size_t)N * nseg * sizeof(BatchState));
     if (e == cudaSuccess) e = cudaMalloc(&rec, fb * 6 * seg * 2);
     if (e == cudaSuccess) e = cudaMalloc(&lphi, fb);
     if (e == cudaSuccess) e = cudaMalloc(&lc, fb);
@@ -1805,61 +1947,47 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
     if (e == cudaSuccess) e = cudaMemsetAsync(ld, 0, fb, main);
     if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, 3 * N * sizeof(double), main);
     if (e == cudaSuccess) {
-        batch_to_state<V><<<1216, 256, 0, main>>>(scs, scl, B.phi, B.c, B.d, B.total, D.params.interp, D.params.a);
+        batch_to_state<V><<<1216, 256, 0, main>>>(scs, scl, B.phi, B.c, B.d, B.total, D.params.interp, D.params.a,
+                                                  B.low);
         e = cudaGetLastError();
     }
-    size_t max_dyn = 0;
-    if (e == cudaSuccess) e = set_smem_limits<V>(&max_dyn, &B.sms);
-    const size_t rsmem = (size_t)13 * nmax * sizeof(V);
-    if (e == cudaSuccess) {
-        static DeviceSetup setup;
-        int dev = 0;
-        e = cudaGetDevice(&dev);
-        if (e == cudaSuccess && (dev < 0 || dev >= DeviceSetup::MAX_DEVICES)) e = cudaErrorInvalidDevice;
-        if (e == cudaSuccess) {
-            std::lock_guard<std::mutex> lock(setup.mu);
-            if (!setup.done[dev]) {
-                int optin = 0;
-                setup.err[dev] = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-                for (int64_t m : {int64_t(1024), int64_t(2048), int64_t(4096)})
-                    if (setup.err[dev] == cudaSuccess) setup.err[dev] = raise_smem(reverse_for<V>(m), optin);
-                cudaFuncAttributes fa;
-                if (setup.err[dev] == cudaSuccess) setup.err[dev] = cudaFuncGetAttributes(&fa, reverse_for<V>(4096));
-                setup.value[dev] = setup.err[dev] == cudaSuccess ? (size_t)optin - fa.sharedSizeBytes : 0;
-                setup.done[dev] = true;
-            }
-            e = setup.err[dev];
-            if (e == cudaSuccess && rsmem > setup.value[dev]) {
-                free_tmp();
-                err = "longest instance does not fit in shared memory for the reverse sweep";
-                return PF_EINVAL;
-            }
-        }
+    size_t max_rev = 0;
+    if (e == cudaSuccess) e = set_smem_limits<V>(&B.max_dyn, &B.sms);
+    if (e == cudaSuccess) e = reverse_setup<V>(&max_rev);
+    constexpr int RUSE = 60;                       // reverse_kernel's cells per strip that hold results
+    const int64_t rstrips = (nmax + 2 + RUSE - 1) / RUSE;
+    const int rcluster = cluster_for(rstrips, N, B.sms);
+    const int64_t rper = (rstrips + rcluster - 1) / rcluster;
+    const int rroom = (int)(rper * RUSE + 4);
+    const size_t rsmem = (size_t)6 * rroom * sizeof(V);
+    if (e == cudaSuccess && rsmem > max_rev) {
+        free_tmp();
+        err = "longest instance does not fit in shared memory for the reverse sweep";
+        return PF_EINVAL;
     }
-    if (e == cudaSuccess && (size_t)6 * (nmax + 34 * batch_jmax<V>()) * sizeof(V) > max_dyn) {
+    if (e == cudaSuccess && (size_t)6 * (nmax + 34 * batch_jmax<V>()) * sizeof(V) > B.max_dyn) {
         free_tmp();
         err = "longest instance does not fit in shared memory";
         return PF_EINVAL;
     }
-    const int cpt = D.cells_per_thread > 0 ? D.cells_per_thread : 8;
+    const int cpt = D.cells_per_thread > 0 ? D.cells_per_thread : 2;
     if (e == cudaSuccess) e = B.make_groups(cpt);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&B.fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreate(&B.t0);
     if (e == cudaSuccess) e = cudaEventCreate(&B.t1);
     if (e == cudaSuccess) e = cudaEventRecord(B.t0, main);
-    // forward: the state (and clock) before every segment, then the segment
+    // forward: segment s from slot s into slot s + 1
     for (int64_t s = 0; s < nseg && e == cudaSuccess; ++s) {
         const int64_t len = std::min(seg, A.nsteps - s * seg);
-        e = cudaMemcpyAsync(ckp + s * B.total, B.phi, fb, cudaMemcpyDeviceToDevice, main);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(ckc + s * B.total, B.c, fb, cudaMemcpyDeviceToDevice, main);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(ckd + s * B.total, B.d, fb, cudaMemcpyDeviceToDevice, main);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(ckst + s * N, B.st, N * sizeof(BatchState), cudaMemcpyDeviceToDevice, main);
-        if (e == cudaSuccess) e = B.issue((int)len);
+        B.slot_in = s;
+        B.slot_out = s + 1;
+        e = B.issue((int)len);
     }
     if (e == cudaSuccess) {
-        value_cmax<V><<<N, 256, 0, main>>>(B.c, B.st, cmax, imax);
-        seed_lambda<V><<<(N + 255) / 256, 256, 0, main>>>(lc, B.st, cmax, imax, D.params.c_inf, N);
+        const V* cf = B.c + nseg * B.total;
+        const BatchState* sf = B.st + nseg * N;
+        value_cmax<V><<<N, 256, 0, main>>>(cf, B.low ? B.low + (3 * nseg + 1) * B.total : nullptr, sf, cmax, imax);
+        seed_lambda<V><<<(N + 255) / 256, 256, 0, main>>>(lc, sf, cmax, imax, D.params.c_inf, N);
         e = cudaGetLastError();
     }
     // backwards: re-run each segment recording every step (main stream, the
@@ -1880,45 +2008,45 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
         const int64_t len = std::min(seg, A.nsteps - s * seg);
         cudaError_t x = cudaSuccess;
         if (s + 2 < nseg) x = cudaStreamWaitEvent(main, erev[b], 0);   // the sweep of s+2 read this buffer
-        if (x == cudaSuccess) x = cudaMemcpyAsync(B.phi, ckp + s * B.total, fb, cudaMemcpyDeviceToDevice, main);
-        if (x == cudaSuccess) x = cudaMemcpyAsync(B.c, ckc + s * B.total, fb, cudaMemcpyDeviceToDevice, main);
-        if (x == cudaSuccess) x = cudaMemcpyAsync(B.d, ckd + s * B.total, fb, cudaMemcpyDeviceToDevice, main);
-        if (x == cudaSuccess)
-            x = cudaMemcpyAsync(B.st, ckst + s * N, N * sizeof(BatchState), cudaMemcpyDeviceToDevice, main);
+        B.slot_in = s;
+        B.slot_out = nseg + 1;
         B.rec = rec + b * rec_elems;
         if (x == cudaSuccess) x = B.issue((int)len);
         if (x == cudaSuccess) x = cudaEventRecord(erec[b], main);
         return x;
     };
+    RevArgs<V> ra = {};
+    {
+        const HostProblem P = B.problem();
+        auto v2 = [](double x) {
+            typename LineNum<V>::V r;
+            r.x = r.y = V(x);
+            return r;
+        };
+        const double dx2 = P.dx * P.dx;
+        ra.K = make_line_consts<V>(P, -1);
+        ra.R.A = v2(P.A); ra.R.oA = v2(1.0 - P.A); ra.R.b = v2(P.b); ra.R.bm1 = v2(P.b - 1.0);
+        ra.R.c4 = v2(4.0 * dx2); ra.R.dx2 = v2(dx2); ra.R.H = v2(P.H); ra.R.inv_Mphi = v2(1.0 / P.M_phi);
+        ra.R.gphi = ra.K.gphi; ra.R.gcs = V(P.dir_cs); ra.R.gcl = V(P.dir_cl);
+        ra.R.gmus = V(std::log(P.dir_cs) - std::log(P.k_e));
+        ra.R.gmul = V(std::log(P.dir_cl));
+        ra.rec_steps = seg;
+        ra.lphi = lphi; ra.lc = lc; ra.ld = ld; ra.grad = grad; ra.v = B.dv; ra.dt = B.ddt;
+        ra.cluster = rcluster; ra.room = rroom;
+        ra.theta_ref = P.theta_ref; ra.G_theta = P.G_theta; ra.x0 = P.x0;
+        ra.dx = (double)V(P.dx);
+        ra.inv_dx2 = 1.0 / dx2;
+    }
     if (e == cudaSuccess) e = rerun(nseg - 1);
     for (int64_t s = nseg - 1; s >= 0 && e == cudaSuccess; --s) {
         const int b = (int)(s & 1);
-        const int64_t len = std::min(seg, A.nsteps - s * seg);
         e = cudaStreamWaitEvent(rs, erec[b], 0);
         if (e == cudaSuccess) {
-            const BatchArgs<V> ba = B.args(B.groups[0], (int)len);
-            RevArgs<V> ra;
             ra.rec = rec + b * rec_elems;
-            ra.rec_steps = seg;
-            ra.lphi = lphi;
-            ra.lc = lc;
-            ra.ld = ld;
-            ra.grad = grad;
-            ra.st0 = ckst + s * N;
-            ra.v = B.dv;
-            ra.dt = B.ddt;
-            ra.nsteps = (int)len;
-            ra.C = value_consts_T<V>(D);
-            ra.theta_ref = ba.theta_ref;
-            ra.G_theta = ba.G_theta;
-            ra.x0 = ba.x0;
-            ra.gphi = V(D.bc.dir_phi);
-            ra.gcs = V(D.bc.dir_cs);
-            ra.gcl = V(D.bc.dir_cl);
-            ra.gmus = V(std::log(D.bc.dir_cs) - std::log(D.params.k_e));
-            ra.gmul = V(std::log(D.bc.dir_cl));
-            reverse_for<V>(nmax)<<<N, NT, rsmem, rs>>>(ra);
-            e = cudaGetLastError();
+            ra.st0 = B.st + s * N;
+            ra.nsteps = (int)std::min(seg, A.nsteps - s * seg);
+            e = launch_clusters(B.std_phys ? reverse_kernel<V, true> : reverse_kernel<V, false>, N, rcluster,
+                                warps_for(rper, rev_warps<V>()), rsmem, rs, ra);
         }
         if (e == cudaSuccess) e = cudaEventRecord(erev[b], rs);
         if (e == cudaSuccess && s > 0) e = rerun(s - 1);

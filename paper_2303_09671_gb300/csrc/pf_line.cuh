@@ -74,6 +74,14 @@ template <typename T>
 PF_D Dual<T> from_below(Dual<T> x) { return make_dual(from_below(x.v), from_below(x.t)); }
 template <typename T>
 PF_D Dual<T> from_above(Dual<T> x) { return make_dual(from_above(x.v), from_above(x.t)); }
+PF_D float2 x_value(float2 a) { return a; }
+PF_D double2 x_value(double2 a) { return a; }
+template <typename V>
+PF_D V x_value(DV<V> a) { return a.v; }
+PF_D void x_set_value(float2& a, float2 v) { a = v; }
+PF_D void x_set_value(double2& a, double2 v) { a = v; }
+template <typename V>
+PF_D void x_set_value(DV<V>& a, V v) { a.v = v; }
 PF_D float value_of(float x) { return x; }
 PF_D double value_of(double x) { return x; }
 template <typename T>
@@ -172,7 +180,7 @@ struct LineConsts {
     X one_m_A_dx2, minus_b, minus_A;
     double one_m_ke;
     // Dirichlet (hot end) ghost and fresh-cell state
-    S gphi, fc, fd;
+    S gphi, fc, fd, gphi_lo, fc_lo, fd_lo;   // and the low words of their FP32 pairs
     int hot_noflux;   // mirror ghost and zero flux at the hot end instead
 };
 
@@ -180,24 +188,43 @@ struct LineConsts {
 // (quintic h, a = 0, M_i = D_i c_i) with parameters in the range where
 // 1/(Mbar |grad phi|^2) stays an FP32 number, so that one reciprocal serves two
 // quotients (line_std below).
-template <bool STD, typename E, typename X>
-PF_D X line_p(const LineConsts<E>& K, X f) {
-    using V = typename LineNum<E>::V;
+template <bool STD, typename E, typename V>
+PF_D V line_dp(const LineConsts<E>& K, V f) {
+    const V g = vmul(f, vsub(vlit<V>(1.0), f));
+    if constexpr (STD) return vmul(vmul(g, g), vlit<V>(30.0));
+    const V dh = vmul(f, vfma(f, vfma(f, vfma(f, K.dh4, K.dh3), K.dh2), K.dh1));
+    // d/dphi [g^2 (phi - 1/2)] = g^2 - 4 g (phi - 1/2)^2
+    const V s = vsub(f, vlit<V>(0.5));
+    return vfma(vmul(g, vsub(g, vmul(vmul(s, s), vlit<V>(4.0)))), K.a_int, dh);
+}
+template <bool STD, typename E, typename V>
+PF_D V line_p(const LineConsts<E>& K, V f) {
     if constexpr (STD)
         return vmul(vmul(f, f), vmul(f, vfma(f, vfma(f, vlit<V>(6.0), vlit<V>(-15.0)), vlit<V>(10.0))));
-    const X h = vmul(vmul(f, f), vfma(f, vfma(f, vfma(f, K.h5, K.h4), K.h3), K.h2));
-    const X g = vmul(f, vsub(vlit<V>(1.0), f));
+    const V h = vmul(vmul(f, f), vfma(f, vfma(f, vfma(f, K.h5, K.h4), K.h3), K.h2));
+    const V g = vmul(f, vsub(vlit<V>(1.0), f));
     return vfma(vmul(vsub(f, vlit<V>(0.5)), K.a_int), vmul(g, g), h);
 }
-template <bool STD, typename E, typename X>
-PF_D X line_dp(const LineConsts<E>& K, X f) {
-    using V = typename LineNum<E>::V;
-    if constexpr (STD) return vmul(f, vmul(f, vfma(f, vfma(f, vlit<V>(30.0), vlit<V>(-60.0)), vlit<V>(30.0))));
-    const X dh = vmul(f, vfma(f, vfma(f, vfma(f, K.dh4, K.dh3), K.dh2), K.dh1));
-    const X g = vmul(f, vsub(vlit<V>(1.0), f));
-    // d/dphi [g^2 (phi - 1/2)] = g^2 - 4 g (phi - 1/2)^2
-    const X s = vsub(f, vlit<V>(0.5));
-    return vfma(vmul(g, vsub(g, vmul(vmul(s, s), vlit<V>(4.0)))), K.a_int, dh);
+// The derivatives along a direction come from p' and p'' themselves: the product
+// rule over the polynomial subtracts terms 3 times f's derivative where p' is 0.
+template <bool STD, typename T, typename V>
+PF_D V line_d2p(const LineConsts<T>& K, V f) {
+    const V g = vmul(f, vsub(vlit<V>(1.0), f));
+    const V s = vfma(f, vlit<V>(-2.0), vlit<V>(1.0));   // 1 - 2 phi
+    if constexpr (STD) return vmul(vmul(g, s), vlit<V>(60.0));
+    const V d2h = vfma(f, vfma(f, vfma(f, vmul(K.dh4, vlit<V>(4.0)), vmul(K.dh3, vlit<V>(3.0))),
+                               vmul(K.dh2, vlit<V>(2.0))), K.dh1);
+    // d^2/dphi^2 [g^2 (phi - 1/2)], with g' = s and phi - 1/2 = -s/2
+    const V w = vsub(vmul(vmul(g, s), vlit<V>(4.0)), vmul(s, vfma(s, s, vmul(g, vlit<V>(-2.0)))));
+    return vfma(K.a_int, w, d2h);
+}
+template <bool STD, typename E, typename V>
+PF_D DV<V> line_p(const LineConsts<E>& K, DV<V> f) {
+    return {line_p<STD>(K, f.v), vmul(line_dp<STD>(K, f.v), f.t)};
+}
+template <bool STD, typename E, typename V>
+PF_D DV<V> line_dp(const LineConsts<E>& K, DV<V> f) {
+    return {line_dp<STD>(K, f.v), vmul(line_d2p<STD>(K, f.v), f.t)};
 }
 
 template <bool STD, typename V, typename X>
@@ -265,7 +292,7 @@ PF_D void line_face(const LineConsts<E>& K, X fL, X fR, X YL, X YR, X sL, X sR, 
     const X cs2 = vadd(csL, csR), cl2 = vadd(clL, clR);
     const X d2 = vsub(cs2, cl2);
     X p;
-    if constexpr (STD)   // p(S/2)
+    if constexpr (STD && !IsDual<E>::value)   // p(S/2)
         p = vmul(vmul(S, S), vmul(S, vfma(S, vfma(S, vlit<V>(6.0 / 32.0), vlit<V>(-15.0 / 16.0)), vlit<V>(10.0 / 8.0))));
     else p = line_p<STD>(K, vmul(S, vlit<V>(0.5)));
     const X omp = vsub(vlit<V>(1.0), p);
@@ -331,10 +358,52 @@ inline LineConsts<E> make_line_consts(const HostProblem& P, int dir) {
     K.one_m_ke = 1.0 - P.k_e;
     const double pg = p_host3(P, P.dir_phi);
     K.gphi = S(P.dir_phi);
-    K.fc = S(pg * P.dir_cs + (1.0 - pg) * P.dir_cl);
-    K.fd = S(P.dir_cs - P.dir_cl);
+    const double fc = pg * P.dir_cs + (1.0 - pg) * P.dir_cl, fd = P.dir_cs - P.dir_cl;
+    K.fc = S(fc); K.fd = S(fd);
+    K.gphi_lo = S(P.dir_phi - (double)K.gphi); K.fc_lo = S(fc - (double)K.fc); K.fd_lo = S(fd - (double)K.fd);
     K.hot_noflux = P.bc_hi[0] == BC_NOFLUX;
     return K;
+}
+
+// The same with a derivative.  The fluxes are smooth in n_phi where their factors
+// are not (n_phi decays by e-folds over a cell or two): with r = 1/G,
+//   F_c = q n_Y w + rd Z + a e afn,  F_d = rd (T_s - T_l) + a e,
+//   w = n_phi^2 r = 1 - rd,  rd = delta^2 dx^2 r,  e = n_phi r,  a = (1-A) d rate,
+// and dw = -d(rd) = 2 e rd dn_phi, de = r (rd - w) dn_phi, so that no large terms
+// cancel (through d(1/G), dk/dM_phi of the FP32 runs lost a further digit).
+template <bool STD, typename E, typename V>
+PF_D void line_face(const LineConsts<E>& K, DV<V> fL, DV<V> fR, DV<V> YL, DV<V> YR, DV<V> sL, DV<V> sR, DV<V> lL,
+                    DV<V> lR, DV<V> csL, DV<V> csR, DV<V> clL, DV<V> clR, DV<V> pdL, DV<V> pdR, DV<V>& Fc,
+                    DV<V>& Fd) {
+    using X = DV<V>;
+    const X n0 = vsub(fR, fL), n1 = vsub(YR, YL), n2 = vsub(sR, sL), n3 = vsub(lR, lL);
+    const X cs2 = vadd(csL, csR), cl2 = vadd(clL, clR);
+    const X p = line_p<STD>(K, vmul(vadd(fL, fR), vlit<V>(0.5)));
+    const X omp = vsub(vlit<V>(1.0), p);
+    const X Ms = line_M<STD>(K.Ms_c_half, K.Ms_0, cs2), Ml = line_M<STD>(K.Ml_c_half, K.Ml_0, cl2);
+    const X bMl = vmul(K.b, Ml);
+    const X M = vfma(bMl, p, vmul(Ms, omp));
+    const V nn = vmul(n0.v, n0.v), G = vadd(nn, K.delta2_dx2);
+    V im, r;
+    if constexpr (STD) {
+        const V t = vrcp_n(vmul(M.v, G));
+        im = vmul(t, G);
+        r = vmul(t, M.v);
+    } else {
+        im = vrcp_n(M.v);
+        r = vrcp_n(G);
+    }
+    const X iM = {im, vsub(vlit<V>(0.0), vmul(M.t, vmul(im, im)))};
+    const V rd = vmul(K.delta2_dx2, r), w = vmul(nn, r), e = vmul(n0.v, r);
+    const V dw = vmul(vmul(vmul(e, rd), vlit<V>(2.0)), n0.t);
+    const X W = {w, dw}, RD = {rd, vsub(vlit<V>(0.0), dw)}, EE = {e, vmul(vmul(r, vsub(rd, w)), n0.t)};
+    const X Ts = vmul(Ms, n2), Tl = vmul(Ml, n3);
+    const X TD = vsub(Ts, Tl);
+    const X ae = vmul(vmul(vmul(K.quarter_one_m_A, vadd(pdL, pdR)), vsub(cs2, cl2)), EE);
+    const X q = vmul(vmul(Ms, Ml), vmul(vfma(K.b, p, omp), iM));
+    const X afn = vmul(vsub(Ms, bMl), vmul(vmul(p, omp), iM));
+    Fc = vfma(vmul(q, n1), W, vfma(RD, vfma(p, TD, Tl), vmul(ae, afn)));
+    Fd = vfma(RD, TD, ae);
 }
 
 template <typename X, typename E>
@@ -342,15 +411,15 @@ PF_D X x_select(X a, E other, bool lo, bool hi) {
     return x_pair(lo ? other : x_lo(a), hi ? other : x_hi(a));
 }
 
-// The strip's state and one step of it.  COMP: c and phi carry the low word of
-// a compensated sum (FP32 single lines).
+// The strip's state and one step of it.  COMP: the values of phi, c and d are
+// unevaluated FP32 pairs (compensated sums).
 template <typename E, int J, bool COMP>
 struct Strip {
     static constexpr int H = J / 2;
     using X = typename LineNum<E>::X;
     using V = typename LineNum<E>::V;
     X phi[H], c[H], d[H];
-    X plo[COMP ? H : 1], clo[COMP ? H : 1];
+    V plo[COMP ? H : 1], clo[COMP ? H : 1], dlo[COMP ? H : 1];
 };
 
 struct NoRecord {
@@ -365,7 +434,7 @@ struct NoRecord {
 // outside the window.  EDGE: the strip reaches an end of the line (a compile-time
 // switch, so that the other strips carry none of its selections).  dtq = dt / dx^2;
 // ke_theta0 = (1 - k_e) theta0 (theta0 as Consts::G_theta describes it).  record(q, phi,
-// c, d, mu_s, mu_l, rate) is called for every pair with its state before the
+// c_s, c_l, mu_s, mu_l, rate) is called for every pair with its state before the
 // step; the rate it is given is in grid units.
 template <bool STD, bool edge, typename E, int J, bool COMP, typename Rec>
 PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n, int m,
@@ -380,8 +449,13 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
     for (int q = 0; q < H; ++q) {
         p[q] = line_p<STD>(K, s.phi[q]);
         const X omp = vsub(vlit<V>(1.0), p[q]);
+        const X mp = vsub(vlit<V>(0.0), p[q]);
         cs[q] = vfma(omp, s.d[q], s.c[q]);
-        cl[q] = vsub(s.c[q], vmul(p[q], s.d[q]));
+        cl[q] = vfma(mp, s.d[q], s.c[q]);
+        if constexpr (COMP) {   // the low words, of the values
+            cs[q] = vadd(cs[q], vfma(x_value(omp), s.dlo[q], s.clo[q]));
+            cl[q] = vadd(cl[q], vfma(x_value(mp), s.dlo[q], s.clo[q]));
+        }
         fine = fine && is_positive(cs[q]) && is_positive(cl[q]);
         mus[q] = ln_normal(cs[q]);
         mul[q] = ln_normal(cl[q]);
@@ -430,7 +504,7 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
         pd[q] = line_rate<STD>(K, s.phi[q], fL, fR, sL, sR, lL, lR, cs[q], cl[q], dmu[q], p[q],
                                vfma(K.ke_G, xc, th0));
         if (edge) pd[q] = x_select(pd[q], E(0), ia >= hot, ib >= hot);
-        if constexpr (Rec::on) record(q, s.phi[q], s.c[q], s.d[q], mus[q], mul[q], pd[q]);
+        if constexpr (Rec::on) record(q, s.phi[q], cs[q], cl[q], mus[q], mul[q], pd[q]);
     }
     const X YB = right_of(Y), csB = right_of(cs), clB = right_of(cl), pdB = right_of(pd);
     X Fc[H], Fd[H];
@@ -460,30 +534,32 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
         const X dFc = vsub(Fc[q], q > 0 ? Fc[q > 0 ? q - 1 : 0] : FcL);
         const X dFd = vsub(Fd[q], q > 0 ? Fd[q > 0 ? q - 1 : 0] : FdL);
         const bool glo = edge && i0 + q >= hot, ghi = edge && i0 + q + H >= hot;
+        auto hold = [&](auto now, auto before) {   // the ghosts' c and d stay
+            return x_pair(glo ? x_lo(before) : x_lo(now), ghi ? x_hi(before) : x_hi(now));
+        };
         if constexpr (COMP) {
-            // compensated (TwoSum) updates of phi = hi + lo and c = hi + lo
-            auto add2 = [&](X& hi, X& lo, X inc) {
-                const X s_ = vadd(hi, inc);
-                const X bv = vsub(s_, hi);
-                const X l = vadd(lo, vadd(vsub(hi, vsub(s_, bv)), vsub(inc, bv)));
-                const X h = vadd(s_, l);
-                lo = vsub(l, vsub(h, s_));
-                hi = h;
+            // compensated (TwoSum) updates of the values phi, c, d = hi + lo; the
+            // derivatives, if any, are added plainly
+            auto add2 = [&](X& x, V& lo, X inc, bool keep) {
+                const V hi = x_value(x), up = x_value(inc);
+                const V s_ = vadd(hi, up);
+                const V bv = vsub(s_, hi);
+                const V l = vadd(lo, vadd(vsub(hi, vsub(s_, bv)), vsub(up, bv)));
+                const V h = vadd(s_, l);
+                const V ln = vsub(l, vsub(h, s_));
+                X n = vadd(x, inc);
+                x_set_value(n, h);
+                x = keep ? hold(n, x) : n;
+                lo = keep ? hold(ln, lo) : ln;
             };
-            X h = s.phi[q], l = s.plo[q], ch = s.c[q], cl_ = s.clo[q];
-            add2(h, l, vmul(pd[q], dtq));
-            add2(ch, cl_, vmul(dFc, dtq));
-            s.phi[q] = h;   // a rate of 0 leaves the ghosts' phi
-            s.plo[q] = l;
-            s.c[q] = x_pair(glo ? x_lo(s.c[q]) : x_lo(ch), ghi ? x_hi(s.c[q]) : x_hi(ch));
-            s.clo[q] = x_pair(glo ? x_lo(s.clo[q]) : x_lo(cl_), ghi ? x_hi(s.clo[q]) : x_hi(cl_));
-            const X dn = vfma(dFd, dtq, s.d[q]);
-            s.d[q] = x_pair(glo ? x_lo(s.d[q]) : x_lo(dn), ghi ? x_hi(s.d[q]) : x_hi(dn));
+            add2(s.phi[q], s.plo[q], vmul(pd[q], dtq), false);   // a rate of 0 leaves the ghosts' phi
+            add2(s.c[q], s.clo[q], vmul(dFc, dtq), edge);
+            add2(s.d[q], s.dlo[q], vmul(dFd, dtq), edge);
         } else {
             s.phi[q] = vfma(pd[q], dtq, s.phi[q]);
             const X cn = vfma(dFc, dtq, s.c[q]), dn = vfma(dFd, dtq, s.d[q]);
-            s.c[q] = x_pair(glo ? x_lo(s.c[q]) : x_lo(cn), ghi ? x_hi(s.c[q]) : x_hi(cn));
-            s.d[q] = x_pair(glo ? x_lo(s.d[q]) : x_lo(dn), ghi ? x_hi(s.d[q]) : x_hi(dn));
+            s.c[q] = edge ? hold(cn, s.c[q]) : cn;
+            s.d[q] = edge ? hold(dn, s.d[q]) : dn;
         }
     }
 }

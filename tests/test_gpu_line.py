@@ -64,3 +64,18 @@ def test_strip_edges_fp32(cpt):
     for k in ("phi", "cs", "cl"):
         assert np.array_equal(few[k], many[k][:len(few[k])]), k
         assert np.abs(few[k] - ref[k]).max() <= 77 * 6e-8 * np.abs(ref[k]).max(), k
+
+
+@pytest.mark.parametrize("kw", [dict(A=1.2, b=0.8), dict(A=1.0, b=1.0, a=-0.3, interp="cubic", mobility="const", D_s=0.1)])
+def test_reverse_sweep_at_strip_edges(kw):
+    """FP64 derivatives by the reverse sweep equal the tangent run's on lengths at
+    the strips' edges, on clusters (10 instances) and on single CTAs (160): within
+    1e-9 of the largest, the bound of the other reverse tests."""
+    pr, f, dt = fronts(LENGTHS, v=0.8, **kw)
+    for rep in (1, 16):
+        args = (pr, LENGTHS * rep, [0.8] * (10 * rep), *[np.tile(a, rep) for a in f], 60)
+        t = pf.adjoint(*args, precision="fp64", dt=[dt] * (10 * rep))
+        r = pf.adjoint(*args, precision="fp64", dt=[dt] * (10 * rep), mode="reverse", checkpoint_every=13)
+        assert np.abs(r["k"] - t["k"]).max() <= 1e-13 * np.abs(t["k"]).max()
+        for j in range(3):
+            assert np.abs(r["dk"][:, j] - t["dk"][:, j]).max() <= 1e-9 * np.abs(t["dk"][:, j]).max(), j
