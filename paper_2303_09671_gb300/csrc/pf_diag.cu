@@ -51,24 +51,29 @@ static int diag_blocks(long long items) {
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
+// An unevaluated sum of two floats, |l| at most half an ulp of h: about 48 bits.
+// The FP64 pipe of a GB300 runs at 1/77 of the FP32 rate, so the sums over FP32
+// states are formed in pairs (Knuth's TwoSum; products by FMA); each thread's
+// totals then enter the FP64 block reduction.
+struct Pair {
+    float h, l;
+};
+static Pair pair_of(double v) {
+    const float h = (float)v;
+    return {h, (float)(v - (double)h)};
+}
+
 struct DiagConsts {
     int n[3], bc_lo[3], bc_hi[3], dim, lap, interp;
     double dir_phi, dx, H, sigma, k_e, a, theta0, G_theta, dV;
+    // in pairs: 1 + ln k_e, k_e - 1, and those above that the FP32 sums use
+    Pair lk2, ke2, H2, th2, Gx2, a2, dir2;
 };
 
 __device__ __forceinline__ double p_d(const DiagConsts& C, double f) {
     double g = f * (1.0 - f);
     double h = (C.interp == 1) ? f * f * (3.0 - 2.0 * f) : f * f * f * (6.0 * f * f - 15.0 * f + 10.0);
     return h + C.a * (f - 0.5) * g * g;
-}
-
-template <typename T>
-__device__ __forceinline__ double fetch_phi(const DiagConsts& C, const T* phi, int i, int j, int k) {
-    int mi = map_coord(i, C.n[0], C.bc_lo[0], C.bc_hi[0]);
-    int mj = (C.dim >= 2) ? map_coord(j, C.n[1], C.bc_lo[1], C.bc_hi[1]) : 0;
-    int mk = (C.dim >= 3) ? map_coord(k, C.n[2], C.bc_lo[2], C.bc_hi[2]) : 0;
-    if (mi < 0 || mj < 0 || mk == DIR_GHOST) return C.dir_phi;
-    return (double)phi[((long long)mk * C.n[1] + mj) * C.n[0] + mi];
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -97,6 +102,86 @@ __device__ void block_reduce2(double& a, double& b) {
     }
 }
 
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = a + b;
+    const float bb = s - a;
+    e = (a - (s - bb)) + (b - bb);
+}
+
+// ------------------------------------------------------ FP32 pairs
+__device__ __forceinline__ Pair quick_sum(float a, float b) {   // |a| >= |b| or a = 0
+    const float s = a + b;
+    return {s, b - (s - a)};
+}
+__device__ __forceinline__ Pair sum2(float a, float b) {
+    float s, e;
+    two_sum(a, b, s, e);
+    return {s, e};
+}
+__device__ __forceinline__ Pair prod2(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    return {p, __fmaf_rn(a, b, -p)};
+}
+__device__ __forceinline__ Pair operator+(Pair a, Pair b) {
+    const Pair s = sum2(a.h, b.h);
+    return quick_sum(s.h, s.l + (a.l + b.l));
+}
+__device__ __forceinline__ Pair operator-(Pair a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Pair operator-(Pair a, Pair b) { return a + (-b); }
+__device__ __forceinline__ Pair operator*(Pair a, Pair b) {
+    const Pair p = prod2(a.h, b.h);
+    return quick_sum(p.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, p.l)));
+}
+__device__ __forceinline__ Pair operator*(Pair a, float b) {
+    const Pair p = prod2(a.h, b);
+    return quick_sum(p.h, __fmaf_rn(a.l, b, p.l));
+}
+
+// ln of a pair to about 2^-48: x = 2^e m, a 9-bit approximation r of 1/m from a
+// table of 128 (with -ln r as a pair), z = m r - 1 exactly, |z| < 2^-7, and the
+// series of ln(1 + z) with its first two terms as pairs.  NaN where x is not a
+// positive normal number.
+struct LogTable {
+    float r[128], h[128], l[128];
+    LogTable() = default;
+    explicit LogTable(int) {
+        for (int t = 0; t < 128; ++t) {
+            const double q = std::rint(512.0 / (1.0 + (t + 0.5) / 128.0)) / 512.0;   // 9 bits
+            const Pair v = pair_of(-std::log(q));
+            r[t] = (float)q;
+            h[t] = v.h;
+            l[t] = v.l;
+        }
+    }
+};
+__device__ __forceinline__ Pair ln_pair(const LogTable& T, Pair x) {
+    if (!(x.h >= 1.17549435e-38f && x.h <= 3.402823466e38f)) return {NAN, 0.0f};
+    const int b = __float_as_int(x.h);
+    const int e = (b >> 23) - 127, t = (b >> 16) & 127;
+    const float m = __int_as_float((b & 0x007fffff) | 0x3f800000);
+    const float ml = __fmul_rn(__fmul_rn(x.l, __int_as_float((127 - e / 2) << 23)),
+                               __int_as_float((127 - (e - e / 2)) << 23));   // x.l 2^-e
+    const float r = T.r[t], ef = (float)e;
+    const Pair p = prod2(m, r);
+    const Pair z = quick_sum(p.h - 1.0f, __fmaf_rn(ml, r, p.l));
+    const float zz = z.h;
+    // ln 2 in parts of 14, 14 and 24 bits: e times the first two is exact
+    const float L1 = 0.693115234375f, L2 = 3.194436430931e-05f, L3 = 1.820635999e-09f;
+    Pair q = prod2(zz, zz);
+    q = {-0.5f * q.h, -__fmaf_rn(zz, z.l, 0.5f * q.l)};
+    const float c = zz * zz * zz *
+                    __fmaf_rn(zz, __fmaf_rn(zz, __fmaf_rn(zz, __fmaf_rn(zz, 1.0f / 7, -1.0f / 6), 0.2f), -0.25f),
+                              1.0f / 3);
+    Pair s = sum2(ef * L1, T.h[t]);
+    Pair a = sum2(s.h, zz);
+    float lo = s.l + a.l;
+    s = sum2(a.h, ef * L2);
+    lo += s.l;
+    a = sum2(s.h, q.h);
+    lo += a.l + (__fmaf_rn(ef, L3, T.l[t]) + (z.l + q.l) + c);
+    return quick_sum(a.h, lo);
+}
+
 // state accessors: c (with its FP32 low word), d -> c_s, c_l in FP64
 template <typename T>
 struct StateView {
@@ -119,6 +204,13 @@ struct StateView {
         s = cc + (1.0 - p) * dd;
         l = cc - p * dd;
     }
+    // total c, c_s and c_l of cell i as FP32 pairs, from its p
+    __device__ __forceinline__ void cell32(long long i, Pair p, Pair& cc, Pair& s, Pair& l) const {
+        cc = {(float)c[i], clo ? (float)clo[i] : 0.0f};
+        const float dd = (float)d[i];
+        l = cc - p * dd;
+        s = l + Pair{dd, 0.0f};
+    }
 };
 
 // the caller's fields (phi, c_s, c_l) read directly (pf_energy_solute_noalloc)
@@ -136,50 +228,235 @@ struct FieldView {
         p = p_d(C, f);
         cc = p * s + (1.0 - p) * l;   // Eq. model1 with g = p
     }
+    __device__ __forceinline__ void cell32(long long i, Pair p, Pair& cc, Pair& s, Pair& l) const {
+        s = {(float)cs[i], 0.0f};
+        l = {(float)cl[i], 0.0f};
+        cc = l + p * (s - l);
+    }
 };
 
-template <typename View, bool ENERGY>
-__global__ void __launch_bounds__(DIAG_THREADS)
-energy_solute_kernel(View S, DiagConsts C, double* __restrict__ part) {
-    const long long N = (long long)C.n[0] * C.n[1] * C.n[2];
-    double eF = 0.0, eS = 0.0;
-    const double one_m_ke = 1.0 - C.k_e, log_ke = log(C.k_e);
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < N;
-         c += (long long)gridDim.x * blockDim.x) {
-        double cc, f = 0.0, p = 0.0, s = 0.0, l = 0.0;
-        S.template cell<ENERGY>(C, c, cc, f, p, s, l);
-        eS += cc;
-        if (!ENERGY) continue;
-        const int i = (int)(c % C.n[0]);
-        const int j = (int)((c / C.n[0]) % C.n[1]);
-        const int k = (int)(c / ((long long)C.n[0] * C.n[1]));
-        const double theta = C.theta0 - C.G_theta * (((double)i + 0.5) * C.dx);
-        const double fs = -one_m_ke * theta + s * (log(s) - log_ke - 1.0);
-        const double fl = l * (log(l) - 1.0);
-        const double fdw = f * f * (1.0 - f) * (1.0 - f);
-        // gradient energy: each stencil pair once, weights of the Laplacian
-        double gs = 0.0;
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int nzc = (dx != 0) + (dy != 0) + (dz != 0);
-                    if (nzc == 0) continue;
-                    double w = 0.0;
-                    if (C.lap == 3) w = (dy == 0 && dz == 0) ? 1.0 : 0.0;
-                    else if (C.lap == 5) w = (dz == 0 && nzc == 1) ? 1.0 : 0.0;
-                    else if (C.lap == 9) w = (dz != 0) ? 0.0 : (nzc == 1 ? 2.0 / 3.0 : 1.0 / 6.0);
-                    else if (C.lap == 7) w = (nzc == 1) ? 1.0 : 0.0;
-                    else w = (nzc == 1) ? 1.0 / 3.0 : (nzc == 2 ? 1.0 / 6.0 : 0.0);
-                    if (w == 0.0) continue;
-                    const double dphi = fetch_phi(C, S.phi, i + dx, j + dy, k + dz) - f;
-                    gs += w * dphi * dphi;
+// A sum of weighted squared differences.
+template <typename T>
+struct SquareSum;
+template <>
+struct SquareSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double v, double f, double weight) { s += weight * ((v - f) * (v - f)); }
+    __device__ __forceinline__ double total() const { return s; }
+};
+template <>
+struct SquareSum<float> {
+    float h = 0.0f, l = 0.0f;
+    __device__ __forceinline__ void add(Pair d, float weight) {   // weight: a power of two
+        const Pair p = prod2(d.h, d.h);
+        const Pair s = sum2(h, weight * p.h);
+        h = s.h;
+        l += s.l + weight * __fmaf_rn(2.0f * d.h, d.l, p.l);
+    }
+    __device__ __forceinline__ void add(float v, float f, float weight) { add(sum2(v, -f), weight); }
+    __device__ __forceinline__ double total() const { return (double)h + (double)l; }
+};
+
+// position of a cell and the step of a grid-stride loop, advanced without divisions
+struct Cursor {
+    int i, j, k, si, sj, sk;
+    __device__ Cursor(const DiagConsts& C, long long c, long long stride) {
+        const long long row = c / C.n[0];
+        i = (int)(c - row * C.n[0]);
+        k = (int)(row / C.n[1]);
+        j = (int)(row - (long long)k * C.n[1]);
+        const long long srow = stride / C.n[0];
+        si = (int)(stride - srow * C.n[0]);
+        sk = (int)(srow / C.n[1]);
+        sj = (int)(srow - (long long)sk * C.n[1]);
+    }
+    __device__ __forceinline__ void next(const DiagConsts& C) {
+        i += si;
+        if (i >= C.n[0]) { i -= C.n[0]; j += 1; }
+        j += sj;
+        if (j >= C.n[1]) { j -= C.n[1]; k += 1; }
+        k += sk;
+    }
+};
+
+// Gradient energy: every pair of a cell c and a neighbour of its stencil with the
+// Laplacian's weight, s1 the face neighbours', s2 the edge neighbours' (corners of
+// a square in 2D).  A pair of cells of the grid is added once, by its lower cell;
+// a pair with a ghost beyond a mirror, Dirichlet or halo side belongs to one cell
+// only and counts half.
+template <int LAP, typename T>
+__device__ __forceinline__ void gradient_pairs(const DiagConsts& C, const T* __restrict__ phi, long long c, int i,
+                                               int j, int k, T f, SquareSum<T>& s1, SquareSum<T>& s2) {
+    constexpr int DIM = LAP == 3 ? 1 : LAP <= 9 && LAP != 7 ? 2 : 3;
+    constexpr bool DIAG = LAP == 9 || LAP == 19;
+    const int nx = C.n[0], ny = C.n[1], nz = C.n[2];
+    const long long oy = nx, oz = (long long)nx * ny;
+    const bool perx = C.bc_hi[0] == BC_PERIODIC, pery = DIM >= 2 && C.bc_hi[1] == BC_PERIODIC,
+               perz = DIM == 3 && C.bc_hi[2] == BC_PERIODIC;
+    // the neighbour above (p) and below (m) along each axis: in the grid, or wrapped
+    const bool px = i < nx - 1 || perx, mx = i > 0 || perx;
+    const bool py = DIM >= 2 && (j < ny - 1 || pery), my = DIM >= 2 && (j > 0 || pery);
+    const bool pz = DIM == 3 && (k < nz - 1 || perz), mz = DIM == 3 && (k > 0 || perz);
+    const long long xp = i < nx - 1 ? 1 : -(long long)(nx - 1), xm = i > 0 ? -1 : nx - 1;
+    const long long yp = j < ny - 1 ? oy : -(ny - 1) * oy, ym = j > 0 ? -oy : (ny - 1) * oy;
+    const long long zp = k < nz - 1 ? oz : -(nz - 1) * oz;
+    const T* q = phi + c;
+    const T one = T(1);
+    s1.add(px ? q[xp] : f, f, one);
+    if constexpr (DIM >= 2) s1.add(py ? q[yp] : f, f, one);
+    if constexpr (DIM == 3) s1.add(pz ? q[zp] : f, f, one);
+    if constexpr (DIAG) {
+        s2.add(px && py ? q[xp + yp] : f, f, one);
+        s2.add(mx && py ? q[xm + yp] : f, f, one);
+        if constexpr (DIM == 3) {
+            s2.add(px && pz ? q[xp + zp] : f, f, one);
+            s2.add(mx && pz ? q[xm + zp] : f, f, one);
+            s2.add(py && pz ? q[yp + zp] : f, f, one);
+            s2.add(my && pz ? q[ym + zp] : f, f, one);
+        }
+    }
+    const bool yz = (DIM < 2 || (py && my)) && (DIM < 3 || (pz && mz));
+    if (px && mx && yz) return;
+    // A mirror side along x, away from the other sides (the same lanes of a warp
+    // throughout the loop when rows are whole warps): the ghosts are the cell's own
+    // column, so only its edge neighbours differ.
+    if (yz && (px || C.bc_hi[0] == BC_NOFLUX) && (mx || C.bc_lo[0] == BC_NOFLUX)) {
+        if constexpr (DIAG) {
+            s2.add(q[yp], f, T(0.5));
+            s2.add(q[ym], f, T(0.5));
+            if constexpr (DIM == 3) {
+                s2.add(q[zp], f, T(0.5));
+                s2.add(q[k > 0 ? -oz : (nz - 1) * oz], f, T(0.5));
+            }
+        }
+        return;
+    }
+    for (int dz = (DIM == 3 ? -1 : 0); dz <= (DIM == 3 ? 1 : 0); ++dz)
+        for (int dy = (DIM >= 2 ? -1 : 0); dy <= (DIM >= 2 ? 1 : 0); ++dy)
+            for (int dx = -1; dx <= 1; ++dx) {
+                const int away = (dx != 0) + (dy != 0) + (dz != 0);
+                if (away == 0 || away > (DIAG ? 2 : 1)) continue;
+                const bool in = (dx == 0 || (dx > 0 ? px : mx)) && (dy == 0 || (dy > 0 ? py : my)) &&
+                                (dz == 0 || (dz > 0 ? pz : mz));
+                if (in) continue;
+                SquareSum<T>& s = away == 1 ? s1 : s2;
+                const int mi = map_coord(i + dx, nx, C.bc_lo[0], C.bc_hi[0]);
+                const int mj = DIM >= 2 ? map_coord(j + dy, ny, C.bc_lo[1], C.bc_hi[1]) : 0;
+                const int mk = DIM == 3 ? map_coord(k + dz, nz, C.bc_lo[2], C.bc_hi[2]) : 0;
+                if (mi < 0 || mj < 0 || mk == DIR_GHOST) {
+                    if constexpr (sizeof(T) == 4) s.add(C.dir2 - Pair{f, 0.0f}, 0.5f);
+                    else s.add(C.dir_phi, f, 0.5);
+                } else {
+                    s.add(phi[((long long)mk * ny + mj) * nx + mi], f, T(0.5));
                 }
-        eF += C.H * fdw + p * fs + (1.0 - p) * fl + 0.5 * C.sigma * 0.5 * gs / (C.dx * C.dx);
+            }
+}
+
+// FP64 energy density of a cell without its gradient part
+__device__ __forceinline__ double bulk_energy(const DiagConsts& C, double f, double p, double s, double l, int i,
+                                              double log_ke) {
+    const double theta = C.theta0 - C.G_theta * (((double)i + 0.5) * C.dx);
+    const double fs = -(1.0 - C.k_e) * theta + s * (log(s) - log_ke - 1.0);
+    const double fl = l * (log(l) - 1.0);
+    const double fdw = f * f * (1.0 - f) * (1.0 - f);
+    return C.H * fdw + p * fs + (1.0 - p) * fl;
+}
+
+// F_h and S_h.  The FP64 form is bound by the FP64 pipe (two logarithms and the
+// pairs).  An FP32 state is summed in FP32 pairs: 256^3 in 0.53 ms, bound by
+// instruction issue (71 % of cycles; 490 FP32 operations per cell), against 5.9 ms
+// in FP64 arithmetic with each pair of neighbours taken twice; the result agrees
+// with FP64's to its last digits.  Threads whose FP32 totals are not finite (a concentration that is not
+// a positive normal number, an overflow) repeat their cells in FP64.
+template <int LAP, typename View, typename T>
+__global__ void __launch_bounds__(DIAG_THREADS, sizeof(T) == 4 ? 3 : 1)
+energy_kernel(View S, const T* __restrict__ phi, const DiagConsts C, const __grid_constant__ LogTable logs,
+              double* __restrict__ part) {
+    const long long N = (long long)C.n[0] * C.n[1] * C.n[2];
+    const long long stride = (long long)gridDim.x * blockDim.x, first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    double eF = 0.0, eS = 0.0;
+    const double w1 = (LAP == 9 ? 2.0 / 3.0 : LAP == 19 ? 1.0 / 3.0 : 1.0), w2 = 1.0 / 6.0;
+    const double grad = 0.5 * C.sigma / (C.dx * C.dx);   // a pair counts twice in the sum over cells, each 1/4
+    bool exact = sizeof(T) == 8;
+    if constexpr (sizeof(T) == 4) {
+        __shared__ LogTable table;   // a copy that lanes read at different entries
+        for (int t = threadIdx.x; t < 128; t += DIAG_THREADS) {
+            table.r[t] = logs.r[t];
+            table.h[t] = logs.h[t];
+            table.l[t] = logs.l[t];
+        }
+        __syncthreads();
+        SquareSum<float> s1, s2;
+        Pair E = {0.0f, 0.0f}, Sc = {0.0f, 0.0f};
+        const Pair lk = C.lk2, ke = C.ke2, H = C.H2, th0 = C.th2, Gx = C.Gx2, ai = C.a2;
+        Cursor at(C, first, stride);
+        for (long long c = first; c < N; c += stride) {
+            const float f = phi[c];
+            gradient_pairs<LAP, float>(C, phi, c, at.i, at.j, at.k, f, s1, s2);
+            // p = h + a (f - 1/2) g^2, g = f (1 - f)
+            const Pair ff = prod2(f, f), omf = sum2(1.0f, -f);
+            Pair h;
+            if (C.interp == 1) h = ff * (Pair{3.0f, 0.0f} - sum2(f, f));
+            else h = (ff * f) * (Pair{10.0f, 0.0f} + (prod2(6.0f, f) - Pair{15.0f, 0.0f}) * f);
+            const Pair g = omf * f, gg = g * g;
+            Pair p = h;
+            if (C.a != 0.0) p = h + (ai * sum2(f, -0.5f)) * gg;
+            Pair cc, s, l;
+            S.cell32(c, p, cc, s, l);
+            const Pair fs0 = s * (ln_pair(table, s) - lk), fl = l * (ln_pair(table, l) - Pair{1.0f, 0.0f});
+            Pair theta = th0;
+            if (C.G_theta != 0.0) theta = th0 - Gx * sum2((float)(at.i & ~4095), (float)(at.i & 4095) + 0.5f);
+            const Pair fs = ke * theta + fs0;
+            const Pair e = (fl + p * (fs - fl)) + H * gg;
+            E = E + e;
+            Sc = Sc + cc;
+            at.next(C);
+        }
+        exact = !(isfinite(E.h) && isfinite(Sc.h) && isfinite(s1.h) && isfinite(s2.h) && isfinite(s1.l) &&
+                  isfinite(s2.l));
+        eS = (double)Sc.h + (double)Sc.l;
+        eF = (double)E.h + (double)E.l + grad * (w1 * s1.total() + w2 * s2.total());
+    }
+    if (exact) {
+        SquareSum<double> s1, s2;
+        eF = eS = 0.0;
+        const double log_ke = log(C.k_e);
+        Cursor at(C, first, stride);
+        for (long long c = first; c < N; c += stride) {
+            double cc, f = 0.0, p = 0.0, s = 0.0, l = 0.0;
+            S.template cell<true>(C, c, cc, f, p, s, l);
+            eS += cc;
+            if constexpr (sizeof(T) == 8) {
+                gradient_pairs<LAP, double>(C, phi, c, at.i, at.j, at.k, f, s1, s2);
+            } else {
+                SquareSum<float> t1, t2;
+                gradient_pairs<LAP, float>(C, phi, c, at.i, at.j, at.k, phi[c], t1, t2);
+                s1.s += t1.total();
+                s2.s += t2.total();
+            }
+            eF += bulk_energy(C, f, p, s, l, at.i, log_ke);
+            at.next(C);
+        }
+        eF += grad * (w1 * s1.s + w2 * s2.s);
     }
     block_reduce2<false>(eF, eS);
     if (threadIdx.x == 0) {
         part[blockIdx.x] = eF;
         part[gridDim.x + blockIdx.x] = eS;
+    }
+}
+
+// total c of an FP64 state
+__global__ void __launch_bounds__(DIAG_THREADS)
+solute_f64_kernel(const double* __restrict__ c, long long n, double* __restrict__ part) {
+    double s = 0.0, unused = 0.0;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x)
+        s += c[i];
+    block_reduce2<false>(s, unused);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = 0.0;
+        part[gridDim.x + blockIdx.x] = s;
     }
 }
 
@@ -205,23 +482,36 @@ finish_sum2(const double* __restrict__ part, int nb, double scale, double* __res
     }
 }
 
+// The largest phi = 0.5 crossing along x and the largest c.  Every cell is one
+// step of a grid-stride loop (a thread per x row read 32 rows' cells per warp
+// access: 0.56 ms at 256^3); a row's largest crossing is the one the scan from
+// the hot end would meet first.  An FP32 c is compared word by word: hi + lo is
+// normalised, so the pairs order as their sums do; NaN in either word is passed
+// over, as fmax passes it over.
 template <typename T>
 __global__ void __launch_bounds__(DIAG_THREADS)
 front_kernel(StateView<T> S, DiagConsts C, double* __restrict__ part) {
-    const long long rows = (long long)C.n[1] * C.n[2];
-    double xf = -INFINITY, cm = -INFINITY;
-    for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < rows;
-         r += (long long)gridDim.x * blockDim.x) {
-        const T* prow = S.phi + r * C.n[0];
-        for (int i = C.n[0] - 2; i >= 0; --i) {
-            const double a = (double)prow[i], b = (double)prow[i + 1];
-            if (a >= 0.5 && b < 0.5) {
-                xf = fmax(xf, ((double)i + 0.5 + (a - 0.5) / (a - b)) * C.dx);
-                break;
+    const long long N = (long long)C.n[0] * C.n[1] * C.n[2];
+    const long long stride = (long long)gridDim.x * blockDim.x, first = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    double xf = -INFINITY;
+    T bh = -INFINITY, bl = T(0);
+    Cursor at(C, first, stride);
+    for (long long c = first; c < N; c += stride) {
+        const T f = S.phi[c], h = S.c[c], l = S.clo != nullptr ? S.clo[c] : T(0);
+        if (at.i < C.n[0] - 1) {
+            const T g = S.phi[c + 1];
+            if (f >= T(0.5) && g < T(0.5)) {
+                const double a = (double)f, b = (double)g;
+                xf = fmax(xf, ((double)at.i + 0.5 + (a - 0.5) / (a - b)) * C.dx);
             }
         }
-        for (int i = 0; i < C.n[0]; ++i) cm = fmax(cm, S.cval(r * C.n[0] + i));
+        if ((h > bh || (h == bh && l > bl)) && l == l) {
+            bh = h;
+            bl = l;
+        }
+        at.next(C);
     }
+    double cm = (double)bh + (double)bl;
     block_reduce2<true>(xf, cm);
     if (threadIdx.x == 0) {
         part[blockIdx.x] = xf;
@@ -290,12 +580,6 @@ __global__ void to_state_kernel(const T* __restrict__ phi, const T* __restrict__
 // two floats: c_s - c_l and c_l + p d by TwoSum, p d by an FMA-based exact
 // product (Knuth; Dekker), so the stored (c, c_lo) carries ~2^-48 relative
 // error with respect to that p.
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
 // one cell: (phi, c_s, c_l) -> (c, c_lo, d)
 __device__ __forceinline__ void convert_f32(float f, float s, float l, float a, bool cubic, float& c,
                                             float& clo, float& d) {
@@ -500,6 +784,13 @@ static DiagConsts make_diag(const HostProblem& P, int64_t step, int64_t shifts) 
     C.theta0 = P.theta_ref + P.G_theta * (P.x0 + P.v_pull * t - (double)shifts * P.dx);
     C.G_theta = P.G_theta;
     C.dV = std::pow(P.dx, P.dim);
+    C.lk2 = pair_of(1.0 + std::log(P.k_e));
+    C.ke2 = pair_of(P.k_e - 1.0);
+    C.H2 = pair_of(P.H);
+    C.th2 = pair_of(C.theta0);
+    C.Gx2 = pair_of(P.G_theta * P.dx);
+    C.a2 = pair_of(P.a);
+    C.dir2 = pair_of(P.dir_phi);
     return C;
 }
 
@@ -508,21 +799,27 @@ static StateView<T> view(const Fields& f) {
     return StateView<T>{(const T*)f.phi, (const T*)f.c, (const T*)f.d, (const T*)f.clo};
 }
 
+template <typename T, typename View>
+static void launch_energy(const View& v, const T* phi, const DiagConsts& C, int nb, double* scratch, cudaStream_t s) {
+    auto k = C.lap == 3 ? energy_kernel<3, View, T> : C.lap == 5 ? energy_kernel<5, View, T>
+           : C.lap == 9 ? energy_kernel<9, View, T> : C.lap == 7 ? energy_kernel<7, View, T>
+                                                                  : energy_kernel<19, View, T>;
+    static const LogTable logs(0);
+    k<<<nb, DIAG_THREADS, 0, s>>>(v, phi, C, logs, scratch);
+}
+
 cudaError_t launch_energy_solute(const HostProblem& P, const Fields& f, int64_t step,
                                  int64_t shifts, bool with_energy, double* scratch, double* out,
                                  cudaStream_t s, long long* slot) {
     const DiagConsts C = make_diag(P, step, shifts);
     const int nb = diag_blocks(P.cells());
-    if (P.precision == 1) {
-        if (with_energy)
-            energy_solute_kernel<StateView<double>, true><<<nb, DIAG_THREADS, 0, s>>>(view<double>(f), C, scratch);
-        else
-            energy_solute_kernel<StateView<double>, false><<<nb, DIAG_THREADS, 0, s>>>(view<double>(f), C, scratch);
+    if (with_energy) {
+        if (P.precision == 1) launch_energy<double>(view<double>(f), (const double*)f.phi, C, nb, scratch, s);
+        else launch_energy<float>(view<float>(f), (const float*)f.phi, C, nb, scratch, s);
+    } else if (P.precision == 1) {
+        solute_f64_kernel<<<nb, DIAG_THREADS, 0, s>>>((const double*)f.c, P.cells(), scratch);
     } else {
-        if (with_energy)
-            energy_solute_kernel<StateView<float>, true><<<nb, DIAG_THREADS, 0, s>>>(view<float>(f), C, scratch);
-        else solute_f32_kernel<<<nb, DIAG_THREADS, 0, s>>>(
-            (const float*)f.c, (const float*)f.clo, P.cells(), scratch);
+        solute_f32_kernel<<<nb, DIAG_THREADS, 0, s>>>((const float*)f.c, (const float*)f.clo, P.cells(), scratch);
     }
     finish_sum2<<<1, DIAG_THREADS, 0, s>>>(scratch, nb, C.dV, out, slot);
     return cudaGetLastError();
@@ -534,11 +831,11 @@ cudaError_t launch_energy_solute_fields(const HostProblem& P, const void* phi, c
     const DiagConsts C = make_diag(P, step, shifts);
     const int nb = diag_blocks(P.cells());
     if (P.precision == 1)
-        energy_solute_kernel<FieldView<double>, true><<<nb, DIAG_THREADS, 0, s>>>(
-            FieldView<double>{(const double*)phi, (const double*)cs, (const double*)cl}, C, scratch);
+        launch_energy<double>(FieldView<double>{(const double*)phi, (const double*)cs, (const double*)cl},
+                              (const double*)phi, C, nb, scratch, s);
     else
-        energy_solute_kernel<FieldView<float>, true><<<nb, DIAG_THREADS, 0, s>>>(
-            FieldView<float>{(const float*)phi, (const float*)cs, (const float*)cl}, C, scratch);
+        launch_energy<float>(FieldView<float>{(const float*)phi, (const float*)cs, (const float*)cl},
+                             (const float*)phi, C, nb, scratch, s);
     finish_sum2<<<1, DIAG_THREADS, 0, s>>>(scratch, nb, C.dV, out, nullptr);
     return cudaGetLastError();
 }
@@ -546,7 +843,7 @@ cudaError_t launch_energy_solute_fields(const HostProblem& P, const void* phi, c
 cudaError_t launch_front(const HostProblem& P, const Fields& f, double* scratch, double* out,
                          cudaStream_t s) {
     const DiagConsts C = make_diag(P, 0, 0);
-    const int nb = diag_blocks(P.cells() / P.n[0]);   // one thread per x row
+    const int nb = diag_blocks(P.cells());
     if (P.precision == 1)
         front_kernel<double><<<nb, DIAG_THREADS, 0, s>>>(view<double>(f), C, scratch);
     else
