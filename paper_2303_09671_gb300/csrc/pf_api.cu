@@ -72,6 +72,12 @@ struct pf_handle {
     cudaEvent_t sp_start = nullptr, sp_done = nullptr;
     bool split = false;
     int split_lo = 0, split_hi = 0;
+    // 1D: the multi-step line kernels (pf_step1d.cu); partial energies of up to
+    // LINE_RECORDS states of line_strips strips each (0: energies by the reduction)
+    bool line = false;
+    int line_strips = 0;
+    double* line_part = nullptr;
+    static constexpr int64_t LINE_RECORDS = 4096;
     std::string err;
 };
 
@@ -331,6 +337,8 @@ int pf_create(const pf_grid* grid, const pf_bc* bc, const pf_params* params, voi
         pf_destroy(h);
         return fail(nullptr, PF_ENOMEM, std::string("allocation failed: ") + cudaGetErrorString(e));
     }
+    h->line = !h->generic && pf::line_eligible(P);
+    h->line_strips = h->line ? pf::line_energy_strips(P) : 0;
     *out = h;
     return PF_OK;
 }
@@ -366,6 +374,7 @@ void pf_destroy(pf_handle* h) {
     if (h->dres) cudaFree(h->dres);
     if (h->hres) cudaFreeHost(h->hres);
     if (h->drec) cudaFree(h->drec);
+    if (h->line_part) cudaFree(h->line_part);
     for (cudaStream_t s : h->ov)
         if (s) cudaStreamDestroy(s);
     for (cudaEvent_t ev : h->ov_ev) cudaEventDestroy(ev);
@@ -679,6 +688,52 @@ int pf_get_fields(pf_handle* h, void* phi, void* cs, void* cl, int where) {
     return step_error(h);
 }
 
+// n steps of a 1D handle's line; with epart, the energies of the states before
+// them into records erec, erec + 1, ... (negative ones left out)
+static int line_steps(pf_handle* h, int64_t n, double* epart, int64_t erec) {
+    pf::LineRun r;
+    r.buf[0] = h->buf[0];
+    r.buf[1] = h->buf[1];
+    r.cur = h->cur;
+    r.step = h->step;
+    r.shifts = h->shifts;
+    r.stream = h->stream;
+    r.epart = epart;
+    r.erec = erec;
+    const cudaError_t e = pf::line_steps(h->P, r, n);
+    h->cur = r.cur;
+    h->step = r.step;
+    h->shifts = r.shifts;
+    return e == cudaSuccess ? PF_OK : cuda_fail(h, e, "step kernel launch");
+}
+
+// the energy of the current state of a 1D handle, as the step kernels sum it,
+// into record erec of epart
+static int line_energy(pf_handle* h, double* epart, int64_t erec) {
+    pf::LineRun r;
+    r.buf[0] = h->buf[0];
+    r.buf[1] = h->buf[1];
+    r.cur = h->cur;
+    r.step = h->step;
+    r.shifts = h->shifts;
+    r.stream = h->stream;
+    r.store = false;
+    r.epart = epart;
+    r.erec = erec;
+    const cudaError_t e = pf::line_steps(h->P, r, 1);
+    return e == cudaSuccess ? PF_OK : cuda_fail(h, e, "energy kernel launch");
+}
+
+// the partial sums' buffer, on first use
+static int line_partials(pf_handle* h) {
+    if (h->line_part) return PF_OK;
+    cudaError_t e = cudaMalloc(&h->line_part, (size_t)pf_handle::LINE_RECORDS * h->line_strips * sizeof(double));
+    if (e == cudaSuccess) return PF_OK;
+    cudaGetLastError();
+    h->line_part = nullptr;
+    return fail(h, PF_ENOMEM, std::string("energy partials: ") + cudaGetErrorString(e));
+}
+
 int pf_step(pf_handle* h, int64_t n) {
     if (!h) return fail(nullptr, PF_EINVAL, "null handle");
     if (int rc = split_closed(h)) return rc;
@@ -692,6 +747,7 @@ int pf_step(pf_handle* h, int64_t n) {
     if (n > 0)
         if (int rc = join_readback(h)) return rc;
     const pf::HostProblem& P = h->P;
+    if (h->line && n > 0) return line_steps(h, n, nullptr, 0);
     for (int64_t s = 0; s < n; ++s) {
         const pf::StepLaunch a = step_launch(h, h->buf[h->cur], h->buf[h->cur ^ 1], h->stream);
         cudaError_t e = pf::launch_step(a);
@@ -731,7 +787,16 @@ int pf_energy(pf_handle* h, double* F) {
     if (!F) return fail(h, PF_EINVAL, "null output");
     if ((h->halo[0] && !h->halo_set[0]) || (h->halo[1] && !h->halo_set[1]))
         return fail(h, PF_EINVAL, "halo not imported: the energy's gradient pairs reach the ghost planes");
-    int rc = energy_solute(h, true);
+    int rc = PF_OK;
+    if (h->line_strips > 0) {   // summed as pf_step_energies' records are (scratch holds 2 x 2048 doubles)
+        rc = line_energy(h, h->scratch, 0);
+        if (rc) return rc;
+        cudaError_t e = pf::line_energy_records(h->P, h->scratch, h->line_strips, 1, h->dres, h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "energy kernel launch");
+        rc = fetch_results(h, 2);
+    } else {
+        rc = energy_solute(h, true);
+    }
     if (rc) return rc;
     *F = h->hres[0];
     if (!std::isfinite(*F)) return fail(h, PF_ENONFINITE, "non-finite free energy");
@@ -765,21 +830,43 @@ int pf_step_energies(pf_handle* h, int64_t n, double* F) {
     long long* slot = reinterpret_cast<long long*>(h->drec + 2 * h->rec_cap);
     cudaError_t e = cudaMemsetAsync(slot, 0, sizeof(long long), h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "record counter");
+    int64_t done = 0;
     auto one = [&]() -> int {
         int rc = pf_step(h, 1);
         if (rc) return rc;
-        cudaError_t x = pf::launch_energy_solute(h->P, h->buf[h->cur], h->step, h->shifts, true, h->scratch,
-                                                 h->drec, h->stream, slot);
+        cudaError_t x;
+        if (h->line_strips > 0) {
+            rc = line_energy(h, h->scratch, 0);
+            if (rc) return rc;
+            x = pf::line_energy_records(h->P, h->scratch, h->line_strips, 1, h->drec + 2 * done, h->stream);
+        } else {
+            x = pf::launch_energy_solute(h->P, h->buf[h->cur], h->step, h->shifts, true, h->scratch, h->drec,
+                                         h->stream, slot);
+        }
         return x == cudaSuccess ? PF_OK : cuda_fail(h, x, "energy kernel launch");
     };
-    int64_t done = 0;
     // Without a moving temperature or window every step launches the same
     // kernels with the same arguments (the ping-pong parity returns after an
     // even count, the record slot advances on the device), so a captured block
     // of GS steps is replayed instead of launching three kernels per step.
     const pf::HostProblem& P = h->P;
     constexpr int64_t GS = 64;
-    if (P.G_theta == 0.0 && P.v_pull == 0.0 && !P.shift && n >= 2 + 2 * GS) {
+    // A 1D FP64 line in a fixed temperature: the step kernels sum the energy of the
+    // state before every step; the last state's follows the last step.
+    if (h->line_strips > 0 && !P.shift && (P.G_theta == 0.0 || P.v_pull == 0.0)) {
+        if (int rc = line_partials(h)) return rc;
+        for (int64_t first = 0; first < n;) {      // records first .. first + count - 1
+            const int64_t count = std::min<int64_t>(n - first, pf_handle::LINE_RECORDS);
+            // record r is the state after r + 1 steps: before step r + 2, or at the end of the chunk
+            if (int rc = line_steps(h, count, h->line_part, -1)) return rc;
+            if (int rc = line_energy(h, h->line_part, count - 1)) return rc;
+            e = pf::line_energy_records(P, h->line_part, h->line_strips, count, h->drec + 2 * first, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "energy records");
+            first += count;
+        }
+        done = n;
+    }
+    if (done < n && P.G_theta == 0.0 && P.v_pull == 0.0 && !P.shift && n >= 2 + 2 * GS) {
         for (; done < 2; ++done)   // first uses set kernel attributes outside the capture
             if (int rc = one()) return rc;
         // capture and replay on a stream of our own, ordered after and before

@@ -123,8 +123,9 @@ struct LineRecord {
         base[4 * n + i] = l;
         base[5 * n + i] = r;
     }
-    __device__ __forceinline__ void operator()(int q, const X& f, const X& c, const X& d, const X& s, const X& l,
-                                               const X& r) const {
+    template <typename V>
+    __device__ __forceinline__ void operator()(int q, const X& f, const X&, const X&, const X& c, const X& d,
+                                               const X& s, const X& l, const X& r, const V&) const {
         if (base == nullptr) return;
         const int i = i0 - m + q;
         one(i, x_lo(f), x_lo(c), x_lo(d), x_lo(s), x_lo(l), x_lo(r));
@@ -176,7 +177,7 @@ batch_kernel(const __grid_constant__ BatchArgs<T> a) {
     constexpr int H = J / 2;
     constexpr int USE = 30 * J;      // cells of a strip that hold results
     constexpr bool REC = MODE == BATCH_RECORD;
-    constexpr bool COMP = MODE != BATCH_PLAIN && sizeof(S) == 4;
+    constexpr int COMP = MODE != BATCH_PLAIN && sizeof(S) == 4 ? 2 : 0;
     const int csize = a.cluster;
     const int inst = a.ids[blockIdx.x / csize];
     const BatchState St = a.st[inst];

@@ -55,6 +55,27 @@ template <typename T>
 cudaError_t step3d_chunks(const HostProblem& P, int requested, int* zchunk, int* nchunks);
 size_t step_smem_bytes(int precision, int dim);
 
+// Several steps of a 1D line per launch (pf_step1d.cu), for lines with a no-flux
+// low end and a no-flux or Dirichlet high end, and for periodic lines in a uniform
+// temperature.  line_steps advances the run's buffers and clock, window shifts
+// included.  With epart it also writes the energy of the state before each step,
+// in line_energy_strips(P) partials per record (0: not for this line); store =
+// false evaluates one state's energy and leaves the state alone.
+struct LineRun {
+    Fields buf[2];
+    int cur;
+    int64_t step, shifts;
+    cudaStream_t stream;
+    bool store = true;
+    double* epart = nullptr;   // [record][strip]
+    int64_t erec = 0;          // record of the next step's state (negative: none)
+};
+bool line_eligible(const HostProblem& P);
+int line_energy_strips(const HostProblem& P);
+cudaError_t line_steps(const HostProblem& P, LineRun& r, int64_t count);
+cudaError_t line_energy_records(const HostProblem& P, const double* epart, int strips, int64_t count, double* out,
+                                cudaStream_t s);
+
 // Diagnostics.  `scratch` must hold diag_scratch_doubles(prob) doubles
 // (2 DIAG_MAX_BLOCKS: one partial pair per block of a reduction grid of at most
 // 8 blocks per SM and at most DIAG_MAX_BLOCKS blocks); results are written as

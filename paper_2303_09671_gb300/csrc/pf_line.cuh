@@ -32,28 +32,56 @@ struct DV {
     V v, t;
 };
 
+// A lane of a Mono strip holds one FP64 cell per value instead of two: short FP64
+// lines, whose cells are fewer than the lanes of the FP64 pipes.
+struct Mono {};
+
 template <typename E>
-struct LineNum;   // element type -> vector types
+struct LineNum;   // element type -> vector types; M: the element in memory
 template <>
 struct LineNum<float> {
     using S = float;    // scalar without derivative
+    using M = float;
     using V = float2;
     using X = float2;
+    static constexpr int LANES = 2;
+};
+template <>
+struct LineNum<Mono> {
+    using S = double;
+    using M = double;
+    using V = double;
+    using X = double;
+    static constexpr int LANES = 1;
 };
 template <>
 struct LineNum<double> {
     using S = double;
+    using M = double;
     using V = double2;
     using X = double2;
+    static constexpr int LANES = 2;
 };
 template <typename T>
 struct LineNum<Dual<T>> {
     using S = T;
+    using M = Dual<T>;
     using V = typename LineNum<T>::V;
     using X = DV<V>;
+    static constexpr int LANES = 2;
 };
 
 #define PF_D __device__ __forceinline__
+// one cell: its value is both "lanes", and a pair of values is its first
+PF_D double x_lo(double a) { return a; }
+PF_D double x_hi(double a) { return a; }
+// (never contracted, so that every kernel that evaluates a cell gets the same bits)
+PF_D double vadd(double a, double b) { return __dadd_rn(a, b); }
+PF_D double vsub(double a, double b) { return __dsub_rn(a, b); }
+PF_D double vmul(double a, double b) { return __dmul_rn(a, b); }
+PF_D double vfma(double a, double b, double c) { return fma(a, b, c); }
+template <>
+PF_D double vlit<double>(double v) { return v; }
 PF_D float x_lo(float2 a) { return a.x; }
 PF_D float x_hi(float2 a) { return a.y; }
 PF_D double x_lo(double2 a) { return a.x; }
@@ -74,6 +102,8 @@ template <typename T>
 PF_D Dual<T> from_below(Dual<T> x) { return make_dual(from_below(x.v), from_below(x.t)); }
 template <typename T>
 PF_D Dual<T> from_above(Dual<T> x) { return make_dual(from_above(x.v), from_above(x.t)); }
+PF_D double x_value(double a) { return a; }
+PF_D void x_set_value(double& a, double v) { a = v; }
 PF_D float2 x_value(float2 a) { return a; }
 PF_D double2 x_value(double2 a) { return a; }
 template <typename V>
@@ -117,6 +147,7 @@ PF_D float2 vrcp_n(float2 x) {
     asm("rcp.approx.f32 %0, %1;" : "=f"(r.y) : "f"(x.y));
     return r;
 }
+PF_D double vrcp_n(double x) { return 1.0 / x; }
 PF_D double2 vrcp_n(double2 x) { return make_double2(1.0 / x.x, 1.0 / x.y); }
 template <typename V> PF_D DV<V> vrcp_n(DV<V> x) {
     const V r = vrcp_n(x.v);
@@ -149,19 +180,33 @@ PF_D float2 ln_normal(float2 x) {
     y = vfma(z, vlit<float2>(-0.5), y);
     return vfma(e, vlit<float2>(0.693359375 / 8388608.0), vadd(f, y));
 }
+PF_D double ln_normal(double x) { return log(x); }
 PF_D double2 ln_normal(double2 x) { return make_double2(log(x.x), log(x.y)); }
 template <typename V> PF_D DV<V> ln_normal(DV<V> x) {
     return {ln_normal(x.v), vmul(x.t, vrcp_n(x.v))};
 }
 PF_D bool is_positive(float2 x) { return x.x >= FLT_MIN && x.y >= FLT_MIN; }   // false for NaN
+PF_D bool is_positive(double) { return true; }
 PF_D bool is_positive(double2) { return true; }   // log() takes any value
 template <typename V> PF_D bool is_positive(DV<V> x) { return is_positive(x.v); }
 // ln x where x is not a positive normal number, else the given l
 PF_D float2 ln_fix(float2 x, float2 l) {
     return make_float2(x.x >= FLT_MIN ? l.x : logf(x.x), x.y >= FLT_MIN ? l.y : logf(x.y));
 }
+PF_D double ln_fix(double, double l) { return l; }
 PF_D double2 ln_fix(double2, double2 l) { return l; }
 template <typename V> PF_D DV<V> ln_fix(DV<V> x, DV<V> l) { return {ln_fix(x.v, l.v), l.t}; }
+
+template <typename V, typename S>
+__host__ __device__ __forceinline__ V line_splat(S v) {
+    if constexpr (sizeof(V) == sizeof(S)) {
+        return v;
+    } else {
+        V r;
+        r.x = r.y = v;
+        return r;
+    }
+}
 
 // ---------------------------------------------------------------- parameters
 // broadcast to both lanes; X carries the derivative of a differentiated parameter
@@ -334,7 +379,7 @@ inline LineConsts<E> make_line_consts(const HostProblem& P, int dir) {
     Consts<double> C;
     C.interp = P.interp; C.mobility = P.mobility; C.D_s = P.D_s; C.D_l = P.D_l;
     set_coefficients(C);
-    auto v = [](double x) { V r; r.x = S(x); r.y = S(x); return r; };
+    auto v = [](double x) { return line_splat<V>(S(x)); };
     auto x = [&](Dual<double> u) {
         if constexpr (IsDual<E>::value) return X{v(u.v), v(u.t)};
         else return v(u.v);
@@ -406,25 +451,32 @@ PF_D void line_face(const LineConsts<E>& K, DV<V> fL, DV<V> fR, DV<V> YL, DV<V> 
     Fd = vfma(RD, TD, ae);
 }
 
+// the vector of two cells' values; of one cell, its own
+template <typename X, typename A>
+PF_D X x_join(A a, A b) {
+    if constexpr (sizeof(X) == sizeof(A)) return a;
+    else return x_pair(a, b);
+}
 template <typename X, typename E>
 PF_D X x_select(X a, E other, bool lo, bool hi) {
-    return x_pair(lo ? other : x_lo(a), hi ? other : x_hi(a));
+    return x_join<X>(lo ? other : x_lo(a), hi ? other : x_hi(a));
 }
 
-// The strip's state and one step of it.  COMP: the values of phi, c and d are
-// unevaluated FP32 pairs (compensated sums).
-template <typename E, int J, bool COMP>
+// The strip's state and one step of it.  COMP: the values of phi and c (1), or of
+// phi, c and d (2), are unevaluated FP32 pairs (compensated sums).
+template <typename E, int J, int COMP>
 struct Strip {
-    static constexpr int H = J / 2;
+    static constexpr int H = J / LineNum<E>::LANES;
     using X = typename LineNum<E>::X;
     using V = typename LineNum<E>::V;
     X phi[H], c[H], d[H];
-    V plo[COMP ? H : 1], clo[COMP ? H : 1], dlo[COMP ? H : 1];
+    V plo[COMP ? H : 1], clo[COMP ? H : 1], dlo[COMP == 2 ? H : 1];
 };
 
 struct NoRecord {
-    template <typename X>
-    PF_D void operator()(int, const X&, const X&, const X&, const X&, const X&, const X&) const {}
+    template <typename X, typename V>
+    PF_D void operator()(int, const X&, const X&, const X&, const X&, const X&, const X&, const X&, const X&,
+                         const V&) const {}
     static constexpr bool on = false;
 };
 
@@ -434,15 +486,17 @@ struct NoRecord {
 // outside the window.  EDGE: the strip reaches an end of the line (a compile-time
 // switch, so that the other strips carry none of its selections).  dtq = dt / dx^2;
 // ke_theta0 = (1 - k_e) theta0 (theta0 as Consts::G_theta describes it).  record(q, phi,
-// c_s, c_l, mu_s, mu_l, rate) is called for every pair with its state before the
-// step; the rate it is given is in grid units.
-template <bool STD, bool edge, typename E, int J, bool COMP, typename Rec>
+// phi of the right neighbour, p, c_s, c_l, mu_s, mu_l, rate, (1 - k_e) theta) is
+// called for every pair with its state before the step; the rate it is given is in
+// grid units.
+template <bool STD, bool edge, typename E, int J, int COMP, typename Rec>
 PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n, int m,
                     typename LineNum<E>::V dtq, double ke_theta0, const Rec& record) {
     using X = typename LineNum<E>::X;
     using V = typename LineNum<E>::V;
     using S = typename LineNum<E>::S;
-    constexpr int H = J / 2;
+    using M = typename LineNum<E>::M;
+    constexpr int H = J / LineNum<E>::LANES;
     X cs[H], cl[H], mus[H], mul[H], Y[H], pd[H], p[H];
     bool fine = true;
 #pragma unroll
@@ -452,9 +506,12 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
         const X mp = vsub(vlit<V>(0.0), p[q]);
         cs[q] = vfma(omp, s.d[q], s.c[q]);
         cl[q] = vfma(mp, s.d[q], s.c[q]);
-        if constexpr (COMP) {   // the low words, of the values
+        if constexpr (COMP == 2) {   // the low words, of the values
             cs[q] = vadd(cs[q], vfma(x_value(omp), s.dlo[q], s.clo[q]));
             cl[q] = vadd(cl[q], vfma(x_value(mp), s.dlo[q], s.clo[q]));
+        } else if constexpr (COMP == 1) {
+            cs[q] = vadd(cs[q], s.clo[q]);
+            cl[q] = vadd(cl[q], s.clo[q]);
         }
         fine = fine && is_positive(cs[q]) && is_positive(cl[q]);
         mus[q] = ln_normal(cs[q]);
@@ -477,13 +534,18 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
         Y[q] = vfma(p[q], dmu[q], mul[q]);
     }
     // neighbours across the lane's ends
-    auto left_of = [&](const X (&a)[H]) { return x_pair(from_below(x_hi(a[H - 1])), x_lo(a[H - 1])); };
-    auto right_of = [&](const X (&a)[H]) { return x_pair(x_hi(a[0]), from_above(x_lo(a[0]))); };
+    auto left_of = [&](const X (&a)[H]) {
+        if constexpr (LineNum<E>::LANES == 1) return from_below(a[H - 1]);
+        else return x_pair(from_below(x_hi(a[H - 1])), x_lo(a[H - 1]));
+    };
+    auto right_of = [&](const X (&a)[H]) {
+        if constexpr (LineNum<E>::LANES == 1) return from_above(a[0]);
+        else return x_pair(x_hi(a[0]), from_above(x_lo(a[0])));
+    };
     const X fA = left_of(s.phi), sA = left_of(mus), lA = left_of(mul);
     const X fB = right_of(s.phi), sB = right_of(mus), lB = right_of(mul);
     const S xi = S(i0 - m) + S(0.5);
-    V th0;   // (1 - k_e) theta = ke_theta0 + ke_G (i + 1/2)
-    th0.x = th0.y = S(ke_theta0);
+    const V th0 = line_splat<V>(S(ke_theta0));   // (1 - k_e) theta = ke_theta0 + ke_G (i + 1/2)
 #pragma unroll
     for (int q = 0; q < H; ++q) {
         X fL = q > 0 ? s.phi[q - 1] : fA, sL = q > 0 ? mus[q - 1] : sA, lL = q > 0 ? mul[q - 1] : lA;
@@ -491,20 +553,18 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
         const int ia = i0 + q, ib = i0 + q + H;
         if (edge) {
             // mirror ghosts: the cold end always, the hot end if it is closed
-            if (ia == m) { fL = x_pair(x_lo(s.phi[q]), x_hi(fL)); sL = x_pair(x_lo(mus[q]), x_hi(sL)); lL = x_pair(x_lo(mul[q]), x_hi(lL)); }
-            if (ib == m) { fL = x_pair(x_lo(fL), x_hi(s.phi[q])); sL = x_pair(x_lo(sL), x_hi(mus[q])); lL = x_pair(x_lo(lL), x_hi(mul[q])); }
+            if (ia == m) { fL = x_join<X>(x_lo(s.phi[q]), x_hi(fL)); sL = x_join<X>(x_lo(mus[q]), x_hi(sL)); lL = x_join<X>(x_lo(mul[q]), x_hi(lL)); }
+            if (ib == m) { fL = x_join<X>(x_lo(fL), x_hi(s.phi[q])); sL = x_join<X>(x_lo(sL), x_hi(mus[q])); lL = x_join<X>(x_lo(lL), x_hi(mul[q])); }
             if (K.hot_noflux) {
-                if (ia == hot - 1) { fR = x_pair(x_lo(s.phi[q]), x_hi(fR)); sR = x_pair(x_lo(mus[q]), x_hi(sR)); lR = x_pair(x_lo(mul[q]), x_hi(lR)); }
-                if (ib == hot - 1) { fR = x_pair(x_lo(fR), x_hi(s.phi[q])); sR = x_pair(x_lo(sR), x_hi(mus[q])); lR = x_pair(x_lo(lR), x_hi(mul[q])); }
+                if (ia == hot - 1) { fR = x_join<X>(x_lo(s.phi[q]), x_hi(fR)); sR = x_join<X>(x_lo(mus[q]), x_hi(sR)); lR = x_join<X>(x_lo(mul[q]), x_hi(lR)); }
+                if (ib == hot - 1) { fR = x_join<X>(x_lo(fR), x_hi(s.phi[q])); sR = x_join<X>(x_lo(sR), x_hi(mus[q])); lR = x_join<X>(x_lo(lR), x_hi(mul[q])); }
             }
         }
-        V xc;   // (1 - k_e) theta at the cell centres
-        xc.x = xi + S(q);
-        xc.y = xi + S(q + H);
+        const V ke_theta = vfma(K.ke_G, x_join<V>(xi + S(q), xi + S(q + H)), th0);
         pd[q] = line_rate<STD>(K, s.phi[q], fL, fR, sL, sR, lL, lR, cs[q], cl[q], dmu[q], p[q],
-                               vfma(K.ke_G, xc, th0));
-        if (edge) pd[q] = x_select(pd[q], E(0), ia >= hot, ib >= hot);
-        if constexpr (Rec::on) record(q, s.phi[q], cs[q], cl[q], mus[q], mul[q], pd[q]);
+                               ke_theta);
+        if (edge) pd[q] = x_select(pd[q], M(0), ia >= hot, ib >= hot);
+        if constexpr (Rec::on) record(q, s.phi[q], fR, p[q], cs[q], cl[q], mus[q], mul[q], pd[q], ke_theta);
     }
     const X YB = right_of(Y), csB = right_of(cs), clB = right_of(cl), pdB = right_of(pd);
     X Fc[H], Fd[H];
@@ -519,15 +579,15 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
             const int ia = i0 + q, ib = i0 + q + H;
             const bool zlo = ia == m - 1 || (K.hot_noflux && ia == hot - 1);
             const bool zhi = ib == m - 1 || (K.hot_noflux && ib == hot - 1);
-            Fc[q] = x_select(Fc[q], E(0), zlo, zhi);
-            Fd[q] = x_select(Fd[q], E(0), zlo, zhi);
+            Fc[q] = x_select(Fc[q], M(0), zlo, zhi);
+            Fd[q] = x_select(Fd[q], M(0), zlo, zhi);
         }
     }
     X FcL = left_of(Fc), FdL = left_of(Fd);
     if (edge) {   // a line that begins at the lane's (or the strip's) first cell
         const bool zlo = i0 == m, zhi = i0 + H == m;
-        FcL = x_select(FcL, E(0), zlo, zhi);
-        FdL = x_select(FdL, E(0), zlo, zhi);
+        FcL = x_select(FcL, M(0), zlo, zhi);
+        FdL = x_select(FdL, M(0), zlo, zhi);
     }
 #pragma unroll
     for (int q = 0; q < H; ++q) {
@@ -535,7 +595,7 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
         const X dFd = vsub(Fd[q], q > 0 ? Fd[q > 0 ? q - 1 : 0] : FdL);
         const bool glo = edge && i0 + q >= hot, ghi = edge && i0 + q + H >= hot;
         auto hold = [&](auto now, auto before) {   // the ghosts' c and d stay
-            return x_pair(glo ? x_lo(before) : x_lo(now), ghi ? x_hi(before) : x_hi(now));
+            return x_join<decltype(now)>(glo ? x_lo(before) : x_lo(now), ghi ? x_hi(before) : x_hi(now));
         };
         if constexpr (COMP) {
             // compensated (TwoSum) updates of the values phi, c, d = hi + lo; the
@@ -554,7 +614,12 @@ PF_D void line_step(const LineConsts<E>& K, Strip<E, J, COMP>& s, int i0, int n,
             };
             add2(s.phi[q], s.plo[q], vmul(pd[q], dtq), false);   // a rate of 0 leaves the ghosts' phi
             add2(s.c[q], s.clo[q], vmul(dFc, dtq), edge);
-            add2(s.d[q], s.dlo[q], vmul(dFd, dtq), edge);
+            if constexpr (COMP == 2) {
+                add2(s.d[q], s.dlo[q], vmul(dFd, dtq), edge);
+            } else {
+                const X dn = vfma(dFd, dtq, s.d[q]);
+                s.d[q] = edge ? hold(dn, s.d[q]) : dn;
+            }
         } else {
             s.phi[q] = vfma(pd[q], dtq, s.phi[q]);
             const X cn = vfma(dFc, dtq, s.c[q]), dn = vfma(dFd, dtq, s.d[q]);

@@ -79,3 +79,80 @@ def test_reverse_sweep_at_strip_edges(kw):
         assert np.abs(r["k"] - t["k"]).max() <= 1e-13 * np.abs(t["k"]).max()
         for j in range(3):
             assert np.abs(r["dk"][:, j] - t["dk"][:, j]).max() <= 1e-9 * np.abs(t["dk"][:, j]).max(), j
+
+
+LINES = [("pulled", dict(V=1.5)), ("closed", dict(bc_hi=("noflux",))),
+         ("periodic", dict(bc_lo=("periodic",), bc_hi=("periodic",))),
+         ("cold_dirichlet", dict(bc_lo=("dirichlet",), bc_hi=("noflux",)))]
+
+
+def line_state(kind, kw, n):
+    if kind == "pulled":
+        pr, *f = wl.pulled_front_1d(N=n, front_cell=max(1, n // 3), A=1.0, b=1.0, **kw)
+        return pr, f
+    if kind == "closed":
+        pr, *f = wl.random_state(1, (n,), A=1.2, b=0.7, a=0.2, seed=n, **kw)
+        return pr, f
+    pr, *f = wl.random_state(1, (n,), A=1.0, b=1.0, a=0.2, seed=n, amp=0.1, **kw)
+    if kind == "periodic":   # a smooth profile that closes on itself
+        f[0] = 0.5 + 0.1 * np.sin(2 * np.pi * (np.arange(n) + 0.3) / n)
+    if kind == "cold_dirichlet":   # a solid cold end
+        pr["dirichlet"] = (1.0, pr["k_e"], 1.0)
+    return pr, f
+
+
+@pytest.mark.parametrize("kind,kw", LINES)
+@pytest.mark.parametrize("n", [3, 16, 17, 33, 113, 500, 2432, 2433])
+def test_single_line_fp64(kind, kw, n):
+    """A Sim's line over the sizes at which strips, their halos and the choice of
+    kernel change: against the oracle, and the same bits however its steps are
+    grouped into calls."""
+    pr, f = line_state(kind, kw, n)
+    steps = 21
+    st = oracle.State(pr, *f)
+    st.step(steps)
+    out = []
+    for groups in ([21], [1] * 21, [2, 9, 3, 7]):
+        with pf.Sim(pr, "fp64") as s:
+            s.set_fields(*f)
+            for g in groups:
+                s.step(g)
+            out.append(s.get_fields())
+            assert s.clock == (steps, st.clock.shifts)
+    for got, ref in zip(out[0], (st.phi, st.cs, st.cl)):
+        assert rel_err(got, ref) <= 1e-11
+    for o in out[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(out[0], o))
+
+
+@pytest.mark.parametrize("n", [3, 33, 500, 19456, 19457])
+def test_single_line_fp32(n):
+    """FP32 with a moving window, both kernels (19456 cells fill the SMs of the
+    first): the same bits in one call and in single steps, and within 21 roundings
+    of FP32 of the FP64 line."""
+    pr, *f = wl.pulled_front_1d(N=n, front_cell=max(1, min(40, n // 3)), V=1.5, A=1.0, b=1.0)
+    f = [a.astype(np.float32) for a in f]
+    out = []
+    for prec, groups in (("fp64", [21]), ("fp32", [21]), ("fp32", [1] * 21)):
+        with pf.Sim(pr, prec) as s:
+            s.set_fields(*f)
+            for g in groups:
+                s.step(g)
+            out.append(s.get_fields())
+    for ref, a, b in zip(*out):
+        assert np.array_equal(a, b)
+        assert np.abs(a - ref).max() <= 21 * 6e-8 * np.abs(ref).max()
+
+
+def test_window_jumps_by_many_cells():
+    """A clock set far ahead: the next step drops every cell it is behind by."""
+    pr, *f = wl.pulled_front_1d(N=100, V=1.0, A=1.0, b=1.0)
+    for prec in ("fp32", "fp64"):
+        with pf.Sim(pr, prec) as s:
+            s.set_fields(*f)
+            s.set_clock(int(30 * pr["dx"] / pr["dt"]), 0)
+            s.step(1)
+            assert s.clock[1] in (30, 31)
+            k = s.clock[1]
+            g = s.get_fields()
+        assert np.abs(g[0][:100 - k] - f[0][k:]).max() < 0.1 and np.all(np.abs(g[0][100 - k:]) < 1e-6)
