@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include "pf_fp64.cuh"
 #include "pf_internal.cuh"
 #include "pf_kernels.h"
 
@@ -41,7 +42,7 @@ __device__ __forceinline__ float2 vsub(float2 a, float2 b) {
 // FP32 reciprocal and natural logarithm from the PTX approximate instructions
 // (rcp.approx, lg2.approx; flush-to-zero, as every operand here is a normal
 // number of moderate size): 1/x to ~1 ulp, ln x = ln 2 log2 x to ~2^-22
-// relative.  The FP64 path below is exact IEEE.
+// relative.  The FP64 path below is within about an ulp (pf_fp64.cuh).
 __device__ __forceinline__ float rcp_fast(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -62,8 +63,8 @@ __device__ __forceinline__ double2 vfma(double2 a, double2 b, double2 c) {
     return make_double2(fma(a.x, b.x, c.x), fma(a.y, b.y, c.y));
 }
 __device__ __forceinline__ double2 vsub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ double2 vrcp(double2 a) { return make_double2(1.0 / a.x, 1.0 / a.y); }
-__device__ __forceinline__ double2 vlog(double2 a) { return make_double2(log(a.x), log(a.y)); }
+__device__ __forceinline__ double2 vrcp(double2 a) { return make_double2(rcp64(a.x), rcp64(a.y)); }
+__device__ __forceinline__ double2 vlog(double2 a) { return make_double2(log64(a.x), log64(a.y)); }
 __device__ __forceinline__ double2 vpair(double a, double b) { return make_double2(a, b); }
 
 // a compile-time constant on both lanes

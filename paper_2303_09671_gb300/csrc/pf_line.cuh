@@ -140,15 +140,15 @@ template <typename V> PF_D DV<V> vfma(DV<V> a, V b, V c) { return vfma(b, a, c);
 
 // Reciprocal.  FP32: the hardware approximation, within 1 ulp; a Newton step
 // after it (errors near half an ulp, as a division has) cost 2 to 3 % and changed
-// the error of no field, k_v or derivative against 64 bits.  FP64: IEEE.
+// the error of no field, k_v or derivative against 64 bits.  FP64: rcp64.
 PF_D float2 vrcp_n(float2 x) {
     float2 r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r.x) : "f"(x.x));
     asm("rcp.approx.f32 %0, %1;" : "=f"(r.y) : "f"(x.y));
     return r;
 }
-PF_D double vrcp_n(double x) { return 1.0 / x; }
-PF_D double2 vrcp_n(double2 x) { return make_double2(1.0 / x.x, 1.0 / x.y); }
+PF_D double vrcp_n(double x) { return rcp64(x); }
+PF_D double2 vrcp_n(double2 x) { return vrcp(x); }
 template <typename V> PF_D DV<V> vrcp_n(DV<V> x) {
     const V r = vrcp_n(x.v);
     return {r, vmul(vsub(vlit<V>(0.0), x.t), vmul(r, r))};
@@ -180,14 +180,14 @@ PF_D float2 ln_normal(float2 x) {
     y = vfma(z, vlit<float2>(-0.5), y);
     return vfma(e, vlit<float2>(0.693359375 / 8388608.0), vadd(f, y));
 }
-PF_D double ln_normal(double x) { return log(x); }
-PF_D double2 ln_normal(double2 x) { return make_double2(log(x.x), log(x.y)); }
+PF_D double ln_normal(double x) { return log64(x); }
+PF_D double2 ln_normal(double2 x) { return vlog(x); }
 template <typename V> PF_D DV<V> ln_normal(DV<V> x) {
     return {ln_normal(x.v), vmul(x.t, vrcp_n(x.v))};
 }
 PF_D bool is_positive(float2 x) { return x.x >= FLT_MIN && x.y >= FLT_MIN; }   // false for NaN
 PF_D bool is_positive(double) { return true; }
-PF_D bool is_positive(double2) { return true; }   // log() takes any value
+PF_D bool is_positive(double2) { return true; }   // log64 takes any value
 template <typename V> PF_D bool is_positive(DV<V> x) { return is_positive(x.v); }
 // ln x where x is not a positive normal number, else the given l
 PF_D float2 ln_fix(float2 x, float2 l) {

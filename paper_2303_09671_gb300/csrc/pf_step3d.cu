@@ -28,7 +28,7 @@
 //     rate is dx^2 dphi/dt, so that F_c, F_d below are dx times the fluxes of
 //     the model and the update is c += dt/dx^2 sum(F+ - F-);
 //   * FP32 reciprocals and logarithms use the hardware approximations (a few
-//     ulp), FP64 is exact IEEE.
+//     ulp), FP64 those of pf_fp64.cuh (about an ulp).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
