@@ -24,7 +24,9 @@
 
 namespace pf {
 
-template <typename T, int TX, int TY>
+// HELP: 64 more threads that take the ring's border and the tile's low edge faces,
+// which are otherwise second tasks of the tile's own warps
+template <typename T, int TX, int TY, bool HELP>
 struct PTile2 {
     static_assert(TY % 2 == 0, "cells are paired along y");
     using V = typename Lanes<T>::V;
@@ -35,9 +37,10 @@ struct PTile2 {
     static constexpr int HP = HX * HYP;
     static constexpr int RW = TX + 2, RX = HX;          // halo-1 ring (all pair rows), pitch HX
     static constexpr int NR = RW * HYP;
-    static constexpr int JH = (HP + NT - 1) / NT;
+    static constexpr int THREADS = NT + (HELP ? 64 : 0);
+    static constexpr int JH = (HP + THREADS - 1) / THREADS;
     static constexpr int NB = NR - NT;                  // ring cells besides the own pairs
-    static_assert(NB == 2 * RW + 2 * TYP && NB <= NT, "ring = own pairs + border");
+    static_assert(NB == 2 * RW + 2 * TYP && NB <= (HELP ? 64 : NT), "ring = own pairs + border");
     static constexpr size_t OFF_A = 0;                               // {phi, Y}
     static constexpr size_t OFF_B = OFF_A + sizeof(Q) * HP;          // {mu_s, mu_l}
     static constexpr size_t OFF_C = OFF_B + sizeof(Q) * HP;          // {c_s, c_l}
@@ -48,18 +51,18 @@ struct PTile2 {
     static constexpr size_t BYTES = OFF_FY + sizeof(V) * (TYP + 1) * TX;
 };
 
-template <typename T, int TX, int TY, bool L9, bool AI>
-__global__ void __launch_bounds__(TX * (TY / 2), sizeof(T) == 4 ? 3 : 1)
+template <typename T, int TX, int TY, bool HELP, bool L9, bool AI>
+__global__ void __launch_bounds__(TX * (TY / 2) + (HELP ? 64 : 0), sizeof(T) == 4 ? 3 : 1)
 step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T* __restrict__ d_in,
               const T* __restrict__ clo_in, T* __restrict__ phi_out, T* __restrict__ c_out,
               T* __restrict__ d_out, T* __restrict__ clo_out, const PairConsts<typename Lanes<T>::V> K,
               const GridConsts<T> G) {
-    using L = PTile2<T, TX, TY>;
+    using L = PTile2<T, TX, TY, HELP>;
     using V = typename L::V;
     using Q = typename L::Q;
     constexpr int HX = L::HX, HP = L::HP, RX = L::RX, RW = L::RW, NT = L::NT, TYP = L::TYP, NB = L::NB;
     static_assert(HP < 4096, "tile too large for the packed ring descriptors");
-    static_assert(NT >= 32 + TX && TYP <= 32, "edge faces need warps 0 and 1");
+    static_assert((HELP ? 64 : NT) >= 32 + TX && TYP <= 32, "edge faces need two warps");
     extern __shared__ __align__(16) unsigned char smem[];
     Q* sA = reinterpret_cast<Q*>(smem + L::OFF_A);
     Q* sB = reinterpret_cast<Q*>(smem + L::OFF_B);
@@ -70,14 +73,16 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
     V* sFy = reinterpret_cast<V*>(smem + L::OFF_FY);
 
     const int tid = threadIdx.x;
-    const int tx = tid % TX, ty = tid / TX;
+    const bool owner = !HELP || tid < NT;   // the others are the helping warps
+    const int extra = HELP ? tid - NT : tid;
+    const int tx = owner ? tid % TX : 0, ty = owner ? tid / TX : 0;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
     const int nx = G.n[0], ny = G.n[1];
     const int own_h = (ty + 1) * HX + tx + 2;
     const int own_r = (ty + 1) * RX + tx + 1;
     const int own_x = x0 + tx, own_y = y0 + 2 * ty;
-    const bool in_lo = own_x < nx && own_y < ny;
-    const bool in_hi = own_x < nx && own_y + 1 < ny;
+    const bool in_lo = owner && own_x < nx && own_y < ny;
+    const bool in_hi = owner && own_x < nx && own_y + 1 < ny;
     const long long own_xy = (long long)own_y * nx + own_x;
 
     // own state for the update, in flight while the tile is converted
@@ -96,8 +101,8 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
     // ---- A: the halo-2 tile into two-lane records
 #pragma unroll
     for (int j = 0; j < L::JH; ++j) {
-        const int h = tid + j * NT;
-        if ((j + 1) * NT > HP && h >= HP) break;
+        const int h = tid + j * L::THREADS;
+        if ((j + 1) * L::THREADS > HP && h >= HP) break;
         const int mx = map_coord(x0 - 2 + h % HX, nx, G.bc_lo[0], G.bc_hi[0]);
         T f2[2], c2[2], d2[2];
 #pragma unroll
@@ -183,9 +188,9 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
         const V R = vfma(K.sigma, lap, vmul(K.dx2, vsub(anti, vfma(K.H, dfdw, vmul(dG, dp)))));
         sD[ry * RX + rx] = vmask(vmul(R, vrcp(Kc)), glo, ghi);
     };
-    rate_cell(tx + 1, ty + 1);
-    if (tid >= NT - NB) {
-        const int b = tid - (NT - NB);
+    if (owner) rate_cell(tx + 1, ty + 1);
+    if (HELP ? extra >= 0 && extra < NB : tid >= NT - NB) {
+        const int b = HELP ? extra : tid - (NT - NB);
         if (b < RW) rate_cell(b, 0);
         else if (b < 2 * RW) rate_cell(b - RW, L::HYP - 1);
         else if (b < 2 * RW + TYP) rate_cell(0, 1 + b - 2 * RW);
@@ -238,23 +243,25 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
     const bool nf_x = own_x == nx - 1 && G.bc_hi[0] == BC_NOFLUX;
     const bool nf_ylo = own_y == ny - 1 && G.bc_hi[1] == BC_NOFLUX;
     const bool nf_yhi = own_y + 1 == ny - 1 && G.bc_hi[1] == BC_NOFLUX;
-    V fxc, fxd, fyc, fyd;
-    xface(own_h, own_r, fxc, fxd);
-    yface(own_h, own_r, fyc, fyd);
-    if (nf_x) fxc = fxd = vpair(T(0), T(0));
-    fyc = vmask(fyc, nf_ylo, nf_yhi);
-    fyd = vmask(fyd, nf_ylo, nf_yhi);
-    sFx[ty * (TX + 1) + tx + 1] = Q{fxc, fxd};
-    sFy[(ty + 1) * TX + tx] = vpair(fyc.y, fyd.y);
-    if (tid < TYP) {
-        // x faces on the tile's low x edge, pair row tid
+    V fxc = vlit<V>(0.0), fxd = fxc, fyc = fxc, fyd = fxc;
+    if (owner) {
+        xface(own_h, own_r, fxc, fxd);
+        yface(own_h, own_r, fyc, fyd);
+        if (nf_x) fxc = fxd = vpair(T(0), T(0));
+        fyc = vmask(fyc, nf_ylo, nf_yhi);
+        fyd = vmask(fyd, nf_ylo, nf_yhi);
+        sFx[ty * (TX + 1) + tx + 1] = Q{fxc, fxd};
+        sFy[(ty + 1) * TX + tx] = vpair(fyc.y, fyd.y);
+    }
+    if (extra >= 0 && extra < TYP) {
+        // x faces on the tile's low x edge, pair row `extra`
         V ec, ed;
-        xface((tid + 1) * HX + 1, (tid + 1) * RX, ec, ed);
+        xface((extra + 1) * HX + 1, (extra + 1) * RX, ec, ed);
         if (x0 == 0 && G.bc_lo[0] == BC_NOFLUX) ec = ed = vpair(T(0), T(0));
-        sFx[tid * (TX + 1)] = Q{ec, ed};
-    } else if (tid >= 32 && tid < 32 + TX) {
+        sFx[extra * (TX + 1)] = Q{ec, ed};
+    } else if (extra >= 32 && extra < 32 + TX) {
         // y face on the tile's low y edge (upper lane of the pair row below the tile)
-        const int ex = tid - 32;
+        const int ex = extra - 32;
         V ec, ed;
         yface(ex + 2, ex + 1, ec, ed);
         sFy[ex] = (y0 == 0 && G.bc_lo[1] == BC_NOFLUX) ? vpair(T(0), T(0)) : vpair(ec.y, ed.y);
@@ -262,6 +269,7 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
     __syncthreads();
 
     // ---- D: conservative update of the pair
+    if (!owner) return;
     const Q left = sFx[ty * (TX + 1) + tx];
     const V below = sFy[ty * TX + tx];
     const V dFc = vadd(vsub(fxc, left.a), vpair(fyc.x - below.x, fyc.y - fyc.x));
@@ -298,14 +306,13 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
     }
 }
 
-template <typename T>
-cudaError_t launch_step2d(const StepLaunch& a, const Consts<T>& C, const Clock<T>& Kc) {
-    constexpr int TX = 32, TY = 16;
-    using L = PTile2<T, TX, TY>;
+template <typename T, int TX, int TY, bool HELP>
+static cudaError_t launch_tile2d(const StepLaunch& a, const Consts<T>& C, const Clock<T>& Kc) {
+    using L = PTile2<T, TX, TY, HELP>;
     // 9- or 5-point Laplacian x shape parameter a != 0 or a = 0
-    decltype(&step2d_kernel<T, TX, TY, true, true>) kerns[2][2] = {
-        {step2d_kernel<T, TX, TY, false, false>, step2d_kernel<T, TX, TY, false, true>},
-        {step2d_kernel<T, TX, TY, true, false>, step2d_kernel<T, TX, TY, true, true>}};
+    decltype(&step2d_kernel<T, TX, TY, HELP, true, true>) kerns[2][2] = {
+        {step2d_kernel<T, TX, TY, HELP, false, false>, step2d_kernel<T, TX, TY, HELP, false, true>},
+        {step2d_kernel<T, TX, TY, HELP, true, false>, step2d_kernel<T, TX, TY, HELP, true, true>}};
     static DeviceSetup setup;
     {
         int dev = 0;
@@ -324,7 +331,7 @@ cudaError_t launch_step2d(const StepLaunch& a, const Consts<T>& C, const Clock<T
     const HostProblem& P = *a.prob;
     const PairConsts<typename L::V> K = make_pair_consts<T>(P, C);
     const GridConsts<T> G = make_grid_consts<T>(P, Kc);
-    const dim3 block(L::NT);
+    const dim3 block(L::THREADS);
     const dim3 grid((C.n[0] + TX - 1) / TX, (C.n[1] + TY - 1) / TY, 1);
     auto kern = kerns[C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
     kern<<<grid, block, L::BYTES, a.stream>>>(
@@ -332,6 +339,34 @@ cudaError_t launch_step2d(const StepLaunch& a, const Consts<T>& C, const Clock<T
         static_cast<const T*>(a.clo_in), static_cast<T*>(a.phi_out), static_cast<T*>(a.c_out),
         static_cast<T*>(a.d_out), static_cast<T*>(a.clo_out), K, G);
     return cudaGetLastError();
+}
+
+// 32 x 16 tiles.  FP64 grids that 16 x 8 tiles with helping warps fit in two per
+// SM take those: the kernel is then bound by the latency of FP64 chains on few
+// warps (128^2: 82 us per step with 32 x 16 tiles, 37 with the small ones; 200 x
+// 160, 260 small tiles: 82 and 51; 256^2, 512 small tiles: 82 and 110).  In FP32
+// both take 6.2 us up to 256^2.
+template <typename T>
+cudaError_t launch_step2d(const StepLaunch& a, const Consts<T>& C, const Clock<T>& Kc) {
+    if constexpr (sizeof(T) == 8) {
+        static DeviceSetup setup;
+        int dev = 0, sms = 1;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev < 0 || dev >= DeviceSetup::MAX_DEVICES) return cudaErrorInvalidDevice;
+        {
+            std::lock_guard<std::mutex> lock(setup.mu);
+            if (!setup.done[dev]) {
+                e = cudaDeviceGetAttribute(&setup.sms[dev], cudaDevAttrMultiProcessorCount, dev);
+                if (e != cudaSuccess) return e;
+                setup.done[dev] = true;
+            }
+            sms = setup.sms[dev];
+        }
+        const long long small = (long long)((C.n[0] + 15) / 16) * ((C.n[1] + 7) / 8);
+        if (small <= 2 * sms) return launch_tile2d<T, 16, 8, true>(a, C, Kc);
+    }
+    return launch_tile2d<T, 32, 16, false>(a, C, Kc);
 }
 
 template cudaError_t launch_step2d<float>(const StepLaunch&, const Consts<float>&, const Clock<float>&);
