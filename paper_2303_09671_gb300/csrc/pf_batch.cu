@@ -658,6 +658,35 @@ cudaError_t set_smem_limits(size_t* max_dynamic, int* sms) {
     return setup.err[dev];
 }
 
+// device arrays of one call: listed, then allocated together and freed together
+// (ten allocations and frees took 0.3 ms of a call)
+struct Arena {
+    std::vector<std::pair<void**, size_t>> want;
+    void* base = nullptr;
+    template <typename P>
+    void add(P** p, size_t bytes) {
+        want.push_back({reinterpret_cast<void**>(p), (bytes + 255) / 256 * 256});
+    }
+    cudaError_t allocate() {
+        size_t total = 0;
+        for (auto& w : want) total += w.second;
+        cudaError_t e = cudaMalloc(&base, total > 0 ? total : 256);
+        if (e != cudaSuccess) {
+            base = nullptr;
+            return e;
+        }
+        char* p = static_cast<char*>(base);
+        for (auto& w : want) {
+            *w.first = p;
+            p += w.second;
+        }
+        return e;
+    }
+    ~Arena() {
+        if (base) cudaFree(base);
+    }
+};
+
 struct Group {
     int warps;         // of a CTA
     int dir = -1;      // seeded parameter of a tangent run (0 M_phi, 1 A, 2 b), -1 none
@@ -682,6 +711,9 @@ struct BatchRun {
     bool deriv = false;                      // a run for derivatives
     int64_t slot_in = 0, slot_out = 0;   // the copies of the state a launch reads and writes
     double *dv = nullptr, *ddt = nullptr;
+    Arena mem;
+    int* ids = nullptr;         // instance numbers, group after group
+    std::vector<int> ids_host;
     std::vector<Group> groups;
     int J = 2, cluster = 1;     // cells per lane and CTAs per instance of the groups
     bool std_phys = false;
@@ -697,14 +729,7 @@ struct BatchRun {
 
     BatchRun(const pf_batch_desc& d_, cudaStream_t s, std::string& e) : D(d_), main(s), err(e) {}
     ~BatchRun() {
-        for (Group& g : groups) {
-            if (g.d_ids) cudaFree(g.d_ids);
-            if (g.stream) cudaStreamDestroy(g.stream);
-            if (g.done) cudaEventDestroy(g.done);
-        }
-        void* ptrs[] = {phi, c, d, st, dv, ddt, energy, low};
-        for (void* p : ptrs)
-            if (p) cudaFree(p);
+        drop_groups();
         if (fork) cudaEventDestroy(fork);
         if (t0) cudaEventDestroy(t0);
         if (t1) cudaEventDestroy(t1);
@@ -761,27 +786,36 @@ struct BatchRun {
     // `count` launches of nsteps steps each, every group's on its own stream: a
     // group does not wait for the others' launches until the last is done
     cudaError_t issue(int nsteps, int count = 1) {
-        cudaError_t e = cudaEventRecord(fork, main);
+        cudaError_t e = groups.size() > 1 ? cudaEventRecord(fork, main) : cudaSuccess;
         for (Group& g : groups) {
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(g.stream, fork, 0);
+            const cudaStream_t on = g.stream ? g.stream : main;
+            if (e == cudaSuccess && g.stream) e = cudaStreamWaitEvent(on, fork, 0);
             const BatchArgs<T> a = args(g, nsteps);
             for (int l = 0; l < count && e == cudaSuccess; ++l)
                 e = launch_clusters(batch_fn<T>(J, std_phys, mode()), a.count, cluster, g.warps,
-                                    g.room * batch_cell_bytes<T>(mode()), g.stream, a);
-            if (e == cudaSuccess) e = cudaEventRecord(g.done, g.stream);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(main, g.done, 0);
+                                    g.room * batch_cell_bytes<T>(mode()), on, a);
+            if (e == cudaSuccess && g.stream) e = cudaEventRecord(g.done, on);
             launches += count;
         }
+        for (Group& g : groups)
+            if (e == cudaSuccess && g.stream) e = cudaStreamWaitEvent(main, g.done, 0);
         return e;
     }
 
-    cudaError_t make_groups(int cpt) {
+    void drop_groups() {
         for (Group& g : groups) {
-            if (g.d_ids) cudaFree(g.d_ids);
             if (g.stream) cudaStreamDestroy(g.stream);
             if (g.done) cudaEventDestroy(g.done);
         }
         groups.clear();
+    }
+
+    cudaError_t make_groups(int cpt) {
+        if (!groups.empty()) {   // an earlier choice: its copies of ids may still be read
+            const cudaError_t e = cudaStreamSynchronize(main);
+            if (e != cudaSuccess) return e;
+            drop_groups();
+        }
         J = deriv ? 2 : cells_per_lane<T>(cpt);
         std_phys = line_std(problem());
         const int64_t use = 30 * J;
@@ -810,18 +844,23 @@ struct BatchRun {
             g.room = std::max(g.room, (int)(strips * use + 2 * J));
             g.ids.push_back(i);
         }
-        // largest instances first inside a group: the long CTAs start early
+        // largest instances first inside a group: the long CTAs start early.  The
+        // last group runs on the main stream, the others on their own.
+        ids_host.clear();
         for (auto& kv : by) {
             Group g = kv.second;
             std::sort(g.ids.begin(), g.ids.end(), [&](int x, int y) { return D.n[x] > D.n[y]; });
-            cudaError_t e = cudaMalloc(&g.d_ids, g.ids.size() * sizeof(int));
-            if (e == cudaSuccess) e = cudaMemcpy(g.d_ids, g.ids.data(), g.ids.size() * sizeof(int), cudaMemcpyHostToDevice);
-            if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming);
+            g.d_ids = ids + ids_host.size();
+            ids_host.insert(ids_host.end(), g.ids.begin(), g.ids.end());
+            cudaError_t e = cudaSuccess;
+            if (groups.size() + 1 < by.size()) {
+                e = cudaStreamCreateWithFlags(&g.stream, cudaStreamNonBlocking);
+                if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g.done, cudaEventDisableTiming);
+            }
             groups.push_back(g);
             if (e != cudaSuccess) return e;
         }
-        return cudaSuccess;
+        return cudaMemcpyAsync(ids, ids_host.data(), ids_host.size() * sizeof(int), cudaMemcpyHostToDevice, main);
     }
 };
 
@@ -858,38 +897,34 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
     }
     if (!batch_time_steps(D, B.dt, err)) return PF_EINVAL;
     const size_t fb = (size_t)B.total * sizeof(T);
-    cudaError_t e = cudaMalloc(&B.phi, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.c, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.d, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.st, N * sizeof(BatchState));
-    if (e == cudaSuccess) e = cudaMalloc(&B.dv, N * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&B.ddt, N * sizeof(double));
-    if (e == cudaSuccess && D.energy_every > 0) {
+    T *scs = nullptr, *scl = nullptr;   // c_s and c_l, on the way in and out
+    B.mem.add(&B.phi, fb);
+    B.mem.add(&B.c, fb);
+    B.mem.add(&B.d, fb);
+    B.mem.add(&B.st, N * sizeof(BatchState));
+    B.mem.add(&B.dv, N * sizeof(double));
+    B.mem.add(&B.ddt, N * sizeof(double));
+    B.mem.add(&B.ids, N * sizeof(int));
+    B.mem.add(&scs, fb);
+    B.mem.add(&scl, fb);
+    if (D.energy_every > 0) {
         // one record per energy_every steps up to max_steps, NaN where never written
-        const int64_t slots = D.max_steps / D.energy_every;
-        B.energy_slots = (int)slots;
-        e = cudaMalloc(&B.energy, (size_t)N * slots * sizeof(double));
-        if (e == cudaSuccess) e = cudaMemsetAsync(B.energy, 0xff, (size_t)N * slots * sizeof(double), main);
+        B.energy_slots = (int)(D.max_steps / D.energy_every);
+        B.mem.add(&B.energy, (size_t)N * B.energy_slots * sizeof(double));
     }
+    cudaError_t e = B.mem.allocate();
     if (e != cudaSuccess) {
         cudaGetLastError();
         err = std::string("device allocation failed: ") + cudaGetErrorString(e);
         return PF_ENOMEM;
     }
-    T *scs = nullptr, *scl = nullptr;
-    e = cudaMalloc(&scs, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&scl, fb);
-    if (e != cudaSuccess) {
-        if (scs) cudaFree(scs);
-        cudaGetLastError();
-        err = "device allocation failed";
-        return PF_ENOMEM;
-    }
+    if (D.energy_every > 0)
+        e = cudaMemsetAsync(B.energy, 0xff, (size_t)N * B.energy_slots * sizeof(double), main);
     std::vector<BatchState> hs(N);
     for (int i = 0; i < N; ++i) {
         hs[i] = BatchState{B.off[i], (int)D.n[i], 0, 0, 0, 0.0, 0.0, 0.0, 0.0};
     }
-    e = cudaMemcpyAsync(B.phi, D.phi0, fb, cudaMemcpyHostToDevice, main);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(B.phi, D.phi0, fb, cudaMemcpyHostToDevice, main);
     if (e == cudaSuccess) e = cudaMemcpyAsync(scs, D.cs0, fb, cudaMemcpyHostToDevice, main);
     if (e == cudaSuccess) e = cudaMemcpyAsync(scl, D.cl0, fb, cudaMemcpyHostToDevice, main);
     if (e == cudaSuccess) e = cudaMemcpyAsync(B.st, hs.data(), N * sizeof(BatchState), cudaMemcpyHostToDevice, main);
@@ -899,9 +934,6 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         batch_to_state<T><<<1216, 256, 0, main>>>(scs, scl, B.phi, B.c, B.d, B.total, D.params.interp, D.params.a);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(main);
-    cudaFree(scs);
-    cudaFree(scl);
     if (e == cudaSuccess) e = set_smem_limits<T>(&B.max_dyn, &B.sms);
     if (e == cudaSuccess) {
         int64_t nbig = 0;
@@ -972,18 +1004,21 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         return PF_ECUDA;
     }
 
-    // capture a chunk of launches as a CUDA graph and replay it
+    // capture a chunk of launches as a CUDA graph and replay it; a run of fewer than
+    // two chunks launches them directly (the capture costs more than it saves)
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    e = cudaStreamBeginCapture(main, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) e = B.issue((int)D.steps_per_launch, D.launches_per_graph);
-    cudaError_t e2 = cudaStreamEndCapture(main, &graph);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
-    if (e != cudaSuccess) {
-        if (graph) cudaGraphDestroy(graph);
-        err = std::string("batch graph: ") + cudaGetErrorString(e);
-        return PF_ECUDA;
+    if (D.max_steps / D.launches_per_graph >= 2 * D.steps_per_launch) {
+        e = cudaStreamBeginCapture(main, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) e = B.issue((int)D.steps_per_launch, D.launches_per_graph);
+        cudaError_t e2 = cudaStreamEndCapture(main, &graph);
+        if (e == cudaSuccess) e = e2;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
+        if (e != cudaSuccess) {
+            if (graph) cudaGraphDestroy(graph);
+            err = std::string("batch graph: ") + cudaGetErrorString(e);
+            return PF_ECUDA;
+        }
     }
     const int64_t per_replay = D.steps_per_launch * D.launches_per_graph;
     B.launches = 0;
@@ -996,7 +1031,8 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         const bool whole = left >= per_replay;
         e = cudaEventRecord(B.t0, main);
         if (whole) {
-            if (e == cudaSuccess) e = cudaGraphLaunch(exec, main);
+            if (e == cudaSuccess)
+                e = exec ? cudaGraphLaunch(exec, main) : B.issue((int)D.steps_per_launch, D.launches_per_graph);
         } else {
             for (int64_t r = left; r > 0 && e == cudaSuccess; r -= D.steps_per_launch)
                 e = B.issue((int)std::min<int64_t>(r, D.steps_per_launch));
@@ -1008,15 +1044,15 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         float ms = 0;
         cudaEventElapsedTime(&ms, B.t0, B.t1);
         total_ms += ms;
-        if (whole) B.launches += (int64_t)D.launches_per_graph * (int64_t)B.groups.size();
+        if (whole && exec) B.launches += (int64_t)D.launches_per_graph * (int64_t)B.groups.size();
         done_steps += whole ? per_replay : left;
         bool all = true;
         for (int i = 0; i < N; ++i)
             if (!hs[i].converged) all = false;
         if (all || done_steps >= D.max_steps) break;
     }
-    cudaGraphExecDestroy(exec);
-    cudaGraphDestroy(graph);
+    if (exec) cudaGraphExecDestroy(exec);
+    if (graph) cudaGraphDestroy(graph);
     if (e != cudaSuccess) {
         err = std::string("batch run: ") + cudaGetErrorString(e);
         return PF_ECUDA;
@@ -1041,19 +1077,12 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         }
     }
     if (R->phi && R->cs && R->cl) {
-        T *ocs = nullptr, *ocl = nullptr;
-        e = cudaMalloc(&ocs, fb);
-        if (e == cudaSuccess) e = cudaMalloc(&ocl, fb);
-        if (e == cudaSuccess) {
-            batch_from_state<T><<<1216, 256, 0, main>>>(B.phi, B.c, B.d, ocs, ocl, B.total, D.params.interp, D.params.a);
-            e = cudaGetLastError();
-        }
+        batch_from_state<T><<<1216, 256, 0, main>>>(B.phi, B.c, B.d, scs, scl, B.total, D.params.interp, D.params.a);
+        e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(R->phi, B.phi, fb, cudaMemcpyDeviceToHost, main);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(R->cs, ocs, fb, cudaMemcpyDeviceToHost, main);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(R->cl, ocl, fb, cudaMemcpyDeviceToHost, main);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(R->cs, scs, fb, cudaMemcpyDeviceToHost, main);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(R->cl, scl, fb, cudaMemcpyDeviceToHost, main);
         if (e == cudaSuccess) e = cudaStreamSynchronize(main);
-        if (ocs) cudaFree(ocs);
-        if (ocl) cudaFree(ocl);
         if (e != cudaSuccess) {
             err = std::string("batch fields: ") + cudaGetErrorString(e);
             return PF_ECUDA;
@@ -1242,27 +1271,19 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
     B.deriv = true;
     V *vphi = nullptr, *vcs = nullptr, *vcl = nullptr, *vc = nullptr, *vd = nullptr, *vlow = nullptr;
     double* dout = nullptr;
-    cudaError_t e = cudaMalloc(&B.phi, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.c, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.d, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&B.st, M * sizeof(BatchState));
-    if (e == cudaSuccess) e = cudaMalloc(&B.dv, M * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&B.ddt, M * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&vphi, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&vcs, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&vcl, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&vc, vb);
-    if (e == cudaSuccess) e = cudaMalloc(&vd, vb);
-    if (e == cudaSuccess && sizeof(V) == 4) e = cudaMalloc(&vlow, 3 * vb);
-    if (e == cudaSuccess && sizeof(V) == 4) e = cudaMalloc(&B.low, 3 * (size_t)B.total * sizeof(V));
-    if (e == cudaSuccess) e = cudaMalloc(&dout, 2 * M * sizeof(double));
-    auto free_tmp = [&] {
-        void* ptrs[] = {vphi, vcs, vcl, vc, vd, vlow, dout};
-        for (void* p : ptrs)
-            if (p) cudaFree(p);
-    };
+    for (T** p : {&B.phi, &B.c, &B.d}) B.mem.add(p, fb);
+    B.mem.add(&B.st, M * sizeof(BatchState));
+    B.mem.add(&B.dv, M * sizeof(double));
+    B.mem.add(&B.ddt, M * sizeof(double));
+    B.mem.add(&B.ids, M * sizeof(int));
+    for (V** p : {&vphi, &vcs, &vcl, &vc, &vd}) B.mem.add(p, vb);
+    if (sizeof(V) == 4) {
+        B.mem.add(&vlow, 3 * vb);
+        B.mem.add(&B.low, 3 * (size_t)B.total * sizeof(V));
+    }
+    B.mem.add(&dout, 2 * M * sizeof(double));
+    cudaError_t e = B.mem.allocate();
     if (e != cudaSuccess) {
-        free_tmp();
         cudaGetLastError();
         err = std::string("device allocation failed: ") + cudaGetErrorString(e);
         return PF_ENOMEM;
@@ -1285,7 +1306,6 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
         int64_t nbig = 0;
         for (int i = 0; i < N; ++i) nbig = std::max(nbig, (int64_t)D.n[i]);
         if ((size_t)6 * (nbig + 34 * batch_jmax<T>()) * sizeof(T) > B.max_dyn) {   // a copy's padding included
-            free_tmp();
             err = "longest instance does not fit in shared memory";
             return PF_EINVAL;
         }
@@ -1309,7 +1329,6 @@ static int run_adjoint_T(const pf_adjoint_desc& A, pf_adjoint_result* R, cudaStr
     if (e == cudaSuccess) e = cudaStreamSynchronize(main);
     float ms = 0;
     if (e == cudaSuccess) cudaEventElapsedTime(&ms, B.t0, B.t1);
-    free_tmp();
     if (e != cudaSuccess) {
         err = std::string("adjoint run: ") + cudaGetErrorString(e);
         return PF_ECUDA;
@@ -1908,29 +1927,19 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
     V *scs = nullptr, *scl = nullptr, *rec = nullptr, *lphi = nullptr, *lc = nullptr, *ld = nullptr;
     double *grad = nullptr, *cmax = nullptr;
     int* imax = nullptr;
-    auto free_tmp = [&] {
-        void* ptrs[] = {scs, scl, rec, lphi, lc, ld, grad, cmax, imax};
-        for (void* p : ptrs)
-            if (p) cudaFree(p);
-    };
-    cudaError_t e = cudaMalloc(&B.phi, fb * slots);
-    if (e == cudaSuccess) e = cudaMalloc(&B.c, fb * slots);
-    if (e == cudaSuccess) e = cudaMalloc(&B.d, fb * slots);
-    if (e == cudaSuccess && sizeof(V) == 4) e = cudaMalloc(&B.low, 3 * fb * slots);
-    if (e == cudaSuccess) e = cudaMalloc(&B.st, N * slots * sizeof(BatchState));
-    if (e == cudaSuccess) e = cudaMalloc(&B.dv, N * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&B.ddt, N * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&scs, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&scl, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&rec, fb * 6 * seg * 2);
-    if (e == cudaSuccess) e = cudaMalloc(&lphi, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&lc, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&ld, fb);
-    if (e == cudaSuccess) e = cudaMalloc(&grad, 3 * N * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&cmax, N * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&imax, N * sizeof(int));
+    for (V** p : {&B.phi, &B.c, &B.d}) B.mem.add(p, fb * slots);
+    if (sizeof(V) == 4) B.mem.add(&B.low, 3 * fb * slots);
+    B.mem.add(&B.st, N * slots * sizeof(BatchState));
+    B.mem.add(&B.dv, N * sizeof(double));
+    B.mem.add(&B.ddt, N * sizeof(double));
+    B.mem.add(&B.ids, N * sizeof(int));
+    for (V** p : {&scs, &scl, &lphi, &lc, &ld}) B.mem.add(p, fb);
+    B.mem.add(&rec, fb * 6 * seg * 2);
+    B.mem.add(&grad, 3 * N * sizeof(double));
+    B.mem.add(&cmax, N * sizeof(double));
+    B.mem.add(&imax, N * sizeof(int));
+    cudaError_t e = B.mem.allocate();
     if (e != cudaSuccess) {
-        free_tmp();
         cudaGetLastError();
         err = std::string("device allocation failed: ") + cudaGetErrorString(e);
         return PF_ENOMEM;
@@ -1962,12 +1971,10 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
     const int rroom = (int)(rper * RUSE + 4);
     const size_t rsmem = (size_t)6 * rroom * sizeof(V);
     if (e == cudaSuccess && rsmem > max_rev) {
-        free_tmp();
         err = "longest instance does not fit in shared memory for the reverse sweep";
         return PF_EINVAL;
     }
     if (e == cudaSuccess && (size_t)6 * (nmax + 34 * batch_jmax<V>()) * sizeof(V) > B.max_dyn) {
-        free_tmp();
         err = "longest instance does not fit in shared memory";
         return PF_EINVAL;
     }
@@ -2068,7 +2075,6 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
     if (e == cudaSuccess) e = cudaStreamSynchronize(main);
     float ms = 0;
     if (e == cudaSuccess) cudaEventElapsedTime(&ms, B.t0, B.t1);
-    free_tmp();
     if (e != cudaSuccess) {
         err = std::string("reverse adjoint run: ") + cudaGetErrorString(e);
         return PF_ECUDA;
