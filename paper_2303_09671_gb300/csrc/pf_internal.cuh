@@ -65,6 +65,7 @@ __host__ __device__ inline void set_coefficients(Consts<T>& C) {
 template <typename T>
 struct Clock {
     T theta0;   // see Consts::G_theta
+    double theta0_exact;
 };
 
 // Map a possibly-ghost coordinate onto the interior (noflux: mirror about

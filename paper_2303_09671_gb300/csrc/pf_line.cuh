@@ -364,11 +364,7 @@ PF_D void line_face(const LineConsts<E>& K, X fL, X fR, X YL, X YR, X sL, X sR, 
 }
 
 // whether a parameter set is one for STD
-inline bool line_std(const HostProblem& P) {
-    auto in = [](double v) { return v >= 1e-10 && v <= 1e10; };
-    return P.interp == 0 && P.mobility == 0 && P.a == 0.0 && P.delta * P.dx >= 1e-8 && P.delta * P.dx <= 1e8 &&
-           in(P.D_s * P.k_e * P.c_inf) && in(P.D_l * P.c_inf) && in(P.b);
-}
+inline bool line_std(const HostProblem& P) { return std_physics(P) && P.a == 0.0; }
 
 // parameters, with the derivative 1 along one of (1/M_phi by M_phi, A, b) if dir >= 0
 template <typename E>

@@ -520,7 +520,8 @@ template <typename T>
 static Clock<T> make_clock(const HostProblem& P, int64_t step, int64_t shifts) {
     const double t = (double)step * P.dt;
     Clock<T> K;
-    K.theta0 = T(P.theta_ref + P.G_theta * (P.x0 + P.v_pull * t - (double)shifts * P.dx));
+    K.theta0_exact = P.theta_ref + P.G_theta * (P.x0 + P.v_pull * t - (double)shifts * P.dx);
+    K.theta0 = T(K.theta0_exact);
     return K;
 }
 

@@ -51,7 +51,7 @@ struct PTile2 {
     static constexpr size_t BYTES = OFF_FY + sizeof(V) * (TYP + 1) * TX;
 };
 
-template <typename T, int TX, int TY, bool HELP, bool L9, bool AI>
+template <typename T, int TX, int TY, bool HELP, bool L9, bool AI, bool STD>
 __global__ void __launch_bounds__(TX * (TY / 2) + (HELP ? 64 : 0), sizeof(T) == 4 ? 3 : 1)
 step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T* __restrict__ d_in,
               const T* __restrict__ clo_in, T* __restrict__ phi_out, T* __restrict__ c_out,
@@ -119,7 +119,7 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
             }
         }
         const V f = vpair(f2[0], f2[1]), c = vpair(c2[0], c2[1]), d = vpair(d2[0], d2[1]);
-        const V p = vp_of<AI>(K, f);
+        const V p = vp_of<AI, STD>(K, f);
         const V cs = vfma(vsub(vlit<V>(1.0), p), d, c);
         const V cl = vsub(c, vmul(p, d));
         const V mus = vsub(vlog(cs), K.log_ke);
@@ -161,32 +161,11 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
         const V gx = vsub(fxp, fxm), gy = vpair(f.y - fS.y, fN.x - f.x);
         const V sx = vsub(bxp.a, bxm.a), sy = vpair(bc.a.y - bS.a.y, bN.a.x - bc.a.x);
         const V lx = vsub(bxp.b, bxm.b), ly = vpair(bc.b.y - bS.b.y, bN.b.x - bc.b.x);
-        const V cs = cc.a, cl = cc.b, mus = bc.a, mul = bc.b;
-        const V p = vp_of<AI>(K, f), dp = vdp_of<AI>(K, f);
-        const V omp = vsub(vlit<V>(1.0), p);
-        const V Ms = vfma(K.Ms_c, cs, K.Ms_0), Ml = vfma(K.Ml_c, cl, K.Ml_0);
-        const V bMl = vmul(K.b, Ml);
-        const V Msq = vmul(Ms, omp);
-        const V iMbar = vrcp(vfma(bMl, p, Msq));
-        const V d = vsub(cs, cl);
         const V g2 = vfma(gx, gx, vmul(gy, gy));
-        const V cross = vsub(vmul(Ms, vfma(sx, gx, vmul(sy, gy))), vmul(bMl, vfma(lx, gx, vmul(ly, gy))));
-        const V rr = vrcp(vadd(g2, K.delta2_4dx2));
-        const V pq = vmul(p, omp);
-        const V Kc = vfma(K.K_anti, vmul(vmul(vmul(d, d), vmul(pq, rr)), vmul(iMbar, vrcp(vfma(K.b, p, omp)))),
-                          K.inv_Mphi);
-        const T th_s = G.theta0 - G.G_theta * xc;
-        const V theta = vpair(th_s, th_s);
-        const V dmu = vsub(mus, mul);
-        // D = [M_s (1-p)(1 - A(1-p)) + A b M_l p^2] / Mbar
-        const V Dd = vmul(vfma(Msq, vsub(vlit<V>(1.0), vmul(K.A, omp)), vmul(vmul(K.A, bMl), vmul(p, p))), iMbar);
-        // DeltaG = c_s (mu_s - mu_l) - d - (1-k_e) theta - D d (mu_s - mu_l)
-        const V dG = vsub(vsub(vmul(cs, dmu), d), vfma(K.one_m_ke, theta, vmul(vmul(Dd, d), dmu)));
-        const V g = vmul(f, vsub(vlit<V>(1.0), f));
-        const V dfdw = vmul(g, vsub(vlit<V>(2.0), vmul(vlit<V>(4.0), f)));
-        const V anti = vmul(vmul(vmul(K.one_m_A, d), vmul(pq, iMbar)), vmul(cross, rr));
-        const V R = vfma(K.sigma, lap, vmul(K.dx2, vsub(anti, vfma(K.H, dfdw, vmul(dG, dp)))));
-        sD[ry * RX + rx] = vmask(vmul(R, vrcp(Kc)), glo, ghi);
+        const V ds = vfma(sx, gx, vmul(sy, gy)), dl = vfma(lx, gx, vmul(ly, gy));
+        const T th = G.ke_theta0 - G.ke_G * xc;
+        sD[ry * RX + rx] = vmask(
+            cell_rate<AI, STD>(K, f, lap, g2, ds, dl, cc.a, cc.b, bc.a, bc.b, vpair(th, th)), glo, ghi);
     };
     if (owner) rate_cell(tx + 1, ty + 1);
     if (HELP ? extra >= 0 && extra < NB : tid >= NT - NB) {
@@ -214,7 +193,7 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
 #pragma unroll
         for (int k = 0; k < 4; ++k) t1[k] = vpair(SP[k].y - SS[k].y, SN[k].x - SP[k].x);
         const Q cL = sC[hL], cR = sC[hR];
-        face_flux<V, false, AI>(K, vmul(vlit<V>(0.5), SP[0]), vadd(cL.a, cR.a), vadd(cL.b, cR.b),
+        face_flux<V, false, AI, STD>(K, vmul(vlit<V>(0.5), SP[0]), vadd(cL.a, cR.a), vadd(cL.b, cR.b),
                             vadd(sD[rL], sD[rL + 1]), n, t1, t1, Fc, Fd);
     };
     // y faces above the two rows of the pair at hL: lanes (y+1/2, y+3/2)
@@ -238,7 +217,7 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
         const V f = vmul(vlit<V>(0.5), vpair(cP[0].x + cP[0].y, cP[0].y + cN[0].x));
         const V cs2 = vpair(cP_.a.x + cP_.a.y, cP_.a.y + cN_.a.x);
         const V cl2 = vpair(cP_.b.x + cP_.b.y, cP_.b.y + cN_.b.x);
-        face_flux<V, false, AI>(K, f, cs2, cl2, vpair(dP.x + dP.y, dP.y + dN.x), n, t1, t1, Fc, Fd);
+        face_flux<V, false, AI, STD>(K, f, cs2, cl2, vpair(dP.x + dP.y, dP.y + dN.x), n, t1, t1, Fc, Fd);
     };
     const bool nf_x = own_x == nx - 1 && G.bc_hi[0] == BC_NOFLUX;
     const bool nf_ylo = own_y == ny - 1 && G.bc_hi[1] == BC_NOFLUX;
@@ -309,10 +288,12 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
 template <typename T, int TX, int TY, bool HELP>
 static cudaError_t launch_tile2d(const StepLaunch& a, const Consts<T>& C, const Clock<T>& Kc) {
     using L = PTile2<T, TX, TY, HELP>;
-    // 9- or 5-point Laplacian x shape parameter a != 0 or a = 0
-    decltype(&step2d_kernel<T, TX, TY, HELP, true, true>) kerns[2][2] = {
-        {step2d_kernel<T, TX, TY, HELP, false, false>, step2d_kernel<T, TX, TY, HELP, false, true>},
-        {step2d_kernel<T, TX, TY, HELP, true, false>, step2d_kernel<T, TX, TY, HELP, true, true>}};
+    // default physics or not x 9- or 5-point Laplacian x shape parameter a != 0 or a = 0
+    decltype(&step2d_kernel<T, TX, TY, HELP, true, true, true>) kerns[2][2][2] = {
+        {{step2d_kernel<T, TX, TY, HELP, false, false, false>, step2d_kernel<T, TX, TY, HELP, false, true, false>},
+         {step2d_kernel<T, TX, TY, HELP, true, false, false>, step2d_kernel<T, TX, TY, HELP, true, true, false>}},
+        {{step2d_kernel<T, TX, TY, HELP, false, false, true>, step2d_kernel<T, TX, TY, HELP, false, true, true>},
+         {step2d_kernel<T, TX, TY, HELP, true, false, true>, step2d_kernel<T, TX, TY, HELP, true, true, true>}}};
     static DeviceSetup setup;
     {
         int dev = 0;
@@ -321,8 +302,8 @@ static cudaError_t launch_tile2d(const StepLaunch& a, const Consts<T>& C, const 
         if (dev < 0 || dev >= DeviceSetup::MAX_DEVICES) return cudaErrorInvalidDevice;
         std::lock_guard<std::mutex> lock(setup.mu);
         if (!setup.done[dev]) {
-            for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-                e = cudaFuncSetAttribute(kerns[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize,
+            for (int i = 0; i < 8 && e == cudaSuccess; ++i)
+                e = cudaFuncSetAttribute(kerns[i / 4][i / 2 % 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)L::BYTES);
             if (e != cudaSuccess) return e;
             setup.done[dev] = true;
@@ -333,7 +314,7 @@ static cudaError_t launch_tile2d(const StepLaunch& a, const Consts<T>& C, const 
     const GridConsts<T> G = make_grid_consts<T>(P, Kc);
     const dim3 block(L::THREADS);
     const dim3 grid((C.n[0] + TX - 1) / TX, (C.n[1] + TY - 1) / TY, 1);
-    auto kern = kerns[C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
+    auto kern = kerns[std_physics(P) ? 1 : 0][C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
     kern<<<grid, block, L::BYTES, a.stream>>>(
         static_cast<const T*>(a.phi_in), static_cast<const T*>(a.c_in), static_cast<const T*>(a.d_in),
         static_cast<const T*>(a.clo_in), static_cast<T*>(a.phi_out), static_cast<T*>(a.c_out),

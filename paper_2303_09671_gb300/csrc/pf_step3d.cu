@@ -386,35 +386,12 @@ step3d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
             const V gx = vsub(fxp, fxm), gy = vpair(f.y - fS.y, fN.x - f.x), gz = vsub(fzp, fzm);
             const V sx = vsub(bxp.a, bxm.a), sy = vpair(bc.a.y - bS.a.y, bN.a.x - bc.a.x), sz_ = vsub(bzp.a, bzm.a);
             const V lx = vsub(bxp.b, bxm.b), ly = vpair(bc.b.y - bS.b.y, bN.b.x - bc.b.x), lz = vsub(bzp.b, bzm.b);
-            const V cs = cc.a, cl = cc.b, mus = bc.a, mul = bc.b;
-            const V p = vp_of<AI, STD>(K, f), dp = vdp_of<AI, STD>(K, f);
-            const V omp = vsub(vlit<V>(1.0), p);
-            const V Ms = STD ? vmul(K.Ms_c, cs) : vfma(K.Ms_c, cs, K.Ms_0);
-            const V Ml = STD ? vmul(K.Ml_c, cl) : vfma(K.Ml_c, cl, K.Ml_0);
-            const V bMl = vmul(K.b, Ml);
-            const V Msq = vmul(Ms, omp);
-            const V iMbar = vrcp(vfma(bMl, p, Msq));
-            const V d = vsub(cs, cl);
             const V g2 = vfma(gx, gx, vfma(gy, gy, vmul(gz, gz)));
             const V ds = vfma(sx, gx, vfma(sy, gy, vmul(sz_, gz)));
             const V dl = vfma(lx, gx, vfma(ly, gy, vmul(lz, gz)));
-            const V cross = vsub(vmul(Ms, ds), vmul(bMl, dl));     // (M_s grad mu_s - b M_l grad mu_l).grad phi
-            const V rr = vrcp(vadd(g2, K.delta2_4dx2));
-            const V pq = vmul(p, omp);
-            const V Kc = vfma(K.K_anti, vmul(vmul(vmul(d, d), vmul(pq, rr)), vmul(iMbar, vrcp(vfma(K.b, p, omp)))),
-                              K.inv_Mphi);
-            const T th_s = G.theta0 - G.G_theta * xc;
-            const V theta = vpair(th_s, th_s);
-            const V dmu = vsub(mus, mul);
-            // D = [M_s (1-p)(1 - A(1-p)) + A b M_l p^2] / Mbar
-            const V Dd = vmul(vfma(Msq, vsub(vlit<V>(1.0), vmul(K.A, omp)), vmul(vmul(K.A, bMl), vmul(p, p))), iMbar);
-            // DeltaG = c_s (mu_s - mu_l) - d - (1-k_e) theta - D d (mu_s - mu_l)
-            const V dG = vsub(vsub(vmul(cs, dmu), d), vfma(K.one_m_ke, theta, vmul(vmul(Dd, d), dmu)));
-            const V g = vmul(f, vsub(vlit<V>(1.0), f));
-            const V dfdw = vmul(g, vsub(vlit<V>(2.0), vmul(vlit<V>(4.0), f)));
-            const V anti = vmul(vmul(vmul(K.one_m_A, d), vmul(pq, iMbar)), vmul(cross, rr));
-            const V R = vfma(K.sigma, lap, vmul(K.dx2, vsub(anti, vfma(K.H, dfdw, vmul(dG, dp)))));
-            pd = vmask(vmul(R, vrcp(Kc)), (dsc >> 12) & 1, (dsc >> 13) & 1);
+            const T th = G.ke_theta0 - G.ke_G * xc;
+            pd = vmask(cell_rate<AI, STD>(K, f, lap, g2, ds, dl, cc.a, cc.b, bc.a, bc.b, vpair(th, th)),
+                       (dsc >> 12) & 1, (dsc >> 13) & 1);
         }
         return pd;
     };
@@ -905,7 +882,7 @@ cudaError_t launch_step3d(const StepLaunch& a, const Consts<T>& C, const Clock<T
     Step3dKernel<T> kt[2][2][2];
     if (flags & 1) step3d_table<T, true>(kt);
     else step3d_table<T, false>(kt);
-    const bool std_phys = P.interp == 0 && P.mobility == 0;
+    const bool std_phys = std_physics(P);
     auto kern = kt[std_phys ? 1 : 0][C.lap == 19 ? 1 : 0][P.a != 0.0 ? 1 : 0];
     kern<<<grid, block, (flags & 1) ? L::BYTES : L::BYTES_CP, a.stream>>>(
         static_cast<const T*>(a.phi_in), static_cast<const T*>(a.c_in), static_cast<const T*>(a.d_in),

@@ -13,7 +13,7 @@ from conftest import rel_err
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [(3, 3), (16, 8), (17, 9), (15, 7), (33, 25), (304, 128), (305, 128), (40, 961)])
+@pytest.mark.parametrize("n", [(5, 4), (16, 8), (17, 9), (15, 7), (33, 25), (304, 128), (305, 128), (40, 961)])
 @pytest.mark.parametrize("kw", [dict(lap=9, bc_lo=("noflux", "periodic"), bc_hi=("noflux", "periodic")),
                                 dict(lap=5, a=0.2, bc_lo=("noflux", "noflux"), bc_hi=("dirichlet", "noflux"))])
 def test_fp64_tiles(n, kw):
