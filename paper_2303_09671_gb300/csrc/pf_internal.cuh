@@ -90,6 +90,35 @@ __device__ __forceinline__ int map_coord(int i, int n, int lo, int hi) {
     return m;
 }
 
+// Programmatic dependent launch: a kernel launched by launch_after may start as the
+// last blocks of the kernel before it in the stream end; it waits in grid_wait() for
+// that kernel's memory and touches none of it before.  The pointers pass through the
+// wait, so that no load through them (all are const __restrict__) is moved ahead of it.
+// A step follows the one before 1.5 to 4 us sooner than by a plain launch (which
+// starts on ticks of 2 us): FP32 2D, 64^2 6.2 -> 4.3 us per step, 1024^2 26.7 -> 24.1;
+// FP64 128^2 36.4 -> 33.4; 3D FP32 150 x 97 x 83 59.7 -> 57.5.  No kernel lets the
+// next one start earlier (griddepcontrol.launch_dependents): its waiting blocks then
+// gather on the SMs that are idle (FP64 128^2: 62 us).
+template <typename... P>
+__device__ __forceinline__ void grid_wait(P&... p) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ((void)([&] { asm volatile("" : "+l"(p)::"memory"); }()), ...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_after(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 __device__ __forceinline__ float flog(float x) { return logf(x); }
 __device__ __forceinline__ double flog(double x) { return log(x); }
 

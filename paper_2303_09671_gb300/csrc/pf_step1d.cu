@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(128) line_kernel(const __grid_constant__ LineA
 #pragma unroll
         for (int k = 0; k < H; ++k) x[k] = x_join<X>(w[k], w[(k + H) % J]);
     };
+    grid_wait();
     get(a.phi, a.K.gphi, s.phi);
     get(a.c, a.K.fc, s.c);
     get(a.d, a.K.fd, s.d);
@@ -227,9 +228,9 @@ cudaError_t line_run(const HostProblem& P, const LinePlan& pl, LineRun& r, int64
         a.m[a.steps] = (int)(shifts - r.shifts);
         a.erec = r.erec;
         line_state(a, r.buf[r.cur], r.store ? &r.buf[r.cur ^ 1] : nullptr);
-        if (std_phys) line_kernel<E, J, KS, true, COMP, ENERGY><<<blocks, 32 * pl.warps, 0, r.stream>>>(a);
-        else line_kernel<E, J, KS, false, COMP, ENERGY><<<blocks, 32 * pl.warps, 0, r.stream>>>(a);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_after(std_phys ? line_kernel<E, J, KS, true, COMP, ENERGY>
+                                                    : line_kernel<E, J, KS, false, COMP, ENERGY>,
+                                           dim3(blocks), dim3(32 * pl.warps), 0, r.stream, a);
         if (e != cudaSuccess) return e;
         r.erec += a.steps;
         if (r.store) {

@@ -85,6 +85,7 @@ step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
     const bool in_hi = owner && own_x < nx && own_y + 1 < ny;
     const long long own_xy = (long long)own_y * nx + own_x;
 
+    grid_wait(phi_in, c_in, d_in, clo_in);
     // own state for the update, in flight while the tile is converted
     T oc[2] = {T(0), T(0)}, od[2] = {T(0), T(0)}, olo[2] = {T(0), T(0)};
     if (in_lo) {
@@ -315,11 +316,11 @@ static cudaError_t launch_tile2d(const StepLaunch& a, const Consts<T>& C, const 
     const dim3 block(L::THREADS);
     const dim3 grid((C.n[0] + TX - 1) / TX, (C.n[1] + TY - 1) / TY, 1);
     auto kern = kerns[std_physics(P) ? 1 : 0][C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
-    kern<<<grid, block, L::BYTES, a.stream>>>(
+    return launch_after(
+        kern, grid, block, L::BYTES, a.stream,
         static_cast<const T*>(a.phi_in), static_cast<const T*>(a.c_in), static_cast<const T*>(a.d_in),
         static_cast<const T*>(a.clo_in), static_cast<T*>(a.phi_out), static_cast<T*>(a.c_out),
         static_cast<T*>(a.d_out), static_cast<T*>(a.clo_out), K, G);
-    return cudaGetLastError();
 }
 
 // 32 x 16 tiles.  FP64 grids that 16 x 8 tiles with helping warps fit in two per

@@ -122,6 +122,7 @@ step3d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T*
     Q* sFx = reinterpret_cast<Q*>(smem + L::OFF_FX) + L::OF;
     V* sFy = reinterpret_cast<V*>(smem + L::OFF_FY);
 
+    grid_wait(phi_in, c_in, d_in, clo_in);
     const int tid = threadIdx.x;
     const int tx = tid % TX, ty = tid / TX;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
@@ -884,12 +885,11 @@ cudaError_t launch_step3d(const StepLaunch& a, const Consts<T>& C, const Clock<T
     else step3d_table<T, false>(kt);
     const bool std_phys = std_physics(P);
     auto kern = kt[std_phys ? 1 : 0][C.lap == 19 ? 1 : 0][P.a != 0.0 ? 1 : 0];
-    kern<<<grid, block, (flags & 1) ? L::BYTES : L::BYTES_CP, a.stream>>>(
-        static_cast<const T*>(a.phi_in), static_cast<const T*>(a.c_in), static_cast<const T*>(a.d_in),
+    return launch_after(
+        kern, grid, block, (flags & 1) ? L::BYTES : L::BYTES_CP, a.stream, static_cast<const T*>(a.phi_in), static_cast<const T*>(a.c_in), static_cast<const T*>(a.d_in),
         static_cast<const T*>(a.clo_in), static_cast<T*>(a.phi_out), static_cast<T*>(a.c_out),
         static_cast<T*>(a.d_out), static_cast<T*>(a.clo_out), K, G, zchunk, zfirst, maps[0], maps[1], maps[2],
         maps[3], maps[4], maps[5], maps[6], maps[7], flags, zpad, a.err);
-    return cudaGetLastError();
 }
 
 // cuTensorMapEncodeTiled, looked up from the driver once per process
