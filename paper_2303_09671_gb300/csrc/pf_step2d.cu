@@ -24,6 +24,9 @@
 
 namespace pf {
 
+// the row-marching kernel of pf_march2d.cu; *taken = false: not for this grid
+cudaError_t launch_march2d(const StepLaunch& a, const Consts<float>& C, const Clock<float>& Kc, bool* taken);
+
 // HELP: 64 more threads that take the ring's border and the tile's low edge faces,
 // which are otherwise second tasks of the tile's own warps
 template <typename T, int TX, int TY, bool HELP>
@@ -347,6 +350,10 @@ cudaError_t launch_step2d(const StepLaunch& a, const Consts<T>& C, const Clock<T
         }
         const long long small = (long long)((C.n[0] + 15) / 16) * ((C.n[1] + 7) / 8);
         if (small <= 2 * sms) return launch_tile2d<T, 16, 8, true>(a, C, Kc);
+    } else {
+        bool taken = false;
+        const cudaError_t e = launch_march2d(a, C, Kc, &taken);
+        if (e != cudaSuccess || taken) return e;
     }
     return launch_tile2d<T, 32, 16, false>(a, C, Kc);
 }
