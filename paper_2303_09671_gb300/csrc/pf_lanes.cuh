@@ -191,7 +191,7 @@ __device__ __forceinline__ void face_flux(const PairConsts<V>& K, V f, V cs2, V 
 // kk/u) = R u / (u/M_phi + kk).  In FP64, where an operation costs 18 issue slots
 // and a reciprocal several operations, one reciprocal t = 1/(Mbar G), G = g2 + 4
 // delta^2 dx^2, serves 1/Mbar = t G as well (2D 128^2: 38.5 -> 36.4 us per step, 3D
-// 96^3: 398.8 -> 389.7); FP32 is not bound by its arithmetic and takes two side by
+// 96^3: 997 -> 974); FP32 is not bound by its arithmetic and takes two side by
 // side.
 template <bool AI, bool STD, typename V>
 __device__ __forceinline__ V cell_rate(const PairConsts<V>& K, V f, V lap, V g2, V ds, V dl, V cs, V cl, V mus, V mul,

@@ -14,7 +14,7 @@
 // fluxes), 500 instructions per 64 cells against 890 in the tile kernel, whose
 // phases also wait for one another at four barriers.  Three warps per scheduler
 // at 168 registers: four at 128 spill (1024^2: 26.7 us per step instead of 22.6),
-// two hide less (2048^2: 103 instead of 69), unrolling by two or three to rename
+// two hide less (2048^2: 107 instead of 70), unrolling by two or three to rename
 // the rows spills as well (2048^2: 106 and 93).  Per step, tile kernel and this
 // one: 1024^2 24.1 and 20.4 us, 2048^2 93.7 and 65.7 us.
 #include <algorithm>

@@ -10,7 +10,7 @@
 // where the line leaves SMs idle, 112 of 128 where it does not.  FP64 is bound by
 // the FP64 pipe of an SM, which issues one warp instruction in about 19 cycles:
 // a short line is spread with one cell per lane, 16 of 32 cells holding results.
-// Measured: 1.2 us per FP32 step (1000 cells), 8.1 us per FP64 step with its energy.
+// Measured: 1.45 us per FP32 step (1000 cells), 6.4 us per FP64 step with its energy.
 //
 // The energy of the state before each step is summed from the values the step
 // evaluates anyway (c_s, c_l, their potentials), per strip in a fixed order.

@@ -329,8 +329,9 @@ static cudaError_t launch_tile2d(const StepLaunch& a, const Consts<T>& C, const 
 // 32 x 16 tiles.  FP64 grids that 16 x 8 tiles with helping warps fit in two per
 // SM take those: the kernel is then bound by the latency of FP64 chains on few
 // warps (128^2: 82 us per step with 32 x 16 tiles, 37 with the small ones; 200 x
-// 160, 260 small tiles: 82 and 51; 256^2, 512 small tiles: 82 and 110).  In FP32
-// both take 6.2 us up to 256^2.
+// 160, 260 small tiles: 82 and 51; 256^2, 512 small tiles: 82 and 110; with today's
+// rate and launches the side taken has 32, 45 and 65 us).  In FP32 both take the
+// same time up to 256^2.
 template <typename T>
 cudaError_t launch_step2d(const StepLaunch& a, const Consts<T>& C, const Clock<T>& Kc) {
     if constexpr (sizeof(T) == 8) {
