@@ -364,7 +364,8 @@ typedef struct {
     double tol;                /* converged when |dk_v/dt| < tol ...                  */
     double min_travel;         /* ... and the temperature has been pulled >= min_travel
                                   (units of W), i.e. t >= min_travel / v */
-    int cells_per_thread;      /* 1, 2, 4 or 8; 0 = autotune */
+    int cells_per_thread;      /* 1, 2, 4 or 8 (at most the kernel's largest is used);
+                                  0 = autotune in long runs */
     int64_t energy_every;      /* > 0: record the free energy F_h (as pf_energy
                                   computes it) after every energy_every-th step,
                                   in FP64 inside the persistent launch; 0: none */
