@@ -12,6 +12,7 @@
 #include <cstdint>
 #include "pf_internal.cuh"
 #include "pf_kernels.h"
+#include "pf_words.cuh"
 
 namespace pf {
 
@@ -51,23 +52,15 @@ static int diag_blocks(long long items) {
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
-// An unevaluated sum of two floats, |l| at most half an ulp of h: about 48 bits.
 // The FP64 pipe of a GB300 runs at 1/77 of the FP32 rate, so the sums over FP32
-// states are formed in pairs (Knuth's TwoSum; products by FMA); each thread's
-// totals then enter the FP64 block reduction.
-struct Pair {
-    float h, l;
-};
-static Pair pair_of(double v) {
-    const float h = (float)v;
-    return {h, (float)(v - (double)h)};
-}
+// states are formed in three FP32 words (pf_words.cuh) for a few cells at a time
+// and added in FP64.
 
 struct DiagConsts {
     int n[3], bc_lo[3], bc_hi[3], dim, lap, interp;
     double dir_phi, dx, H, sigma, k_e, a, theta0, G_theta, dV;
-    // in pairs: 1 + ln k_e, k_e - 1, and those above that the FP32 sums use
-    Pair lk2, ke2, H2, th2, Gx2, a2, dir2;
+    // in FP32 words, for FP32 states: 1 + ln k_e, H, -(1 - k_e) theta = th + Gx (i + 1/2), a, dir_phi
+    Triple lk3, H3, th3, Gx3, a3, dir3;
 };
 
 __device__ __forceinline__ double p_d(const DiagConsts& C, double f) {
@@ -102,86 +95,6 @@ __device__ void block_reduce2(double& a, double& b) {
     }
 }
 
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-// ------------------------------------------------------ FP32 pairs
-__device__ __forceinline__ Pair quick_sum(float a, float b) {   // |a| >= |b| or a = 0
-    const float s = a + b;
-    return {s, b - (s - a)};
-}
-__device__ __forceinline__ Pair sum2(float a, float b) {
-    float s, e;
-    two_sum(a, b, s, e);
-    return {s, e};
-}
-__device__ __forceinline__ Pair prod2(float a, float b) {
-    const float p = __fmul_rn(a, b);
-    return {p, __fmaf_rn(a, b, -p)};
-}
-__device__ __forceinline__ Pair operator+(Pair a, Pair b) {
-    const Pair s = sum2(a.h, b.h);
-    return quick_sum(s.h, s.l + (a.l + b.l));
-}
-__device__ __forceinline__ Pair operator-(Pair a) { return {-a.h, -a.l}; }
-__device__ __forceinline__ Pair operator-(Pair a, Pair b) { return a + (-b); }
-__device__ __forceinline__ Pair operator*(Pair a, Pair b) {
-    const Pair p = prod2(a.h, b.h);
-    return quick_sum(p.h, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, p.l)));
-}
-__device__ __forceinline__ Pair operator*(Pair a, float b) {
-    const Pair p = prod2(a.h, b);
-    return quick_sum(p.h, __fmaf_rn(a.l, b, p.l));
-}
-
-// ln of a pair to about 2^-48: x = 2^e m, a 9-bit approximation r of 1/m from a
-// table of 128 (with -ln r as a pair), z = m r - 1 exactly, |z| < 2^-7, and the
-// series of ln(1 + z) with its first two terms as pairs.  NaN where x is not a
-// positive normal number.
-struct LogTable {
-    float r[128], h[128], l[128];
-    LogTable() = default;
-    explicit LogTable(int) {
-        for (int t = 0; t < 128; ++t) {
-            const double q = std::rint(512.0 / (1.0 + (t + 0.5) / 128.0)) / 512.0;   // 9 bits
-            const Pair v = pair_of(-std::log(q));
-            r[t] = (float)q;
-            h[t] = v.h;
-            l[t] = v.l;
-        }
-    }
-};
-__device__ __forceinline__ Pair ln_pair(const LogTable& T, Pair x) {
-    if (!(x.h >= 1.17549435e-38f && x.h <= 3.402823466e38f)) return {NAN, 0.0f};
-    const int b = __float_as_int(x.h);
-    const int e = (b >> 23) - 127, t = (b >> 16) & 127;
-    const float m = __int_as_float((b & 0x007fffff) | 0x3f800000);
-    const float ml = __fmul_rn(__fmul_rn(x.l, __int_as_float((127 - e / 2) << 23)),
-                               __int_as_float((127 - (e - e / 2)) << 23));   // x.l 2^-e
-    const float r = T.r[t], ef = (float)e;
-    const Pair p = prod2(m, r);
-    const Pair z = quick_sum(p.h - 1.0f, __fmaf_rn(ml, r, p.l));
-    const float zz = z.h;
-    // ln 2 in parts of 14, 14 and 24 bits: e times the first two is exact
-    const float L1 = 0.693115234375f, L2 = 3.194436430931e-05f, L3 = 1.820635999e-09f;
-    Pair q = prod2(zz, zz);
-    q = {-0.5f * q.h, -__fmaf_rn(zz, z.l, 0.5f * q.l)};
-    const float c = zz * zz * zz *
-                    __fmaf_rn(zz, __fmaf_rn(zz, __fmaf_rn(zz, __fmaf_rn(zz, 1.0f / 7, -1.0f / 6), 0.2f), -0.25f),
-                              1.0f / 3);
-    Pair s = sum2(ef * L1, T.h[t]);
-    Pair a = sum2(s.h, zz);
-    float lo = s.l + a.l;
-    s = sum2(a.h, ef * L2);
-    lo += s.l;
-    a = sum2(s.h, q.h);
-    lo += a.l + (__fmaf_rn(ef, L3, T.l[t]) + (z.l + q.l) + c);
-    return quick_sum(a.h, lo);
-}
-
 // state accessors: c (with its FP32 low word), d -> c_s, c_l in FP64
 template <typename T>
 struct StateView {
@@ -204,12 +117,12 @@ struct StateView {
         s = cc + (1.0 - p) * dd;
         l = cc - p * dd;
     }
-    // total c, c_s and c_l of cell i as FP32 pairs, from its p
-    __device__ __forceinline__ void cell32(long long i, Pair p, Pair& cc, Pair& s, Pair& l) const {
-        cc = {(float)c[i], clo ? (float)clo[i] : 0.0f};
+    // total c, c_s and c_l of cell i in FP32 words, from its p
+    __device__ __forceinline__ void cell32(long long i, Triple p, Triple& cc, Triple& s, Triple& l) const {
+        cc = {(float)c[i], clo ? (float)clo[i] : 0.0f, 0.0f};
         const float dd = (float)d[i];
         l = cc - p * dd;
-        s = l + Pair{dd, 0.0f};
+        s = l + dd;
     }
 };
 
@@ -228,10 +141,10 @@ struct FieldView {
         p = p_d(C, f);
         cc = p * s + (1.0 - p) * l;   // Eq. model1 with g = p
     }
-    __device__ __forceinline__ void cell32(long long i, Pair p, Pair& cc, Pair& s, Pair& l) const {
-        s = {(float)cs[i], 0.0f};
-        l = {(float)cl[i], 0.0f};
-        cc = l + p * (s - l);
+    __device__ __forceinline__ void cell32(long long i, Triple p, Triple& cc, Triple& s, Triple& l) const {
+        s = {(float)cs[i], 0.0f, 0.0f};
+        l = {(float)cl[i], 0.0f, 0.0f};
+        cc = p * widen(sum2(s.h, -l.h)) + l.h;
     }
 };
 
@@ -254,6 +167,11 @@ struct SquareSum<float> {
         l += s.l + weight * __fmaf_rn(2.0f * d.h, d.l, p.l);
     }
     __device__ __forceinline__ void add(float v, float f, float weight) { add(sum2(v, -f), weight); }
+    __device__ __forceinline__ void settle() {   // after a cell: a small l is added to with small errors
+        const Pair s = sum2(h, l);
+        h = s.h;
+        l = s.l;
+    }
     __device__ __forceinline__ double total() const { return (double)h + (double)l; }
 };
 
@@ -284,9 +202,9 @@ struct Cursor {
 // a square in 2D).  A pair of cells of the grid is added once, by its lower cell;
 // a pair with a ghost beyond a mirror, Dirichlet or halo side belongs to one cell
 // only and counts half.
-template <int LAP, typename T>
+template <int LAP, typename T, typename S>
 __device__ __forceinline__ void gradient_pairs(const DiagConsts& C, const T* __restrict__ phi, long long c, int i,
-                                               int j, int k, T f, SquareSum<T>& s1, SquareSum<T>& s2) {
+                                               int j, int k, T f, SquareSum<S>& s1, SquareSum<S>& s2) {
     constexpr int DIM = LAP == 3 ? 1 : LAP <= 9 && LAP != 7 ? 2 : 3;
     constexpr bool DIAG = LAP == 9 || LAP == 19;
     const int nx = C.n[0], ny = C.n[1], nz = C.n[2];
@@ -301,7 +219,7 @@ __device__ __forceinline__ void gradient_pairs(const DiagConsts& C, const T* __r
     const long long yp = j < ny - 1 ? oy : -(ny - 1) * oy, ym = j > 0 ? -oy : (ny - 1) * oy;
     const long long zp = k < nz - 1 ? oz : -(nz - 1) * oz;
     const T* q = phi + c;
-    const T one = T(1);
+    const S one = S(1);
     s1.add(px ? q[xp] : f, f, one);
     if constexpr (DIM >= 2) s1.add(py ? q[yp] : f, f, one);
     if constexpr (DIM == 3) s1.add(pz ? q[zp] : f, f, one);
@@ -322,11 +240,11 @@ __device__ __forceinline__ void gradient_pairs(const DiagConsts& C, const T* __r
     // column, so only its edge neighbours differ.
     if (yz && (px || C.bc_hi[0] == BC_NOFLUX) && (mx || C.bc_lo[0] == BC_NOFLUX)) {
         if constexpr (DIAG) {
-            s2.add(q[yp], f, T(0.5));
-            s2.add(q[ym], f, T(0.5));
+            s2.add(q[yp], f, S(0.5));
+            s2.add(q[ym], f, S(0.5));
             if constexpr (DIM == 3) {
-                s2.add(q[zp], f, T(0.5));
-                s2.add(q[k > 0 ? -oz : (nz - 1) * oz], f, T(0.5));
+                s2.add(q[zp], f, S(0.5));
+                s2.add(q[k > 0 ? -oz : (nz - 1) * oz], f, S(0.5));
             }
         }
         return;
@@ -339,15 +257,18 @@ __device__ __forceinline__ void gradient_pairs(const DiagConsts& C, const T* __r
                 const bool in = (dx == 0 || (dx > 0 ? px : mx)) && (dy == 0 || (dy > 0 ? py : my)) &&
                                 (dz == 0 || (dz > 0 ? pz : mz));
                 if (in) continue;
-                SquareSum<T>& s = away == 1 ? s1 : s2;
+                SquareSum<S>& s = away == 1 ? s1 : s2;
                 const int mi = map_coord(i + dx, nx, C.bc_lo[0], C.bc_hi[0]);
                 const int mj = DIM >= 2 ? map_coord(j + dy, ny, C.bc_lo[1], C.bc_hi[1]) : 0;
                 const int mk = DIM == 3 ? map_coord(k + dz, nz, C.bc_lo[2], C.bc_hi[2]) : 0;
                 if (mi < 0 || mj < 0 || mk == DIR_GHOST) {
-                    if constexpr (sizeof(T) == 4) s.add(C.dir2 - Pair{f, 0.0f}, 0.5f);
+                    if constexpr (sizeof(S) == 4) {
+                        const Triple d = C.dir3 + -f;
+                        s.add(Pair{d.h, d.l}, 0.5f);
+                    }
                     else s.add(C.dir_phi, f, 0.5);
                 } else {
-                    s.add(phi[((long long)mk * ny + mj) * nx + mi], f, T(0.5));
+                    s.add(phi[((long long)mk * ny + mj) * nx + mi], f, S(0.5));
                 }
             }
 }
@@ -362,12 +283,18 @@ __device__ __forceinline__ double bulk_energy(const DiagConsts& C, double f, dou
     return C.H * fdw + p * fs + (1.0 - p) * fl;
 }
 
+// cells whose terms a thread sums in FP32 words before it adds them to its FP64 sums
+// (12 operations of the FP64 pipe; 2 % of the time of 32 cells)
+constexpr int ENERGY_RUN = 32;
+
 // F_h and S_h.  The FP64 form is bound by the FP64 pipe (two logarithms and the
-// pairs).  An FP32 state is summed in FP32 pairs: 256^3 in 0.53 ms, bound by
-// instruction issue (71 % of cycles; 490 FP32 operations per cell), against 5.9 ms
-// in FP64 arithmetic with each pair of neighbours taken twice; the result agrees
-// with FP64's to its last digits.  Threads whose FP32 totals are not finite (a concentration that is not
-// a positive normal number, an overflow) repeat their cells in FP64.
+// pairs).  The terms of an FP32 state's cells are formed in three FP32 words, which
+// leaves F_h as exact as FP64 arithmetic does (against extended precision, 48 states
+// of 3000 to 130,000 cells: 1e-16 rms either way, the last bit; with two words, whose
+// cells of equal value all repeat one rounding, 1.3e-15).  256^3: 0.74 ms, bound
+// by instruction issue; two words took 0.53, FP64 arithmetic with each pair of
+// neighbours taken twice 5.9.  Threads whose sums are not finite (a concentration
+// below ln_triple's range, an overflow) repeat their cells in FP64.
 template <int LAP, typename View, typename T>
 __global__ void __launch_bounds__(DIAG_THREADS, sizeof(T) == 4 ? 3 : 1)
 energy_kernel(View S, const T* __restrict__ phi, const DiagConsts C, const __grid_constant__ LogTable logs,
@@ -382,40 +309,42 @@ energy_kernel(View S, const T* __restrict__ phi, const DiagConsts C, const __gri
         __shared__ LogTable table;   // a copy that lanes read at different entries
         for (int t = threadIdx.x; t < 128; t += DIAG_THREADS) {
             table.r[t] = logs.r[t];
-            table.h[t] = logs.h[t];
-            table.l[t] = logs.l[t];
+            table.a[t] = logs.a[t];
+            table.b[t] = logs.b[t];
+            table.c[t] = logs.c[t];
+            table.d[t] = logs.d[t];
         }
         __syncthreads();
-        SquareSum<float> s1, s2;
-        Pair E = {0.0f, 0.0f}, Sc = {0.0f, 0.0f};
-        const Pair lk = C.lk2, ke = C.ke2, H = C.H2, th0 = C.th2, Gx = C.Gx2, ai = C.a2;
+        const Triple lk = C.lk3, H = C.H3, th = C.th3, Gx = C.Gx3, ai = C.a3;
         Cursor at(C, first, stride);
-        for (long long c = first; c < N; c += stride) {
-            const float f = phi[c];
-            gradient_pairs<LAP, float>(C, phi, c, at.i, at.j, at.k, f, s1, s2);
-            // p = h + a (f - 1/2) g^2, g = f (1 - f)
-            const Pair ff = prod2(f, f), omf = sum2(1.0f, -f);
-            Pair h;
-            if (C.interp == 1) h = ff * (Pair{3.0f, 0.0f} - sum2(f, f));
-            else h = (ff * f) * (Pair{10.0f, 0.0f} + (prod2(6.0f, f) - Pair{15.0f, 0.0f}) * f);
-            const Pair g = omf * f, gg = g * g;
-            Pair p = h;
-            if (C.a != 0.0) p = h + (ai * sum2(f, -0.5f)) * gg;
-            Pair cc, s, l;
-            S.cell32(c, p, cc, s, l);
-            const Pair fs0 = s * (ln_pair(table, s) - lk), fl = l * (ln_pair(table, l) - Pair{1.0f, 0.0f});
-            Pair theta = th0;
-            if (C.G_theta != 0.0) theta = th0 - Gx * sum2((float)(at.i & ~4095), (float)(at.i & 4095) + 0.5f);
-            const Pair fs = ke * theta + fs0;
-            const Pair e = (fl + p * (fs - fl)) + H * gg;
-            E = E + e;
-            Sc = Sc + cc;
-            at.next(C);
+        for (long long c = first; c < N && !exact;) {
+            SquareSum<float> s1, s2;
+            Triple E = {0.0f, 0.0f, 0.0f}, Sc = E;
+            for (int k = 0; k < ENERGY_RUN && c < N; ++k, c += stride) {
+                const float f = phi[c];
+                gradient_pairs<LAP>(C, phi, c, at.i, at.j, at.k, f, s1, s2);
+                s1.settle();
+                s2.settle();
+                // p = h + a (f - 1/2) g^2, g = f (1 - f)
+                const Triple ff = widen(prod2(f, f));
+                Triple p;
+                if (C.interp == 1) p = ff * widen(sum2(3.0f, -(f + f)));
+                else p = (ff * f) * ((widen(prod2(-15.0f, f)) + 10.0f) + ff * 6.0f);
+                const Triple g = widen(sum2(1.0f, -f)) * f, gg = g * g;
+                if (C.a != 0.0) p = p + (ai * widen(sum2(f, -0.5f))) * gg;
+                Triple cc, s, l;
+                S.cell32(c, p, cc, s, l);
+                const Triple fl = l * (ln_triple(table, l) + -1.0f);
+                Triple fs = s * (ln_triple(table, s) - lk) + th;
+                if (C.G_theta != 0.0) fs = fs + Gx * widen(sum2((float)(at.i & ~4095), (float)(at.i & 4095) + 0.5f));
+                E = E + ((fl + p * (fs - fl)) + H * gg);
+                Sc = Sc + cc;
+                at.next(C);
+            }
+            eS += value(Sc);
+            eF += value(E) + grad * (w1 * s1.total() + w2 * s2.total());
+            exact = !(isfinite(eF) && isfinite(eS));
         }
-        exact = !(isfinite(E.h) && isfinite(Sc.h) && isfinite(s1.h) && isfinite(s2.h) && isfinite(s1.l) &&
-                  isfinite(s2.l));
-        eS = (double)Sc.h + (double)Sc.l;
-        eF = (double)E.h + (double)E.l + grad * (w1 * s1.total() + w2 * s2.total());
     }
     if (exact) {
         SquareSum<double> s1, s2;
@@ -426,14 +355,7 @@ energy_kernel(View S, const T* __restrict__ phi, const DiagConsts C, const __gri
             double cc, f = 0.0, p = 0.0, s = 0.0, l = 0.0;
             S.template cell<true>(C, c, cc, f, p, s, l);
             eS += cc;
-            if constexpr (sizeof(T) == 8) {
-                gradient_pairs<LAP, double>(C, phi, c, at.i, at.j, at.k, f, s1, s2);
-            } else {
-                SquareSum<float> t1, t2;
-                gradient_pairs<LAP, float>(C, phi, c, at.i, at.j, at.k, phi[c], t1, t2);
-                s1.s += t1.total();
-                s2.s += t2.total();
-            }
+            gradient_pairs<LAP>(C, phi, c, at.i, at.j, at.k, phi[c], s1, s2);
             eF += bulk_energy(C, f, p, s, l, at.i, log_ke);
             at.next(C);
         }
@@ -784,13 +706,14 @@ static DiagConsts make_diag(const HostProblem& P, int64_t step, int64_t shifts) 
     C.theta0 = P.theta_ref + P.G_theta * (P.x0 + P.v_pull * t - (double)shifts * P.dx);
     C.G_theta = P.G_theta;
     C.dV = std::pow(P.dx, P.dim);
-    C.lk2 = pair_of(1.0 + std::log(P.k_e));
-    C.ke2 = pair_of(P.k_e - 1.0);
-    C.H2 = pair_of(P.H);
-    C.th2 = pair_of(C.theta0);
-    C.Gx2 = pair_of(P.G_theta * P.dx);
-    C.a2 = pair_of(P.a);
-    C.dir2 = pair_of(P.dir_phi);
+    const double log_ke = std::log(P.k_e), lk = 1.0 + log_ke;   // what its rounding leaves goes into the last word
+    C.lk3 = triple_of(lk);
+    C.lk3.t += (float)((1.0 - (lk - (lk - 1.0))) + (log_ke - (lk - 1.0)));
+    C.H3 = triple_of(P.H);
+    C.th3 = triple_of((P.k_e - 1.0) * C.theta0);
+    C.Gx3 = triple_of((1.0 - P.k_e) * P.G_theta * P.dx);
+    C.a3 = triple_of(P.a);
+    C.dir3 = triple_of(P.dir_phi);
     return C;
 }
 
