@@ -364,8 +364,10 @@ typedef struct {
     double tol;                /* converged when |dk_v/dt| < tol ...                  */
     double min_travel;         /* ... and the temperature has been pulled >= min_travel
                                   (units of W), i.e. t >= min_travel / v */
-    int cells_per_thread;      /* 1, 2, 4 or 8 (at most the kernel's largest is used);
-                                  0 = autotune in long runs */
+    int cells_per_thread;      /* 1, 2, 4 or 8 cells per lane of a warp's strip, taken to
+                                  the nearest that the kernels have (FP32: 2 and 4,
+                                  FP64: 2); instances hold at most 1024 times the
+                                  request.  0 = chosen, by timing in long runs */
     int64_t energy_every;      /* > 0: record the free energy F_h (as pf_energy
                                   computes it) after every energy_every-th step,
                                   in FP64 inside the persistent launch; 0: none */
@@ -382,7 +384,7 @@ typedef struct {
     void* phi;             /* optional (may be NULL): packed final fields, host */
     void* cs;
     void* cl;
-    int cells_per_thread;  /* the value used (autotuned or given) */
+    int cells_per_thread;  /* the cells per lane of the kernel that ran (2 or 4) */
     int64_t launches;      /* batch-kernel launches issued */
     double gpu_ms;         /* device time of the stepping (CUDA events) */
     double* energy;        /* optional (may be NULL), with energy_every > 0: host

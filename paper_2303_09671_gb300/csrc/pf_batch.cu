@@ -1064,7 +1064,7 @@ static int run_batch_T(const pf_batch_desc& D, pf_batch_result* R, cudaStream_t 
         if (R->steps) R->steps[i] = hs[i].step;
         if (R->converged) R->converged[i] = hs[i].converged == 1 ? 1 : 0;
     }
-    R->cells_per_thread = cpt;
+    R->cells_per_thread = B.J;
     R->launches = B.launches;
     R->gpu_ms = total_ms;
     if (R->energy && B.energy) {
