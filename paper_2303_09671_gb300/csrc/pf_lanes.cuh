@@ -230,11 +230,13 @@ __device__ __forceinline__ V cell_rate(const PairConsts<V>& K, V f, V lap, V g2,
 }
 
 // whether a parameter set is one for STD: the default physics (quintic h, M_i =
-// D_i c_i) with 1/(Mbar G) well inside FP32's range
-inline bool std_physics(const HostProblem& P) {
+// D_i c_i) and, where the kernel forms the product Mbar G (`product`: cell_rate in
+// FP64, the line kernels), 1/(Mbar G) well inside FP32's range
+inline bool std_physics(const HostProblem& P, bool product) {
+    if (P.interp != 0 || P.mobility != 0) return false;
     auto in = [](double v) { return v >= 1e-10 && v <= 1e10; };
-    return P.interp == 0 && P.mobility == 0 && P.delta * P.dx >= 1e-8 && P.delta * P.dx <= 1e8 &&
-           in(P.D_s * P.k_e * P.c_inf) && in(P.D_l * P.c_inf) && in(P.b);
+    return !product || (P.delta * P.dx >= 1e-8 && P.delta * P.dx <= 1e8 && in(P.D_s * P.k_e * P.c_inf) &&
+                        in(P.D_l * P.c_inf) && in(P.b));
 }
 
 // lane-wise zero

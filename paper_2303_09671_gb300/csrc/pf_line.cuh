@@ -364,7 +364,7 @@ PF_D void line_face(const LineConsts<E>& K, X fL, X fR, X YL, X YR, X sL, X sR, 
 }
 
 // whether a parameter set is one for STD
-inline bool line_std(const HostProblem& P) { return std_physics(P) && P.a == 0.0; }
+inline bool line_std(const HostProblem& P) { return std_physics(P, true) && P.a == 0.0; }
 
 // parameters, with the derivative 1 along one of (1/M_phi by M_phi, A, b) if dir >= 0
 template <typename E>

@@ -243,7 +243,7 @@ cudaError_t launch_march2d(const StepLaunch& a, const Consts<float>& C, const Cl
          {march2d_kernel<true, false, false>, march2d_kernel<true, true, false>}},
         {{march2d_kernel<false, false, true>, march2d_kernel<false, true, true>},
          {march2d_kernel<true, false, true>, march2d_kernel<true, true, true>}}};
-    auto kern = kerns[std_physics(P) ? 1 : 0][C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
+    auto kern = kerns[std_physics(P, false) ? 1 : 0][C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
     bool even = C.n[0] % 2 == 0;   // rows start on 8-byte boundaries in every array
     for (const void* q : {a.phi_in, a.c_in, a.d_in, a.clo_in, (const void*)a.phi_out, (const void*)a.c_out,
                           (const void*)a.d_out, (const void*)a.clo_out})

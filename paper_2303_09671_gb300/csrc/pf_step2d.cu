@@ -318,7 +318,7 @@ static cudaError_t launch_tile2d(const StepLaunch& a, const Consts<T>& C, const 
     const GridConsts<T> G = make_grid_consts<T>(P, Kc);
     const dim3 block(L::THREADS);
     const dim3 grid((C.n[0] + TX - 1) / TX, (C.n[1] + TY - 1) / TY, 1);
-    auto kern = kerns[std_physics(P) ? 1 : 0][C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
+    auto kern = kerns[std_physics(P, sizeof(T) == 8) ? 1 : 0][C.lap == 9 ? 1 : 0][P.a != 0.0 ? 1 : 0];
     return launch_after(
         kern, grid, block, L::BYTES, a.stream,
         static_cast<const T*>(a.phi_in), static_cast<const T*>(a.c_in), static_cast<const T*>(a.d_in),

@@ -883,7 +883,7 @@ cudaError_t launch_step3d(const StepLaunch& a, const Consts<T>& C, const Clock<T
     Step3dKernel<T> kt[2][2][2];
     if (flags & 1) step3d_table<T, true>(kt);
     else step3d_table<T, false>(kt);
-    const bool std_phys = std_physics(P);
+    const bool std_phys = std_physics(P, sizeof(T) == 8);
     auto kern = kt[std_phys ? 1 : 0][C.lap == 19 ? 1 : 0][P.a != 0.0 ? 1 : 0];
     return launch_after(
         kern, grid, block, (flags & 1) ? L::BYTES : L::BYTES_CP, a.stream, static_cast<const T*>(a.phi_in), static_cast<const T*>(a.c_in), static_cast<const T*>(a.d_in),
