@@ -93,7 +93,10 @@ __device__ __forceinline__ int map_coord(int i, int n, int lo, int hi) {
 // Programmatic dependent launch: a kernel launched by launch_after may start as the
 // last blocks of the kernel before it in the stream end; it waits in grid_wait() for
 // that kernel's memory and touches none of it before.  The pointers pass through the
-// wait, so that no load through them (all are const __restrict__) is moved ahead of it.
+// wait, so that no load through them is moved ahead of it; and as the kernel before may
+// still write the state while blocks of this one are resident, the state is not read-only
+// for the kernel's lifetime: its inputs carry no __restrict__ and are read by coherent
+// loads, never by ld.global.nc.
 // A step follows the one before 1.5 to 4 us sooner than by a plain launch (which
 // starts on ticks of 2 us): FP32 2D, 64^2 6.2 -> 4.3 us per step, 1024^2 26.7 -> 24.1;
 // FP64 128^2 36.4 -> 33.4; 3D FP32 150 x 97 x 83 59.7 -> 57.5.  No kernel lets the

@@ -41,7 +41,7 @@ __device__ __forceinline__ float2 from_left(float2 v) {    // v at x - 1
 
 __device__ __forceinline__ float word(const float* p, unsigned off) {
     float v;   // issued here, a row ahead of its use
-    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(reinterpret_cast<const char*>(p) + off));
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(reinterpret_cast<const char*>(p) + off));
     return v;
 }
 __device__ __forceinline__ void put(float* p, unsigned off, bool a, bool b, bool even, float2 v) {
@@ -56,10 +56,10 @@ __device__ __forceinline__ void put(float* p, unsigned off, bool a, bool b, bool
 
 template <bool L9, bool AI, bool STD>
 __global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_PER_SM / MARCH_WARPS)
-march2d_kernel(const float* __restrict__ phi_in, const float* __restrict__ c_in, const float* __restrict__ d_in,
-               const float* __restrict__ clo_in, float* __restrict__ phi_out, float* __restrict__ c_out,
-               float* __restrict__ d_out, float* __restrict__ clo_out, const PairConsts<float2> K,
-               const GridConsts<float> G, const int strips, const int rows, const bool even) {
+march2d_kernel(const float* phi_in, const float* c_in, const float* d_in, const float* clo_in,
+               float* __restrict__ phi_out, float* __restrict__ c_out, float* __restrict__ d_out,
+               float* __restrict__ clo_out, const PairConsts<float2> K, const GridConsts<float> G, const int strips,
+               const int rows, const bool even) {
     using V = float2;
     const int w = blockIdx.x * MARCH_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int nx = G.n[0], ny = G.n[1];

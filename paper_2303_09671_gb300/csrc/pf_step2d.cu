@@ -56,8 +56,8 @@ struct PTile2 {
 
 template <typename T, int TX, int TY, bool HELP, bool L9, bool AI, bool STD>
 __global__ void __launch_bounds__(TX * (TY / 2) + (HELP ? 64 : 0), sizeof(T) == 4 ? 3 : 1)
-step2d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T* __restrict__ d_in,
-              const T* __restrict__ clo_in, T* __restrict__ phi_out, T* __restrict__ c_out,
+step2d_kernel(const T* phi_in, const T* c_in, const T* d_in,
+              const T* clo_in, T* __restrict__ phi_out, T* __restrict__ c_out,
               T* __restrict__ d_out, T* __restrict__ clo_out, const PairConsts<typename Lanes<T>::V> K,
               const GridConsts<T> G) {
     using L = PTile2<T, TX, TY, HELP>;

@@ -97,8 +97,8 @@ __device__ __forceinline__ int slot3(int z) { return ((z % 3) + 3) % 3; }
 
 template <typename T, int TX, int TY, bool L19, bool AI, bool STD, bool TMA>
 __global__ void __launch_bounds__(TX * (TY / 2), (sizeof(T) == 4 ? 2 : 1))
-step3d_kernel(const T* __restrict__ phi_in, const T* __restrict__ c_in, const T* __restrict__ d_in,
-              const T* __restrict__ clo_in, T* __restrict__ phi_out, T* __restrict__ c_out,
+step3d_kernel(const T* phi_in, const T* c_in, const T* d_in,
+              const T* clo_in, T* __restrict__ phi_out, T* __restrict__ c_out,
               T* __restrict__ d_out, T* __restrict__ clo_out, const PairConsts<typename Lanes<T>::V> K,
               const GridConsts<T> G, int zchunk, int zbase, const __grid_constant__ CUtensorMap tm_phi,
               const __grid_constant__ CUtensorMap tm_c, const __grid_constant__ CUtensorMap tm_d,
