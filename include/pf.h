@@ -289,10 +289,12 @@ int pf_energy(pf_handle* h, double* F);
  * after each step and copied back once at the end, so the host does not wait
  * on every step (the planar-front run of Sec. "Numerical technique", which
  * checks the energy decrease of Eq. model1.1 step by step).  Without a moving
- * temperature or window the steps are replayed as captured 64-step CUDA
- * graphs on an internal stream ordered after and before the handle's.
- * Synchronises the stream once; PF_ENONFINITE if any record is not finite
- * (the steps are taken). */
+ * temperature or window, FP64 lines of up to about 16 cells per SM sum the
+ * energies in the step kernels, several steps per launch (their partial sums
+ * are kept in the handle: up to 5 MB, allocated on first use), and other grids
+ * replay captured 64-step CUDA graphs on an internal stream ordered after and
+ * before the handle's.  Synchronises the stream once; PF_ENONFINITE if any
+ * record is not finite (the steps are taken). */
 int pf_step_energies(pf_handle* h, int64_t n, double* F);
 
 /* Total solute S_h = dV sum_i [p_i c_s,i + (1-p_i) c_l,i] (Eq. model1), FP64.
@@ -411,14 +413,16 @@ int pf_run_batch(const pf_batch_desc* desc, pf_batch_result* res, void* stream);
  * the maximum the derivative of the maximising cell is taken (a subgradient
  * where two cells tie).  Two ways to the same numbers:
  *   PF_ADJ_TANGENT  tangent-linear: the state is carried as value + derivative
- *                   along one parameter, one CTA per instance and parameter,
- *                   all concurrent;
+ *                   along one parameter, one CTA per instance and parameter
+ *                   (a cluster of CTAs where that leaves SMs idle), all
+ *                   concurrent;
  *   PF_ADJ_REVERSE  reverse sweep: the forward run stores its state every
  *                   checkpoint_every steps (0: ceil(sqrt(nsteps)), at most 1024);
  *                   each segment is then re-run recording every step and swept
  *                   backwards with the adjoint of the fused step, from
- *                   d k_i / d c at the maximum, one CTA per instance.  The cost
- *                   does not grow with the number of parameters.
+ *                   d k_i / d c at the maximum, one CTA or cluster per instance.
+ *                   The cost does not grow with the number of parameters.  FP32
+ *                   states are stored with the low words of phi, c and d.
  * With k_target given, the loss is
  *   L = sum_i (k_i - k_target_i)^2,  dL/dtheta = sum_i 2 (k_i - k_target_i) dk_i/dtheta.
  * batch.params.precision selects FP32 or FP64 arithmetic for value and

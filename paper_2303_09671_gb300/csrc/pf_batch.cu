@@ -1604,7 +1604,7 @@ constexpr int rev_warps() {
 // Bound by the latency of a step's chain of dependent operations and by the
 // shuffles.  It replaces one CTA of 512 threads per instance with 13 arrays of the
 // line in shared memory and FP64 sums in every thread: 16 fronts of 2048 cells
-// take 4 us per step instead of 21.
+// take 4.1 us per step instead of 9.5.
 //
 // One instance per cluster, as batch_kernel, with two cells per lane: one step
 // backwards moves information by two cells, so the first and the last lane of a

@@ -52,7 +52,7 @@ static int diag_blocks(long long items) {
     return (int)(b < 1 ? 1 : (b > cap ? cap : b));
 }
 
-// The FP64 pipe of a GB300 runs at 1/77 of the FP32 rate, so the sums over FP32
+// The FP64 pipe of a GB300 runs at about 1/70 of the FP32 rate, so the sums over FP32
 // states are formed in three FP32 words (pf_words.cuh) for a few cells at a time
 // and added in FP64.
 

@@ -1,6 +1,6 @@
 // pf_fp64.cuh -- FP64 logarithm and reciprocal for the step kernels, in fewer
 // instructions of the FP64 pipe than log() and the IEEE division: a GB300's FP64
-// pipe takes about 19 cycles per warp instruction and SM and bounds every FP64
+// pipe takes about 18 cycles per warp instruction and SM and bounds every FP64
 // step.  The logarithm takes 14 of them, the reciprocal 4.
 #pragma once
 #include <cuda_runtime.h>

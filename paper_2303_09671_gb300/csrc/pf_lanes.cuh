@@ -87,10 +87,10 @@ struct alignas(2 * sizeof(V)) Q2 {
 template <typename V>
 struct PairConsts {
     V h2, h3, h4, h5, dh1, dh2, dh3, dh4, a_int;
-    V Ms_c, Ms_0, Ml_c, Ml_0, b, A, one_m_A, one_m_ke, log_ke;
+    V Ms_c, Ms_0, Ml_c, Ml_0, b, log_ke;
     V Ms_c_half, Ml_c_half, quarter_one_m_A;   // for face sums in place of face means
     V minus_b, minus_A, one_m_A_dx2, H_dx2, dp_dx2;   // factors folded for cell_rate (dp_dx2 = 30 dx^2)
-    V sigma, H, dx2, inv_Mphi, K_anti, delta2_dx2, delta2_4dx2, dt_dx2;
+    V sigma, dx2, inv_Mphi, K_anti, delta2_dx2, delta2_4dx2, dt_dx2;
 };
 
 // Grid, boundaries, frozen temperature and the Dirichlet ghost state.
@@ -271,13 +271,13 @@ inline PairConsts<typename Lanes<T>::V> make_pair_consts(const HostProblem& P, c
     K.dh1 = S(C.dh1); K.dh2 = S(C.dh2); K.dh3 = S(C.dh3); K.dh4 = S(C.dh4);
     K.a_int = S(P.a);
     K.Ms_c = S(C.Ms_c); K.Ms_0 = S(C.Ms_0); K.Ml_c = S(C.Ml_c); K.Ml_0 = S(C.Ml_0);
-    K.b = S(P.b); K.A = S(P.A); K.one_m_A = S(1.0 - P.A);
+    K.b = S(P.b);
     K.Ms_c_half = S(0.5 * C.Ms_c); K.Ml_c_half = S(0.5 * C.Ml_c); K.quarter_one_m_A = S(0.25 * (1.0 - P.A));
     K.minus_b = S(-P.b); K.minus_A = S(-P.A); K.one_m_A_dx2 = S((1.0 - P.A) * P.dx * P.dx);
     K.H_dx2 = S(P.H * P.dx * P.dx); K.dp_dx2 = S(30.0 * P.dx * P.dx);
-    K.one_m_ke = S(1.0 - P.k_e); K.log_ke = S(std::log(P.k_e));
+    K.log_ke = S(std::log(P.k_e));
     const double dx2 = P.dx * P.dx;
-    K.sigma = S(P.sigma); K.H = S(P.H); K.dx2 = S(dx2); K.inv_Mphi = S(1.0 / P.M_phi);
+    K.sigma = S(P.sigma); K.dx2 = S(dx2); K.inv_Mphi = S(1.0 / P.M_phi);
     K.K_anti = S((1.0 - P.A) * (1.0 - P.A) * P.b * 4.0 * dx2);
     K.delta2_dx2 = S(P.delta * P.delta * dx2);
     K.delta2_4dx2 = S(4.0 * P.delta * P.delta * dx2);

@@ -8,7 +8,7 @@
 // nothing within a launch; the window's shifts are changes of index, applied when
 // the strip is written.  The halo is computed twice: 32 of 64 cells hold results
 // where the line leaves SMs idle, 112 of 128 where it does not.  FP64 is bound by
-// the FP64 pipe of an SM, which issues one warp instruction in about 19 cycles:
+// the FP64 pipe of an SM, which issues one warp instruction in about 18 cycles:
 // a short line is spread with one cell per lane, 16 of 32 cells holding results.
 // Measured: 1.45 us per FP32 step (1000 cells), 6.4 us per FP64 step with its energy.
 //
