@@ -55,6 +55,24 @@ template <typename T>
 cudaError_t step3d_chunks(const HostProblem& P, int requested, int* zchunk, int* nchunks);
 size_t step_smem_bytes(int precision, int dim);
 
+// Rows of a warp in the kernel of large FP32 2D grids (pf_march2d.cu), such that all
+// warps are resident at once; 0: the grid stays with the tile kernel.  A warp takes
+// 60 columns whatever the grid has of them and evaluates four rows besides its own,
+// so its time goes with rows + 4; the tile kernel's goes with the number of its 32 x
+// 16 tiles.  30 grids of 330,000 to 4.2 million cells on 152 SMs, 8 to 50,000 wide,
+// put the line at 110 tiles per row: 1024^2 (2048 tiles, 15 rows) 23.8 and 20.6 us
+// per step with tiles and marching, 8192 x 64 (1024, 9) 14.0 and 12.8, 182 x 4000
+// (1500, 13) 19.0 and 18.4; on the other side 512 x 1024 (1024, 10) 13.9 and 14.2,
+// 600^2 (722, 8) 10.0 and 11.6, 64 x 8192 (1024, 13) 14.1 and 18.2.
+constexpr int MARCH_X = 60;         // columns a warp updates
+constexpr int MARCH_PER_SM = 12;    // resident warps
+inline long long march2d_rows(long long nx, long long ny, int sms) {
+    const long long strips = (nx + MARCH_X - 1) / MARCH_X, room = (long long)MARCH_PER_SM * sms;
+    const long long rows = (ny * strips + room - 1) / room;
+    const long long tiles = ((nx + 31) / 32) * ((ny + 15) / 16);
+    return rows >= 4 && 18 * tiles >= 13 * (rows + 4) * sms ? rows : 0;   // 13/18 of 152: 110
+}
+
 // Several steps of a 1D line per launch (pf_step1d.cu), for lines with a no-flux
 // low end and a no-flux or Dirichlet high end, and for periodic lines in a uniform
 // temperature.  line_steps advances the run's buffers and clock, window shifts

@@ -27,8 +27,6 @@ namespace pf {
 namespace {
 
 constexpr int MARCH_WARPS = 4;                 // per block
-constexpr int MARCH_PER_SM = 12;               // resident warps
-constexpr int MARCH_X = 60;                    // columns a warp updates
 
 __device__ __forceinline__ float2 from_right(float2 v) {   // v at x + 1
     return make_float2(v.y, __shfl_down_sync(0xffffffffu, v.x, 1));
@@ -206,11 +204,6 @@ march2d_kernel(const float* phi_in, const float* c_in, const float* d_in, const 
     }
 }
 
-// Rows per warp such that all warps are resident at once.  Each warp evaluates four
-// rows besides its own, so grids with fewer than four rows per warp (below about
-// 330,000 cells on 152 SMs) stay with the tile kernel: per step, tiles and this
-// kernel, 512^2 (3 rows) 9.1 and 10.2 us, 4000 x 100 (4 rows) 11.9 and 11.3, 100 x
-// 4000 (5 rows) 14.2 and 13.0.
 cudaError_t launch_march2d(const StepLaunch& a, const Consts<float>& C, const Clock<float>& Kc, bool* taken) {
     *taken = false;
     const HostProblem& P = *a.prob;
@@ -230,9 +223,8 @@ cudaError_t launch_march2d(const StepLaunch& a, const Consts<float>& C, const Cl
         sms = setup.sms[dev];
     }
     const long long strips = (C.n[0] + MARCH_X - 1) / MARCH_X;
-    const long long room = (long long)MARCH_PER_SM * sms;
-    const long long rows = (C.n[1] * strips + room - 1) / room;
-    if (rows < 4) return cudaSuccess;
+    const long long rows = march2d_rows(C.n[0], C.n[1], sms);
+    if (rows == 0) return cudaSuccess;
     const long long warps = strips * ((C.n[1] + rows - 1) / rows);
     *taken = true;
     const PairConsts<float2> K = make_pair_consts<float>(P, C);
