@@ -417,7 +417,8 @@ int pf_run_batch(const pf_batch_desc* desc, pf_batch_result* res, void* stream);
  *                   (a cluster of CTAs where that leaves SMs idle), all
  *                   concurrent;
  *   PF_ADJ_REVERSE  reverse sweep: the forward run stores its state every
- *                   checkpoint_every steps (0: ceil(sqrt(nsteps)), at most 1024);
+ *                   checkpoint_every steps (0: ceil(sqrt(nsteps)), at most 1024;
+ *                   farther apart where so many states do not fit the device);
  *                   each segment is then re-run recording every step and swept
  *                   backwards with the adjoint of the fused step, from
  *                   d k_i / d c at the maximum, one CTA or cluster per instance.

@@ -1913,32 +1913,42 @@ static int run_adjoint_reverse_T(const pf_adjoint_desc& A, pf_adjoint_result* R,
     if (!batch_time_steps(D, B.dt, err)) return PF_EINVAL;
     int64_t nmax = 0;
     for (int i = 0; i < N; ++i) nmax = std::max(nmax, (int64_t)D.n[i]);
-    const int64_t seg = std::min<int64_t>(
-        {A.checkpoint_every > 0 ? (int64_t)A.checkpoint_every
-                                : (int64_t)std::ceil(std::sqrt((double)A.nsteps)),
-         (int64_t)RMAX_SEG, A.nsteps});
-    const int64_t nseg = (A.nsteps + seg - 1) / seg;
+    const int64_t most = std::min<int64_t>(RMAX_SEG, A.nsteps);
+    int64_t seg = std::min<int64_t>(
+        A.checkpoint_every > 0 ? (int64_t)A.checkpoint_every : (int64_t)std::ceil(std::sqrt((double)A.nsteps)), most);
+    int64_t nseg = 0;
     const size_t fb = (size_t)B.total * sizeof(V);
-    // States before every segment (each segment's run reads its own and writes the
-    // next), the final state, and one for the re-runs' results, which nothing
-    // reads: slots 0 .. nseg + 1 of every array.
-    const size_t slots = (size_t)nseg + 2;
     B.deriv = true;
     V *scs = nullptr, *scl = nullptr, *rec = nullptr, *lphi = nullptr, *lc = nullptr, *ld = nullptr;
     double *grad = nullptr, *cmax = nullptr;
     int* imax = nullptr;
-    for (V** p : {&B.phi, &B.c, &B.d}) B.mem.add(p, fb * slots);
-    if (sizeof(V) == 4) B.mem.add(&B.low, 3 * fb * slots);
-    B.mem.add(&B.st, N * slots * sizeof(BatchState));
-    B.mem.add(&B.dv, N * sizeof(double));
-    B.mem.add(&B.ddt, N * sizeof(double));
-    B.mem.add(&B.ids, N * sizeof(int));
-    for (V** p : {&scs, &scl, &lphi, &lc, &ld}) B.mem.add(p, fb);
-    B.mem.add(&rec, fb * 6 * seg * 2);
-    B.mem.add(&grad, 3 * N * sizeof(double));
-    B.mem.add(&cmax, N * sizeof(double));
-    B.mem.add(&imax, N * sizeof(int));
-    cudaError_t e = B.mem.allocate();
+    cudaError_t e = cudaSuccess;
+    for (;; seg = std::min(2 * seg, most)) {
+        nseg = (A.nsteps + seg - 1) / seg;
+        // States before every segment (each segment's run reads its own and writes
+        // the next), the final state, and one for the re-runs' results, which nothing
+        // reads: slots 0 .. nseg + 1 of every array.
+        const size_t slots = (size_t)nseg + 2;
+        B.mem.want.clear();
+        for (V** p : {&B.phi, &B.c, &B.d}) B.mem.add(p, fb * slots);
+        if (sizeof(V) == 4) B.mem.add(&B.low, 3 * fb * slots);
+        B.mem.add(&B.st, N * slots * sizeof(BatchState));
+        B.mem.add(&B.dv, N * sizeof(double));
+        B.mem.add(&B.ddt, N * sizeof(double));
+        B.mem.add(&B.ids, N * sizeof(int));
+        for (V** p : {&scs, &scl, &lphi, &lc, &ld}) B.mem.add(p, fb);
+        B.mem.add(&rec, fb * 6 * seg * 2);
+        B.mem.add(&grad, 3 * N * sizeof(double));
+        B.mem.add(&cmax, N * sizeof(double));
+        B.mem.add(&imax, N * sizeof(int));
+        e = B.mem.allocate();
+        // Checkpoints that do not fit are taken twice as far apart (the results' sums
+        // then group otherwise, no more), while that saves more than the records (12
+        // words a cell and step of a segment) grow: with their low words FP32 checkpoints take 6 words, and dense
+        // ones that fitted with 3 still have to run.
+        if (e == cudaSuccess || seg == most || 4 * seg >= nseg) break;
+        cudaGetLastError();
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         err = std::string("device allocation failed: ") + cudaGetErrorString(e);
